@@ -40,9 +40,10 @@ namespace vbq {
 namespace {
 
 constexpr int kTa = 128;          // output tile rows i (MMA M, tensor-memory lanes): A = X_i
-constexpr int kTb = 112;          // output tile columns j of S and of H: B = [X_j; Y_j], N = 224
+constexpr int kTb = 112;          // widest output tile, columns j of S and of H: B = [X_j; Y_j], N = 224
 constexpr int kColBlock = 256;    // threads of a column-sum block (and samples per sub-tile)
-constexpr int kCenTiles = 8;      // 64-sample tiles per centring block: 512 samples
+constexpr int kCenTiles = 8;      // most 64-sample tiles per centring block: 512 samples
+constexpr int kSeg = 64;          // rows the workspace's second partial array holds beyond one per 512 samples
 constexpr float kScaleTop = 16384.0f;  // scaled values stay below 2^14 (half precision max 65504)
 
 __host__ __device__ inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
@@ -72,6 +73,34 @@ __device__ __forceinline__ void load4(const Tin* __restrict__ row, int c, int P,
 #pragma unroll
     for (int u = 0; u < 4; ++u) v[u] = c + u < P ? row[c + u] : (Tin)0;
   }
+}
+
+// Largest |x| seen, kept as the value's own bits: for finite doubles the order of the absolute
+// values is the order of their bit patterns, so the FP64 pipe (64 cycles per warp instruction, a
+// conversion to float like any other) takes no part; rounding to float commutes with the maximum.
+template <class Tin> struct AbsMax {
+  unsigned long long b = 0;
+  __device__ __forceinline__ void take(Tin x) {
+    const unsigned long long v = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+    b = v > b ? v : b;
+  }
+  __device__ __forceinline__ float value() const { return (float)__longlong_as_double((long long)b); }
+};
+template <> struct AbsMax<float> {
+  float m = 0.0f;
+  __device__ __forceinline__ void take(float x) { m = fmaxf(m, fabsf(x)); }
+  __device__ __forceinline__ float value() const { return m; }
+};
+
+// double -> float, round to nearest even, on the bit pattern (about ten integer instructions in
+// place of one on the FP64 pipe); values outside the normal float range take the conversion.
+__device__ __forceinline__ float to_float(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned ex = (unsigned)(b >> 52) & 0x7ffu;
+  if (ex < 897u || ex > 1150u) return (float)x;
+  unsigned long long m = (b & 0x7fffffffffffffffull) - (896ull << 52);
+  m += 0x0fffffffull + ((m >> 29) & 1ull);
+  return __uint_as_float((unsigned)(m >> 29) | ((unsigned)(b >> 32) & 0x80000000u));
 }
 
 // (1) Block partials: row b = [sum w, sum w E, sum w O (P), sum w dE (P)] over samples
@@ -137,7 +166,7 @@ __global__ void __launch_bounds__(kColBlock) lin_colsum_kernel(int P, long long 
     }
     const int c = blockIdx.x * 64 + 4 * q;
     Tin so[4] = {0, 0, 0, 0}, sd[4] = {0, 0, 0, 0};
-    float mo[4] = {0.0f, 0.0f, 0.0f, 0.0f}, md[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    AbsMax<Tin> mo[4], md[4];
     auto take = [&](int sl) {
       Tin o[4], d[4];
       load4<Tin, VEC>(O + (s0 + sl) * P, c, P, o);
@@ -147,8 +176,8 @@ __global__ void __launch_bounds__(kColBlock) lin_colsum_kernel(int P, long long 
       for (int u = 0; u < 4; ++u) {
         so[u] += ws * o[u];
         sd[u] += ws * d[u];
-        mo[u] = fmaxf(mo[u], fabsf((float)o[u]));
-        md[u] = fmaxf(md[u], fabsf((float)d[u]));
+        mo[u].take(o[u]);
+        md[u].take(d[u]);
       }
     };
     if (c < P) {
@@ -164,8 +193,8 @@ __global__ void __launch_bounds__(kColBlock) lin_colsum_kernel(int P, long long 
     for (int u = 0; u < 4; ++u) {
       red_o[r][4 * q + u] = so[u];
       red_d[r][4 * q + u] = sd[u];
-      red_mo[r][4 * q + u] = mo[u];
-      red_md[r][4 * q + u] = md[u];
+      red_mo[r][4 * q + u] = mo[u].value();
+      red_md[r][4 * q + u] = md[u].value();
     }
     __syncthreads();
     if (tid < 64) {
@@ -188,73 +217,99 @@ __global__ void __launch_bounds__(kColBlock) lin_colsum_kernel(int P, long long 
   }
 }
 
-// Block partials added in a fixed order, in two levels so that the whole machine takes part:
-// (a) grid (columns / 32, kSeg): block (x, g) sums for its 32 columns the partial rows of
-//     segment g (rows [g nb / kSeg, (g + 1) nb / kSeg)), warp w the rows w, w + 8, ... of the
-//     segment, the 8 warp sums added in warp order: seg[g][q];
-// (b) acc[q] = sum over g of seg[g][q] in segment order.
-constexpr int kSeg = 64;
-__global__ void __launch_bounds__(256) lin_seg_reduce(int L, int nb, const double* __restrict__ part,
-                                                      double* __restrict__ seg) {
-  __shared__ double red[8][32];
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  const int q = blockIdx.x * 32 + lane, g = blockIdx.y;
-  const int b0 = (int)((long long)g * nb / kSeg), b1 = (int)((long long)(g + 1) * nb / kSeg);
+// Sum over rows of part[row][q] for the 8 columns q0 + (tid & 7) < L, by a block of NT threads: thread
+// (r, c) = (tid / 8, tid % 8) adds rows r, r + NT / 8, ... (64 contiguous bytes per row of threads),
+// then the row sums are added in a fixed order.  The sum is returned by the threads tid < 8.
+// 'red' holds NT doubles.
+template <int NT>
+__device__ __forceinline__ double column_sum(int L, int nrow, const double* __restrict__ part, int q0, double* red) {
+  const int c = threadIdx.x & 7, r = threadIdx.x >> 3;
   double s = 0.0;
-  if (q < L)
-#pragma unroll 4
-    for (int b = b0 + wp; b < b1; b += 8) s += part[(size_t)b * L + q];
-  red[wp][lane] = s;
+  if (q0 + c < L)
+#pragma unroll 8
+    for (int b = r; b < nrow; b += NT / 8) s += part[(size_t)b * L + q0 + c];
+  __syncthreads();  // the previous use of red is over
+  red[threadIdx.x] = s;
   __syncthreads();
-  if (wp == 0 && q < L) {
-    double t = red[0][lane];
+  if (threadIdx.x < 64) {
+    double t = red[threadIdx.x];
 #pragma unroll
-    for (int k = 1; k < 8; ++k) t += red[k][lane];
-    seg[(size_t)g * L + q] = t;
+    for (int k = 64; k < NT; k += 64) t += red[threadIdx.x + k];
+    red[threadIdx.x] = t;
   }
-}
-__global__ void lin_final_reduce(int L, const double* __restrict__ seg, double* __restrict__ acc) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= L) return;
-  double s = 0.0;
-  for (int g = 0; g < kSeg; ++g) s += seg[(size_t)g * L + q];
-  acc[q] = s;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < 8)
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t += red[threadIdx.x + 8 * k];
+  return t;
 }
 
-// Per-sample float copies for the centring pass: sqrt(w_s) and E_s.
-__global__ void lin_sample_kernel(long long M, const double* __restrict__ E, const double* __restrict__ w,
-                                  float* __restrict__ rw, float* __restrict__ Ef) {
-  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= M) return;
-  rw[s] = w ? sqrtf((float)w[s]) : 1.0f;
-  Ef[s] = (float)E[s];
-}
-
-// (2a) Power-of-two scales: scl[c] for X (bound sqrt(max w)(max|O_c| + |<O_c>|)) and scl[Pr + c]
-// for Y (bound sqrt(max w)(max|E| (max|O_c| + |<O_c>|) + max|dE_c|)), 1 for padding rows.
-__global__ void lin_scale_kernel(int P, int Pr, const double* __restrict__ acc, const unsigned* __restrict__ mx,
-                                 float* __restrict__ scl) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= Pr) return;
-  float sx = 1.0f, sy = 1.0f;
-  if (c < P) {
-    const double mu = acc[2 + c] / acc[0];
-    const double rw = sqrt((double)__uint_as_float(mx[0]));
-    const double ox = (double)__uint_as_float(mx[2 + c]) + fabs(mu);
-    const double bx = rw * ox;
-    const double by = rw * ((double)__uint_as_float(mx[1]) * ox + (double)__uint_as_float(mx[2 + P + c]));
-    int e;
-    if (bx > 0.0) {
-      frexp(bx, &e);  // bx <= 2^e
-      sx = ldexpf(kScaleTop, -max(e, -100));
+// (2a) Column totals and power-of-two scales: block b sums columns 8 b .. 8 b + 7 of the block
+// partials into acc; for the columns of O it also forms scl[c] for X (bound
+// sqrt(max w)(max|O_c| + |<O_c>|)) and scl[Pr + c] for Y (bound
+// sqrt(max w)(max|E| (max|O_c| + |<O_c>|) + max|dE_c|)); the padding rows' scales are 1.  Every
+// block sums w for itself (one column more).  The blocks after the first nq write the per-sample
+// float copies sqrt(w_s) and E_s that the centring pass reads.  One launch in place of a two-level sum, a scale and
+// a per-sample launch: on a small sample these took 23 of 238 us, each a few microseconds of
+// latency with most SMs idle (15001 x 216 doubles).
+constexpr int kStatThreads = 512;
+__global__ void __launch_bounds__(kStatThreads) lin_stats_kernel(int P, int Pr, int nb, const double* __restrict__ part,
+                                                                 const unsigned* __restrict__ mx,
+                                                                 double* __restrict__ acc, float* __restrict__ scl,
+                                                                 int nq, long long M, const double* __restrict__ E,
+                                                                 const double* __restrict__ w, float* __restrict__ rw,
+                                                                 float* __restrict__ Ef) {
+  if ((int)blockIdx.x >= nq) {
+    for (long long s = (long long)(blockIdx.x - nq) * kStatThreads + threadIdx.x; s < M;
+         s += (long long)(gridDim.x - nq) * kStatThreads) {
+      rw[s] = w ? sqrtf((float)w[s]) : 1.0f;
+      Ef[s] = (float)E[s];
     }
-    if (by > 0.0) {
-      frexp(by, &e);
-      sy = ldexpf(kScaleTop, -max(e, -100));
+    return;
+  }
+  __shared__ double red[kStatThreads];
+  __shared__ double sw;
+  const int L = 2 * P + 2, q0 = blockIdx.x * 8;
+  {
+    double s = 0.0;
+#pragma unroll 4
+    for (int b = threadIdx.x; b < nb; b += kStatThreads) s += part[(size_t)b * L];
+    __syncthreads();
+    red[threadIdx.x] = s;
+    for (int k = kStatThreads / 2; k > 0; k >>= 1) {
+      __syncthreads();
+      if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) sw = red[0];
+  }
+  const double t = column_sum<kStatThreads>(L, nb, part, q0, red);
+  const int q = q0 + threadIdx.x;
+  if (threadIdx.x < 8 && q < L) {
+    acc[q] = q == 0 ? sw : t;  // one value of sum w for everyone
+    const int c = q - 2;
+    if (c >= 0 && c < P) {
+      float sx = 1.0f, sy = 1.0f;
+      const double rw = sqrt((double)__uint_as_float(mx[0]));
+      const double ox = (double)__uint_as_float(mx[2 + c]) + fabs(t / sw);
+      const double bx = rw * ox;
+      const double by = rw * ((double)__uint_as_float(mx[1]) * ox + (double)__uint_as_float(mx[2 + P + c]));
+      int e;
+      if (bx > 0.0) {
+        frexp(bx, &e);  // bx <= 2^e
+        sx = ldexpf(kScaleTop, -max(e, -100));
+      }
+      if (by > 0.0) {
+        frexp(by, &e);
+        sy = ldexpf(kScaleTop, -max(e, -100));
+      }
+      scl[c] = sx;
+      scl[Pr + c] = sy;
     }
   }
-  scl[c] = sx;
-  scl[Pr + c] = sy;
+  if (blockIdx.x == 0)
+    for (int c = P + threadIdx.x; c < Pr; c += kStatThreads) scl[c] = scl[Pr + c] = 1.0f;
 }
 
 // x and y split into high and low halves (v = hi + lo, hi = half(v), lo = half(v - hi)), the
@@ -275,14 +330,20 @@ __device__ __forceinline__ void split_half2(float x, float y, __half& xh, __half
 // M <= s < Mp.  A tile of the tensor-core pass (rows r0 .. r0 + 127 of one group) is then one
 // contiguous 16 KB block.  A block of this kernel transposes 64 samples x 64 parameters through
 // shared memory: reads along parameters and writes along samples are both coalesced.
-template <class Tin, bool VEC>
-__global__ void __launch_bounds__(256, 4) lin_center_kernel(int P, long long M, long long Mp, const Tin* __restrict__ O,
-                                                         const Tin* __restrict__ dEL, const double* __restrict__ E,
-                                                         const double* __restrict__ w, const float* __restrict__ rwf,
-                                                         const float* __restrict__ Ef, const double* __restrict__ acc,
-                                                         const float* __restrict__ scl, int Pr,
-                                                         __half* __restrict__ XI, __half* __restrict__ YI,
-                                                         double* __restrict__ part2, long long nb) {
+// Blocks take ntile tiles (a sample block is 64 ntile samples, one row of part2).  Issuing the next
+// tile's loads before the stores was tried: at 85 registers and 3 blocks per SM it ran 1.55 in place
+// of 1.51 ms (2^20 x 400), so the blocks stay 4 to an SM and load at the top.  With double input the
+// FP64 pipe bounds the pass: three instructions per value (difference, y, w Ot E) and none for the
+// conversions to float (99 -> 59 us at 15001 x 216, with more and shorter blocks).
+template <class Tin> struct CenBlocks { static constexpr int n = 4; };
+template <> struct CenBlocks<double> { static constexpr int n = 2; };
+template <class Tin, bool VEC, int ntile>
+__global__ void __launch_bounds__(256, CenBlocks<Tin>::n)
+    lin_center_kernel(int P, long long M, long long Mp, const Tin* __restrict__ O, const Tin* __restrict__ dEL,
+                      const double* __restrict__ E, const double* __restrict__ w, const float* __restrict__ rwf,
+                      const float* __restrict__ Ef, const double* __restrict__ acc, const float* __restrict__ scl,
+                      int Pr, __half* __restrict__ XI, __half* __restrict__ YI, double* __restrict__ part2,
+                      long long nb) {
   // [array][parameter][sample]: rows of 72 halves (144 bytes) keep the 16-byte chunks aligned
   __shared__ __align__(16) __half t[4][64][72];
   __shared__ double red[16][64];
@@ -303,8 +364,8 @@ __global__ void __launch_bounds__(256, 4) lin_center_kernel(int P, long long M, 
       sx[u] = scl[c + u];
       sy[u] = scl[Pr + c + u];
     }
-    for (int tt = 0; tt < kCenTiles; ++tt) {
-      const long long s0 = (sb * kCenTiles + tt) * 64;
+    for (int tt = 0; tt < ntile; ++tt) {
+      const long long s0 = (sb * ntile + tt) * 64;
       if (s0 >= M) break;
       __syncthreads();  // the previous tile's stores have read t
       // the tile's 8 loads of 4 values first (memory-level parallelism), then the arithmetic
@@ -333,11 +394,17 @@ __global__ void __launch_bounds__(256, 4) lin_center_kernel(int P, long long M, 
           float xv = 0.0f, yv = 0.0f;
           if (in && c + u < P) {
             const Tin x = ov[k][u] - mo[u];
-            const Tin ex = e * x;
-            const Tin y = ex + dv[k][u];
-            xv = (float)x * rw * sx[u];
-            yv = (float)y * rw * sy[u];
-            part[u] += ws * ex;
+            if constexpr (std::is_same<Tin, double>::value) {
+              xv = to_float(x) * rw * sx[u];
+              yv = to_float(fma(e, x, dv[k][u])) * rw * sy[u];
+              part[u] = fma(ws * e, x, part[u]);
+            } else {
+              const Tin ex = e * x;
+              const Tin y = ex + dv[k][u];
+              xv = (float)x * rw * sx[u];
+              yv = (float)y * rw * sy[u];
+              part[u] += ws * ex;
+            }
           }
           split_half2(xv, yv, t[0][4 * q + u][sl], t[1][4 * q + u][sl], t[2][4 * q + u][sl], t[3][4 * q + u][sl]);
         }
@@ -397,42 +464,51 @@ constexpr int kTcThreads = 32 * kTcWarps;
 constexpr int kCopyWarp = 8, kMmaWarp = 9;
 constexpr int kK = 32;                                     // samples per stage
 constexpr int kRow = 2 * kK * 2;                           // 128-byte rows: high and low halves
-constexpr int kStages = 5;
-constexpr int kN = 2 * kTb;                                // MMA N: the j rows of X and of Y
 constexpr int kABytes = kTa * kRow;                        // 16 KB
-constexpr int kHBytes = kTb * kRow;                        // 14 KB: the X_j (or Y_j) half of B
-constexpr int kBBytes = 2 * kHBytes;                       // 28 KB
-constexpr int kStageBytes = kABytes + kBBytes;             // A, B
-constexpr int kNumBars = 2 * kStages + 5;                  // full, empty, set full x2, set empty x2, done
-constexpr int kTcSmem = kStages * kStageBytes + 1024 + 8 * kNumBars + 64;
-constexpr int kSetCols = 256;                              // tensor-memory columns per accumulator set
 constexpr uint64_t kWaitNs = 1000000000ull;
-static_assert(kHBytes % 1024 == 0 && kABytes % 1024 == 0, "128-byte swizzled tiles stay 1024-byte aligned");
-static_assert(kN % 16 == 0 && kN <= 256 && kN <= kSetCols, "MMA shape M = 128 needs N a multiple of 16, <= 256");
-static_assert(kTcSmem <= 232448, "shared memory of one CTA");
+// Output tiles of TB columns.  112 (MMA N = 224) for samples that fill the chip; 64 and 32 for small
+// ones, whose chunks (fixed by the sample count: the FP32 sums of a chunk are part of the result)
+// times 112-column tiles leave most SMs idle (15001 x 216: 32 CTAs 61 us, 112 CTAs of 32 columns 38 us).
+// An element's products and sums do not depend on the tile it is computed in.
+template <int TB> struct TcShape {
+  static constexpr int kN = 2 * TB;                          // MMA N: the j rows of X and of Y
+  static constexpr int kStages = TB == 112 ? 5 : 6;
+  static constexpr int kHBytes = TB * kRow;                  // the X_j (or Y_j) half of B
+  static constexpr int kStageBytes = kABytes + 2 * kHBytes;  // A, B (44 KB at 112)
+  static constexpr int kNumBars = 2 * kStages + 5;           // full, empty, set full x2, set empty x2, done
+  static constexpr int kSmem = kStages * kStageBytes + 1024 + 8 * kNumBars + 64;
+  static constexpr int kSetCols = kN <= 64 ? 64 : (kN <= 128 ? 128 : 256);  // tensor-memory columns per set
+  static_assert(kHBytes % 1024 == 0 && kABytes % 1024 == 0, "128-byte swizzled tiles stay 1024-byte aligned");
+  static_assert(TB % 16 == 0 && kN <= 256, "MMA shape M = 128 needs N a multiple of 16, <= 256");
+  static_assert(kSmem <= 232448, "shared memory of one CTA");
+};
 
-// adds this warp's 112 accumulator columns (lanes 32 (warp % 4) + lane; warps 0-3 the S half
+// adds this warp's TB accumulator columns (lanes 32 (warp % 4) + lane; warps 0-3 the S half
 // of the set, warps 4-7 the H half) starting at tensor-memory address 'base'; the loads go out
 // two at a time behind one wait
-__device__ __forceinline__ void drain(uint32_t base, float acc[kTb]) {
+template <int TB> __device__ __forceinline__ void drain(uint32_t base, float acc[TB]) {
   uint32_t v[2][16];
 #pragma unroll
-  for (int g = 0; g < kTb / 16; g += 2) {
+  for (int g = 0; g < TB / 16; g += 2) {
     tmem_ld16_async(base + 16 * g, v[0]);
-    if (g + 1 < kTb / 16) tmem_ld16_async(base + 16 * (g + 1), v[1]);
+    if (g + 1 < TB / 16) tmem_ld16_async(base + 16 * (g + 1), v[1]);
     tmem_wait_ld();
 #pragma unroll
     for (int q = 0; q < 16; ++q) acc[16 * g + q] += __uint_as_float(v[0][q]);
-    if (g + 1 < kTb / 16)
+    if (g + 1 < TB / 16)
 #pragma unroll
       for (int q = 0; q < 16; ++q) acc[16 * (g + 1) + q] += __uint_as_float(v[1][q]);
   }
 }
 
+template <int TB>
 __global__ void __launch_bounds__(kTcThreads, 1)
     lin_tc_kernel(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tBX,
                   const __grid_constant__ CUtensorMap tBY, int Pa, int Pb, long long M, long long chunk,
                   double* __restrict__ part, int* __restrict__ err) {
+  using Sh = TcShape<TB>;
+  constexpr int kStages = Sh::kStages, kStageBytes = Sh::kStageBytes, kHBytes = Sh::kHBytes, kN = Sh::kN,
+                kSetCols = Sh::kSetCols;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full = reinterpret_cast<uint64_t*>(sm + kStages * kStageBytes);  // [kStages] copies landed
@@ -443,9 +519,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(mdone + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int ntb = Pb / kTb;
-  const int ta = blockIdx.x / ntb, tb = blockIdx.x % ntb;
-  const int i0 = ta * kTa, j0 = tb * kTb;
+  const int nta = Pa / kTa;
+  const int ta = blockIdx.x % nta, tb = blockIdx.x / nta;
+  const int i0 = ta * kTa, j0 = tb * TB;
   const long long s0 = (long long)blockIdx.y * chunk, s1 = min(M, s0 + chunk);
   const int nsteps = s1 > s0 ? (int)((s1 - s0 + kK - 1) / kK) : 0;
   const int npairs = (nsteps + 1) / 2;
@@ -466,12 +542,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     *abort_flag = 0;
     fence_async_smem();
   }
-  if (warp == kMmaWarp) tmem_alloc(tmem_holder, 512);  // set b at columns 256 b: S (+0), H (+112)
+  if (warp == kMmaWarp) tmem_alloc(tmem_holder, 2 * kSetCols);  // set b at columns kSetCols b: S (+0), H (+TB)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_holder;
-  float acc[kTb];
+  float acc[TB];
 
   if (warp == kCopyWarp) {
     if (lane == 0) {
@@ -543,8 +619,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __syncwarp();
   } else {
 #pragma unroll
-    for (int c = 0; c < kTb; ++c) acc[c] = 0.0f;
-    const uint32_t base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (warp < 4 ? 0u : (uint32_t)kTb);
+    for (int c = 0; c < TB; ++c) acc[c] = 0.0f;
+    const uint32_t base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (warp < 4 ? 0u : (uint32_t)TB);
     for (int p = 0; p < npairs; ++p) {
       const int set = p & 1;
       int ok = 0;
@@ -555,7 +631,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         break;
       }
       tc_fence_after();
-      drain(base + kSetCols * set, acc);
+      drain<TB>(base + kSetCols * set, acc);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&sempty[set]);
@@ -567,26 +643,32 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int row = i0 + 32 * (warp & 3) + lane;
     double* out = part + ((size_t)blockIdx.y * 2 + (warp < 4 ? 0 : 1)) * Pa * Pb + (size_t)row * Pb + j0;
 #pragma unroll
-    for (int c = 0; c < kTb; ++c) out[c] = (double)acc[c];
+    for (int c = 0; c < TB; ++c)
+      if (j0 + c < Pb) out[c] = (double)acc[c];
   }
   if (threadIdx.x == 0 && !good) atomicExch(err, 1);
   tc_fence_after();
-  if (warp == kMmaWarp) tmem_dealloc(tmem, 512);
+  if (warp == kMmaWarp) tmem_dealloc(tmem, 2 * kSetCols);
 }
 
-// (4) thread (i, j): S[i][j] and H[i][j] from the chunk partials [chunk][2][Pa][Pb], unscaled;
-// gL, gR, E0 from the column sums.
-__global__ void lin_reduce_kernel(int P, int Pa, int Pb, int Pr, int nchunk, const double* __restrict__ part,
-                                  const double* __restrict__ acc, const double* __restrict__ sxe,
-                                  const float* __restrict__ scl, double* E0,
-                                  double* gL, double* gR, double* S, double* H, const int* __restrict__ err) {
+// (4) Blocks b < P * nj (nj = blocks per row): thread (i, j) forms S[i][j] and H[i][j] from the chunk
+// partials [chunk][2][Pa][Pb], unscaled; the blocks after them sum w Ot E over the centring blocks'
+// partials, 8 parameters each, for gL and gR.
+constexpr int kRedThreads = 256;
+__global__ void __launch_bounds__(kRedThreads)
+    lin_reduce_kernel(int P, int Pa, int Pb, int Pr, int nchunk, int nj, int nb2, const double* __restrict__ part,
+                      const double* __restrict__ acc, const double* __restrict__ part2, const float* __restrict__ scl,
+                      double* E0, double* gL, double* gR, double* S, double* H, const int* __restrict__ err) {
+  __shared__ double red[kRedThreads];
   // a timed-out tensor-core stage leaves NaN outputs
   const double isw = *err ? __longlong_as_double(0x7ff8000000000000ll) : 1.0 / acc[0];
-  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < (long long)P * P) {
-    const int i = (int)(q / P), j = (int)(q % P);
+  const int b = blockIdx.x;
+  if (b < P * nj) {
+    const int i = b / nj, j = (b - i * nj) * kRedThreads + threadIdx.x;
+    if (j >= P) return;
     const size_t o = (size_t)i * Pb + j, plane = (size_t)Pa * Pb;
     double s = 0.0, h = 0.0;
+#pragma unroll 4
     for (int c = 0; c < nchunk; ++c) {
       s += part[(size_t)c * 2 * plane + o];
       h += part[(size_t)c * 2 * plane + plane + o];
@@ -594,9 +676,13 @@ __global__ void lin_reduce_kernel(int P, int Pa, int Pb, int Pr, int nchunk, con
     const double sxi = scl[i], sxj = scl[j], syj = scl[Pr + j];
     S[(size_t)i * P + j] = s / (sxi * sxj) * isw;
     H[(size_t)i * P + j] = h / (sxi * syj) * isw;
+    return;
   }
-  if (q < P) {
-    const double oe = sxe[q] * isw;  // <Ot E>
+  const int q0 = (b - P * nj) * 8;
+  const double t = column_sum<kRedThreads>(Pr, nb2, part2, q0, red);
+  const int q = q0 + threadIdx.x;
+  if (threadIdx.x < 8 && q < P) {
+    const double oe = t * isw;  // <Ot E>
     gL[q] = 2.0 * oe;
     gR[q] = 2.0 * (oe + acc[2 + P + q] * isw);
   }
@@ -629,11 +715,13 @@ LinGrid lin_grid(int P, long long M, int nsm) {
 
 namespace {
 struct LinWs {
-  double *part1, *acc, *part2, *sxe, *seg, *part;
+  double *part1, *acc, *part2, *part;
   unsigned* mx;
   float *scl, *rw, *Ef;
   __half *XI, *YI;
-  int* err;
+  int* err;            // right after mx: both are cleared together
+  size_t zero_bytes;
+  size_t part2_rows;   // rows of [Pr] doubles that part2 has room for
   size_t bytes;
 };
 LinWs carve(void* ws, int P, long long M, int nchunk) {
@@ -649,21 +737,32 @@ LinWs carve(void* ws, int P, long long M, int nchunk) {
     return r;
   };
   LinWs w{};
-  w.part1 = reinterpret_cast<double*>(take(sizeof(double) * (size_t)nb1 * L1));
+  // the column-sum partials are read before the centring pass writes part2 over them and what follows
+  w.part1 = w.part2 = reinterpret_cast<double*>(take(sizeof(double) * (size_t)nb1 * L1));
+  take(sizeof(double) * ((size_t)nb2 + kSeg) * Pr);
+  w.part2_rows = off / (sizeof(double) * Pr);
   w.acc = reinterpret_cast<double*>(take(sizeof(double) * (size_t)L1));
-  w.part2 = reinterpret_cast<double*>(take(sizeof(double) * (size_t)nb2 * Pr));
-  w.sxe = reinterpret_cast<double*>(take(sizeof(double) * (size_t)Pr));
-  w.seg = reinterpret_cast<double*>(take(sizeof(double) * (size_t)kSeg * std::max(L1, Pr)));
-  w.mx = reinterpret_cast<unsigned*>(take(sizeof(unsigned) * (2 + 2 * (size_t)P)));
+  const size_t nmx = 2 + 2 * (size_t)P;
+  w.zero_bytes = sizeof(unsigned) * nmx + sizeof(int);
+  w.mx = reinterpret_cast<unsigned*>(take(w.zero_bytes));
+  w.err = reinterpret_cast<int*>(w.mx + nmx);
   w.scl = reinterpret_cast<float*>(take(sizeof(float) * 2 * (size_t)Pr));
   w.rw = reinterpret_cast<float*>(take(sizeof(float) * (size_t)M));
   w.Ef = reinterpret_cast<float*>(take(sizeof(float) * (size_t)M));
   w.XI = reinterpret_cast<__half*>(take(sizeof(__half) * (size_t)Pr * 2 * Mp));
   w.YI = reinterpret_cast<__half*>(take(sizeof(__half) * (size_t)Pr * 2 * Mp));
   w.part = reinterpret_cast<double*>(take(sizeof(double) * (size_t)nchunk * 2 * Pa * Pb));
-  w.err = reinterpret_cast<int*>(take(sizeof(int)));
   w.bytes = off;
   return w;
+}
+// 64-sample tiles per centring block: 8, fewer while the blocks fill less than two per SM and their
+// partial sums have room.  Float input keeps at least the 4 tiles whose samples a thread sums in
+// float before it goes to double; double input goes down to 1.
+int center_tiles(int Pr, long long M, bool in_float, int nsm, size_t rows) {
+  int nt = kCenTiles;
+  auto nblocks = [&](int n) { return (M + 64 * n - 1) / (64 * n); };
+  while (nt > (in_float ? 4 : 1) && nblocks(nt) * (Pr / 64) < 2ll * nsm && (size_t)nblocks(nt / 2) <= rows) nt /= 2;
+  return nt;
 }
 }  // namespace
 
@@ -698,6 +797,23 @@ static cudaError_t encode_tile_map(CUtensorMap* map, const __half* base, int P, 
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+template <int TB>
+static cudaError_t launch_tc(const LinWs& L, int P, long long M, long long Mp, const LinGrid& G, cudaStream_t st) {
+  // A tiles: 128 rows of X; B tiles: TB rows of X and of Y
+  const int Pa = rows_a(P), Pb = rows_b(P), Pr = rows_t(P);
+  CUtensorMap mA, mBX, mBY;
+  cudaError_t e = encode_tile_map(&mA, L.XI, P, Pr, Mp, kTa);
+  if (e == cudaSuccess) e = encode_tile_map(&mBX, L.XI, P, Pr, Mp, TB);
+  if (e == cudaSuccess) e = encode_tile_map(&mBY, L.YI, P, Pr, Mp, TB);
+  if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(lin_tc_kernel<TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, TcShape<TB>::kSmem);
+  if (e != cudaSuccess) return e;
+  const int ntile = (Pa / kTa) * ((P + TB - 1) / TB);
+  lin_tc_kernel<TB><<<dim3(ntile, G.nchunk), kTcThreads, TcShape<TB>::kSmem, st>>>(mA, mBX, mBY, Pa, Pb, M, G.chunk,
+                                                                                   L.part, L.err);
+  return cudaGetLastError();
+}
+
 template <class Tin>
 static cudaError_t launch_lin_t(int P, long long M, const Tin* O, const Tin* dEL, const double* E, const double* w,
                                 void* ws, size_t ws_bytes, int nsm, double* E0, double* gL, double* gR, double* S,
@@ -707,13 +823,13 @@ static cudaError_t launch_lin_t(int P, long long M, const Tin* O, const Tin* dEL
   };
   const int L1 = 2 * P + 2, Pa = rows_a(P), Pb = rows_b(P), Pr = rows_t(P);
   const long long Mp = (M + 31) / 32 * 32;
-  const int nb2 = (int)((M + 64 * kCenTiles - 1) / (64 * kCenTiles));
   const LinGrid G = lin_grid(P, M, nsm);
   const int nb1 = (int)((M + kColBlock - 1) / kColBlock);
   const LinWs L = carve(ws, P, M, G.nchunk);
   if (L.bytes > ws_bytes) return cudaErrorInvalidValue;  // workspace sized for another grid
-  cudaError_t e = cudaMemsetAsync(L.mx, 0, sizeof(unsigned) * (2 + 2 * (size_t)P), st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(L.err, 0, sizeof(int), st);
+  const int nt = center_tiles(Pr, M, std::is_same<Tin, float>::value, nsm, L.part2_rows);
+  const int nb2 = (int)((M + 64 * nt - 1) / (64 * nt));
+  cudaError_t e = cudaMemsetAsync(L.mx, 0, L.zero_bytes, st);
   if (e != cudaSuccess) return e;
   mark(0);
   // 16-byte loads of the [M][P] inputs when every row starts on a 16-byte boundary
@@ -723,37 +839,36 @@ static cudaError_t launch_lin_t(int P, long long M, const Tin* O, const Tin* dEL
     lin_colsum_kernel<Tin, true><<<gcol, kColBlock, 0, st>>>(P, M, O, dEL, E, w, L.part1, L.mx, nb1);
   else
     lin_colsum_kernel<Tin, false><<<gcol, kColBlock, 0, st>>>(P, M, O, dEL, E, w, L.part1, L.mx, nb1);
-  lin_seg_reduce<<<dim3((L1 + 31) / 32, kSeg), 256, 0, st>>>(L1, nb1, L.part1, L.seg);
-  lin_final_reduce<<<(L1 + 255) / 256, 256, 0, st>>>(L1, L.seg, L.acc);
-  lin_scale_kernel<<<(Pr + 255) / 256, 256, 0, st>>>(P, Pr, L.acc, L.mx, L.scl);
-  lin_sample_kernel<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(M, E, w, L.rw, L.Ef);
+  const int nq = (L1 + 7) / 8, ns = (int)std::min<long long>((M + 4 * kStatThreads - 1) / (4 * kStatThreads), 256);
+  lin_stats_kernel<<<nq + ns, kStatThreads, 0, st>>>(P, Pr, nb1, L.part1, L.mx, L.acc, L.scl, nq, M, E, w, L.rw, L.Ef);
   mark(1);
-  if (vec)
-    lin_center_kernel<Tin, true><<<dim3(Pr / 64, (unsigned)std::min(nb2, 65535)), 256, 0, st>>>(
-        P, M, Mp, O, dEL, E, w, L.rw, L.Ef, L.acc, L.scl, Pr, L.XI, L.YI, L.part2, nb2);
-  else
-    lin_center_kernel<Tin, false><<<dim3(Pr / 64, (unsigned)std::min(nb2, 65535)), 256, 0, st>>>(
-        P, M, Mp, O, dEL, E, w, L.rw, L.Ef, L.acc, L.scl, Pr, L.XI, L.YI, L.part2, nb2);
-  lin_seg_reduce<<<dim3((Pr + 31) / 32, kSeg), 256, 0, st>>>(Pr, nb2, L.part2, L.seg);
-  lin_final_reduce<<<(Pr + 255) / 256, 256, 0, st>>>(Pr, L.seg, L.sxe);
+  const dim3 gcen(Pr / 64, (unsigned)std::min(nb2, 65535));
+  auto center = [&](auto kernel) {
+    kernel<<<gcen, 256, 0, st>>>(P, M, Mp, O, dEL, E, w, L.rw, L.Ef, L.acc, L.scl, Pr, L.XI, L.YI, L.part2, nb2);
+  };
+  auto center_nt = [&](auto tiles) {
+    constexpr int NT = decltype(tiles)::value;
+    if (vec) center(lin_center_kernel<Tin, true, NT>);
+    else center(lin_center_kernel<Tin, false, NT>);
+  };
+  if (nt == 8) center_nt(std::integral_constant<int, 8>{});
+  else if (nt == 4) center_nt(std::integral_constant<int, 4>{});
+  else if constexpr (std::is_same<Tin, double>::value) {
+    if (nt == 2) center_nt(std::integral_constant<int, 2>{});
+    else center_nt(std::integral_constant<int, 1>{});
+  }
   mark(2);
-  // A tiles: 128 rows of X; B tiles: 112 rows of X and of Y
-  CUtensorMap mA, mBX, mBY;
-  e = encode_tile_map(&mA, L.XI, P, Pr, Mp, kTa);
-  if (e == cudaSuccess) e = encode_tile_map(&mBX, L.XI, P, Pr, Mp, kTb);
-  if (e == cudaSuccess) e = encode_tile_map(&mBY, L.YI, P, Pr, Mp, kTb);
+  // the narrowest tiles whose CTAs still run in one wave
+  auto ctas = [&](int tb) { return (long long)(Pa / kTa) * ((P + tb - 1) / tb) * G.nchunk; };
+  e = ctas(32) <= nsm ? launch_tc<32>(L, P, M, Mp, G, st)
+                      : (ctas(64) <= nsm ? launch_tc<64>(L, P, M, Mp, G, st) : launch_tc<kTb>(L, P, M, Mp, G, st));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(lin_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
-  if (e != cudaSuccess) return e;
-  const int ntile = (Pa / kTa) * (Pb / kTb);
-  lin_tc_kernel<<<dim3(ntile, G.nchunk), kTcThreads, kTcSmem, st>>>(mA, mBX, mBY, Pa, Pb, M, G.chunk, L.part,
-                                                                     L.err);
   mark(3);
-  const long long nq = std::max<long long>((long long)P * P, 1);
-  lin_reduce_kernel<<<(int)((nq + 255) / 256), 256, 0, st>>>(P, Pa, Pb, Pr, G.nchunk, L.part, L.acc, L.sxe, L.scl,
-                                                              E0, gL, gR, S, H, L.err);
+  const int nj = (P + kRedThreads - 1) / kRedThreads;
+  lin_reduce_kernel<<<P * nj + (P + 7) / 8, kRedThreads, 0, st>>>(P, Pa, Pb, Pr, G.nchunk, nj, nb2, L.part, L.acc,
+                                                                  L.part2, L.scl, E0, gL, gR, S, H, L.err);
   mark(4);
-  *nlaunch = 11;
+  *nlaunch = 5;
   return cudaGetLastError();
 }
 
