@@ -11,61 +11,6 @@ namespace vbq {
 
 namespace {
 
-// Lane-group LU + inverse of every unique determinant of spin sp from the double orbital
-// values PhiD[(e0 + e) * ld + idx[u][o]]: Bt[u] = A^-1 in the bulk type, ln|det|, sign,
-// t_u = tr(A^-1 L) with L read at Lphi[(e0 + e) * ldL + idx[u][o]]; the double inverse is
-// also written to st_binv[u] when st_binv is not null.
-template <class Tb>
-__device__ __forceinline__ void lu_det_all(const SysDev& s, int sp, int lane, const double* PhiD, int ld,
-                                           const Tb* Lphi, int ldL, const int* idx, int G, Tb* Bt, double* scr,
-                                           double* ldet, double* dsg, double* tdet, double* st_binv) {
-  const int n = s.n[sp], U = s.U[sp], e0 = sp ? s.Nup : 0;
-  if (n == 0) {
-    for (int u = lane; u < U; u += 32) {
-      ldet[u] = 0.0;
-      dsg[u] = 1.0;
-      tdet[u] = 0.0;
-    }
-    __syncwarp();
-    return;
-  }
-  const LaneGroup lgp(lane, G);
-  const int ng = lgp.ng, g = lgp.g, gl = lgp.gl;
-  double* A = scr + g * n * n;
-  double* B = scr + ng * n * n + g * n * n;
-  int* perm = reinterpret_cast<int*>(scr + 2 * ng * n * n) + g * n;
-  for (int u0 = 0; u0 < U; u0 += ng) {
-    const int u = u0 + g;
-    const bool act = u < U;
-    if (act && gl < n) {  // lane gl fills column (orbital slot) gl
-      const int col = __ldg(idx + u * n + gl);
-      for (int e = 0; e < n; ++e) A[e * n + gl] = PhiD[(e0 + e) * ld + col];
-    }
-    __syncwarp();
-    double lg, sg;
-    group_lu_inverse(A, B, perm, n, gl, G, act, lg, sg);
-    __syncwarp();
-    double t = 0.0;
-    if (act && gl < n) {
-      const int o = gl, col = __ldg(idx + u * n + o);
-      for (int e = 0; e < n; ++e) t = fma(B[o * n + e], (double)Lphi[(e0 + e) * ldL + col], t);
-    }
-    t = group_sum(t, G);
-    if (act) {
-      for (int q = gl; q < n * n; q += G) {
-        Bt[u * n * n + q] = (Tb)B[q];
-        if (st_binv) st_binv[u * n * n + q] = B[q];
-      }
-      if (gl == 0) {
-        ldet[u] = lg;
-        dsg[u] = sg;
-        tdet[u] = t;
-      }
-    }
-    __syncwarp();
-  }
-}
-
 template <class Tb>
 __device__ __forceinline__ void det_body(const SysDev& s, const DetLayout& L, int w, unsigned char* base,
                                          const Tb* JG, const Tb* JL, const double* JS, const Tb* OB,
@@ -168,10 +113,15 @@ __device__ __forceinline__ void det_body(const SysDev& s, const DetLayout& L, in
     __syncwarp();
   } else {
     double* st = state_out ? state_out + (size_t)w * s.state_doubles : nullptr;
-    lu_det_all<Tb>(s, 0, lane, PhiD, nevd, Lphi, nev, s.det_ev[0], L.G0, Bt[0], reinterpret_cast<double*>(scr), ldet,
-                   dsg, tdet, st);
-    lu_det_all<Tb>(s, 1, lane, PhiD, nevd, Lphi, nev, s.det_ev[1], L.G1, Bt[1], reinterpret_cast<double*>(scr),
-                   ldet + U0, dsg + U0, tdet + U0, st ? st + nb0 : nullptr);
+    for (int sp = 0; sp < 2; ++sp) {
+      const int uo = sp ? U0 : 0;
+      double* Bd = nullptr;
+      float* Bf = nullptr;
+      if constexpr (kSameType<Tb, double>) Bd = Bt[sp];
+      else Bf = Bt[sp];
+      invert_all<Tb>(s, sp, lane, PhiD, nevd, s.det_ev[sp], sp ? L.G1 : L.G0, Bd, Bf, st ? st + (sp ? nb0 : 0) : nullptr,
+                     reinterpret_cast<int*>(scr), ldet + uo, dsg + uo, Lphi, nev, tdet + uo);
+    }
     term_ratios(s, lane, ldet, dsg, rk, lnPhi, sgnPhi);
     if (st) {
       for (int q = lane; q < Utot; q += 32) {

@@ -110,12 +110,6 @@ __device__ __forceinline__ void dettab_body(const SysDev& s, const DetTabLayout&
     const int* xl = s.tab_x[sp];
     int Gs = 1;
     while (Gs < n) Gs <<= 1;
-    const LaneGroup lg(lane, Gs);
-    const bool act = lg.g == 0;  // one group: n <= 32
-    if (act && lg.gl < n) {
-      const int col = __ldg(ref + lg.gl);
-      for (int e = 0; e < n; ++e) A[e * n + lg.gl] = OD[((size_t)w * N + e0 + e) * nevd + col];
-    }
     for (int i = lane; i < n * nevd; i += 32) {
       const int e = i / nevd, q = i - e * nevd;
       const Tb* ob = OB + ((size_t)w * N + e0 + e) * 5 * nev;
@@ -125,12 +119,15 @@ __device__ __forceinline__ void dettab_body(const SysDev& s, const DetTabLayout&
                      (double)g[2] * (double)ob[3 * nev + q]);
     }
     __syncwarp();
-    double lg0 = 0.0, sg0 = 1.0;
     double* B = Bd[sp];
-    group_lu_inverse(A, B, perm, n, lg.gl, Gs, act, lg0, sg0);
-    lg0 = __shfl_sync(kFull, lg0, 0);
-    sg0 = __shfl_sync(kFull, sg0, 0);
-    __syncwarp();
+    double lg0 = 0.0, sg0 = 1.0;
+    {  // one group (n <= 32): group 0
+      const GroupDet d = group_inverse<Tb>(OD + ((size_t)w * N + e0) * nevd, nevd, ref, n, Gs, lane < Gs, perm, B,
+                                           nullptr, nullptr, nullptr, 0);
+      sg0 = (double)__shfl_sync(kFull, d.sgn, 0);
+      const double mant = __shfl_sync(kFull, d.mant, 0);
+      lg0 = sg0 != 0.0 ? log(mant) + (double)__shfl_sync(kFull, d.ex, 0) * 0.6931471805599453 : -INFINITY;
+    }
     // Y0 = B L_0 (into A), t0 = tr Y0
     for (int i = lane; i < n * n; i += 32) {
       const int o = i / n, o2 = i - o * n, col = __ldg(ref + o2);

@@ -74,8 +74,8 @@ int make_det_layout(const SysDev& s, int tb, int max_smem, DetLayout& L, bool ca
   L.rk = take(8 * s.nterm);
   int scr = 16;
   for (int sp = 0; sp < 2; ++sp) {
-    const int n = s.n[sp], G = sp ? L.G1 : L.G0, ng = 32 / G;
-    if (!carried) scr = std::max(scr, ng * (16 * n * n + 4 * n) + 16);  // LU: A, inverse, pivots per group
+    const int n = s.n[sp], G = sp ? L.G1 : L.G0;
+    if (!carried) scr = std::max(scr, inverse_scratch_bytes(n, s.U[sp], G));
     scr = std::max(scr, 8 * s.U[sp] * n);                  // carried state: trace partials
   }
   // Gam and Aux rows of both spins, one product B_u L_u

@@ -196,17 +196,8 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
           }
           int G = 1;
           while (G < n) G <<= 1;
-          const LaneGroup lg(lane, G);
-          const bool act = lg.g == 0;
-          double* A = scr;
-          int* perm = reinterpret_cast<int*>(scr + n * n);
-          if (act && lg.gl < n) {
-            const int col = __ldg(s.det_loc[sp] + lg.gl);
-            for (int e = 0; e < n; ++e) A[e * n + lg.gl] = PhiO[(e0 + e) * ldo + col];
-          }
-          __syncwarp();
-          double lgd, sgd;
-          group_lu_inverse(A, Binv[sp], perm, n, lg.gl, G, act, lgd, sgd);
+          group_inverse<double>(PhiO + e0 * ldo, ldo, s.det_loc[sp], n, G, lane < G, reinterpret_cast<int*>(scr),
+                                Binv[sp], nullptr, nullptr, nullptr, 0);
           const double* B = Binv[sp];
           for (int t = lane; t < n * nx; t += 32) {
             const int o = t / nx, x = t - o * nx, col = __ldg(s.tab_xl[sp] + x);
@@ -224,10 +215,9 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
           sg = fma(__ldg(s.term_coef + k), wk[__ldg(s.term_det + 2 * k)] * wk[U0 + __ldg(s.term_det + 2 * k + 1)], sg);
         Sig = warp_sum(sg);
       } else {
-        lu_all(s, 0, lane, PhiO, ldo, (const double*)nullptr, 0, s.det_loc[0], L.G0, Binv[0], scr, ldet, dsg,
-               nullptr);
-        lu_all(s, 1, lane, PhiO, ldo, (const double*)nullptr, 0, s.det_loc[1], L.G1, Binv[1], scr, ldet + U0,
-               dsg + U0, nullptr);
+        for (int sp = 0; sp < 2; ++sp)
+          invert_all<double>(s, sp, lane, PhiO, ldo, s.det_loc[sp], sp ? L.G1 : L.G0, Binv[sp], nullptr, nullptr,
+                             reinterpret_cast<int*>(scr), ldet + (sp ? U0 : 0), dsg + (sp ? U0 : 0), nullptr, 0, nullptr);
       }
     }
     if (!TAB && do_refresh) {

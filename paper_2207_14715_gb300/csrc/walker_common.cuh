@@ -230,13 +230,15 @@ __device__ __forceinline__ void pade_eval(const PadeCoef& c, Tb r, Tb kap, Tb& f
   pade_poly<Tb, DERIV>(r, kap, (Tb)c.a1, (Tb)c.a2, q, f, df, d2f);
 }
 
-// Lane-group LU + inverse of every unique determinant of spin sp, from orbital values
-// Phi[(e0 + e) * ld + idx[u][o]].  Writes Binv[u], ldet[u], dsg[u] (and, if Lphi is given,
-// t[u] = tr(Binv L_occ) with L read at Lphi[(e0 + e) * ldL + idx[u][o]]).
-template <class TP, class TL>
-__device__ __forceinline__ void lu_all(const SysDev& s, int sp, int lane, const TP* Phi, int ld, const TL* Lphi,
-                                       int ldL, const int* idx, int G, double* Binv, double* scr, double* ldet,
-                                       double* dsg, double* tdet) {
+// Inverse of every unique determinant of spin sp by lane groups, from the double orbital values
+// Phi[(e0 + e) * ld + idx[u][o]]: ldet[u], dsg[u], and each where given Bd[u], Bg[u] (double) and
+// Bf[u] (float), and t[u] = tr(A_u^-1 L) with L read at Lphi[(e0 + e) * ldL + idx[u][o]].
+// scr: inverse_scratch_bytes.
+__host__ __device__ inline int inverse_scratch_bytes(int n, int U, int G) { return 4 * ((32 / G) * n + U) + 16; }
+template <class Tb>
+__device__ __forceinline__ void invert_all(const SysDev& s, int sp, int lane, const double* Phi, int ld, const int* idx,
+                                           int G, double* Bd, float* Bf, double* Bg, int* scr, double* ldet,
+                                           double* dsg, const Tb* Lphi, int ldL, double* tdet) {
   const int n = s.n[sp], U = s.U[sp], e0 = sp ? s.Nup : 0;
   if (n == 0) {
     for (int u = lane; u < U; u += 32) {
@@ -248,33 +250,24 @@ __device__ __forceinline__ void lu_all(const SysDev& s, int sp, int lane, const 
     return;
   }
   const LaneGroup lgp(lane, G);
-  const int ng = lgp.ng, g = lgp.g, gl = lgp.gl;
-  double* A = scr + g * n * n;
-  int* perm = reinterpret_cast<int*>(scr + ng * n * n) + g * n;
+  const int ng = lgp.ng, g = lgp.g;
+  int* ex = scr + ng * n;
   for (int u0 = 0; u0 < U; u0 += ng) {
     const int u = u0 + g;
     const bool act = u < U;
-    if (act && gl < n) {  // lane gl fills column (orbital slot) gl
-      const int col = __ldg(idx + u * n + gl);
-      for (int e = 0; e < n; ++e) A[e * n + gl] = (double)Phi[(e0 + e) * ld + col];
-    }
-    __syncwarp();
-    double lg, sg;
-    double* B = Binv + (act ? u : 0) * n * n;
-    group_lu_inverse(A, B, perm, n, gl, G, act, lg, sg);
-    double t = 0.0;
-    if (tdet && act && gl < n) {
-      const int o = gl, col = __ldg(idx + u * n + o);
-      for (int e = 0; e < n; ++e) t = fma(B[o * n + e], (double)Lphi[(e0 + e) * ldL + col], t);
-    }
-    t = group_sum(t, G);
-    if (act && gl == 0) {
-      ldet[u] = lg;
-      dsg[u] = sg;
-      if (tdet) tdet[u] = t;
+    const int o = (act ? u : 0) * n * n;
+    const GroupDet d = group_inverse<Tb>(Phi + e0 * ld, ld, idx + (act ? u : 0) * n, n, G, act, scr + g * n,
+                                         Bd ? Bd + o : nullptr, Bf ? Bf + o : nullptr, Bg ? Bg + o : nullptr,
+                                         Lphi ? Lphi + e0 * ldL : nullptr, ldL);
+    if (act && lgp.gl == 0) {
+      ldet[u] = d.mant;
+      ex[u] = d.ex;
+      dsg[u] = (double)d.sgn;
+      if (tdet) tdet[u] = d.trace;
     }
     __syncwarp();
   }
+  finish_logdets(U, lane, ldet, ex, dsg);
 }
 
 // r_k = D_k/Phi for every determinant term and ln|Phi|, sign(Phi) (structure sum in the log

@@ -137,6 +137,30 @@ __device__ __forceinline__ double f2d_bits(float f) {
                                           ((unsigned long long)(u & 0x80000000u) << 32)));
 }
 
+// double -> float, round to nearest even, on the bit pattern; values outside the normal float
+// range take the conversion.
+__device__ __forceinline__ float d2f_bits(double x) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const unsigned ex = (unsigned)(b >> 52) & 0x7ffu;
+  if (ex < 897u || ex > 1150u) return (float)x;
+  unsigned long long m = (b & 0x7fffffffffffffffull) - (896ull << 52);
+  m += 0x0fffffffull + ((m >> 29) & 1ull);
+  return __uint_as_float((unsigned)(m >> 29) | ((unsigned)(b >> 32) & 0x80000000u));
+}
+
+// the bulk type to double and back without the FP64 pipe
+__device__ __forceinline__ double widen(float x) { return f2d_bits(x); }
+__device__ __forceinline__ double widen(double x) { return x; }
+template <class T> __device__ __forceinline__ T narrow(double x);
+template <> __device__ __forceinline__ double narrow<double>(double x) { return x; }
+template <> __device__ __forceinline__ float narrow<float>(double x) { return d2f_bits(x); }
+
+// x != 0 and |x| < inf on the bit patterns (a comparison of doubles runs on the FP64 pipe)
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+__device__ __forceinline__ bool finite_bits(double x) {
+  return ((unsigned)__double2hiint(x) & 0x7ff00000u) != 0x7ff00000u;
+}
+
 // a < b for a >= 0 and b >= 0 or NaN (false for NaN), on the bit patterns: for non-negative
 // doubles their order is the order of the patterns as integers
 __device__ __forceinline__ bool less_nonneg(double a, double b) {
@@ -145,103 +169,136 @@ __device__ __forceinline__ bool less_nonneg(double a, double b) {
 }
 
 // ------------------------------------------------------------------------------------
-// Lane-group LU with partial pivoting and explicit inverse.
-// A (n x n, row-major, rows = electrons, columns = orbital slots) is overwritten with its
-// LU factors; Binv receives A^{-1} row-major ([slot][electron]).  A group of G lanes
-// (G = power of two >= n) handles one matrix; every lane of the warp must call this with
-// the same n and G (inactive groups pass active = false).  Pivot ties go to the lowest row.
-// Returns ln|det A| and sign(det A) in every lane of the group; a zero pivot gives
-// sign 0, ln|det| = -inf and a zero inverse.
+// Lane-group inverse of a Slater matrix, in registers.
+// A group of G lanes (G = power of two >= n, n <= 32) inverts one n x n matrix A (rows =
+// electrons, columns = orbital slots): lane o holds column o of A, that is row o of A^T, and A^T
+// is inverted in place by Gauss-Jordan elimination with partial pivoting over the lanes.  Step c
+// eliminates electron c: the pivot lane p is the one, among those not yet chosen, with the
+// largest |a_c|; its row is broadcast by shuffles and every lane subtracts its multiple.  The
+// registers move down by one per step (the finished column enters at the end), so that the loop
+// over c stays rolled with every register index a constant.  After n steps lane p(i), i its own
+// step, holds A^-1[p(j)][i] in register j.
+//
+// Bound: the FP64 pipe (64 cycles per warp instruction of an SM sub-partition, whatever its active
+// lanes): n + 4 instructions per step (a reciprocal, the multiplier, n - 1 updates).  The
+// factorisation in shared memory that this replaces issued about as many but waited for them: each
+// lane walked its own row serially, with the rows of a group 8 n bytes apart (16-way bank
+// conflicts at n = 8).
+//
+// Every lane of the warp calls this with the same n and G (inactive groups pass active = false).
+// Phi [n][ld] holds the orbital values of the spin's electrons, idx [n] the column of each slot (null:
+// column o).  Bd may be Phi itself (ld = n): the values are read first.
+// Outputs, row-major [slot][electron], each may be null: Bd, Bg in double, Bf in float.  perm: n
+// ints per group.  If Lphi is given, 'trace' returns tr(A^-1 L), L read at Lphi[e * ldL + idx[o]].
+// det A = sgn * mant * 2^ex; a zero pivot gives sgn = 0, mant = 1 and a zero inverse.
 // ------------------------------------------------------------------------------------
-__device__ __forceinline__ void group_lu_inverse(double* A, double* Binv, int* perm, int n, int glane, int G,
-                                                 bool active, double& logdet, double& sgn) {
-  double s = 1.0;
-  bool singular = false;
-  if (active && glane < n) perm[glane] = glane;
-  __syncwarp();
-  for (int c = 0; c < n; ++c) {
-    double v = (active && glane >= c && glane < n) ? fabs(A[glane * n + c]) : -1.0;
-    int idx = glane;
-    for (int o = G >> 1; o > 0; o >>= 1) {
-      const double ov = __shfl_xor_sync(kFull, v, o, G);
-      const int oi = __shfl_xor_sync(kFull, idx, o, G);
-      if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
-    }
-    if (v <= 0.0) singular = true;
-    if (idx != c) {
-      if (active && !singular)
-        for (int j = glane; j < n; j += G) {
-          const double t = A[c * n + j];
-          A[c * n + j] = A[idx * n + j];
-          A[idx * n + j] = t;
-        }
-      if (active && glane == 0) {
-        const int t = perm[c];
-        perm[c] = perm[idx];
-        perm[idx] = t;
-      }
-      s = -s;
-    }
-    __syncwarp();
-    // pivot reciprocal: computed by the pivot lane and broadcast (one reciprocal per column)
-    double ip = 0.0;
-    if (active && !singular && glane == c) ip = recip_dd(A[c * n + c]);
-    ip = __shfl_sync(kFull, ip, (lane_id() & ~(G - 1)) + c);
-    if (active && !singular && glane > c && glane < n) {
-      const double l = A[glane * n + c] * ip;
-      A[glane * n + c] = l;
-      for (int j = c + 1; j < n; ++j) A[glane * n + j] = fma(-l, A[c * n + j], A[glane * n + j]);
-    }
-    __syncwarp();
-  }
-  // reciprocal of the U diagonal: lane i of the group holds 1/U_ii; the back substitution
-  // multiplies by it (broadcast by shuffle) instead of dividing in every lane
-  const double dinv = (active && glane < n && !singular) ? recip_dd(A[glane * n + glane]) : 0.0;
-  if (active && glane < n) {
-    const int j = glane;
-    if (!singular) {
-      for (int i = 0; i < n; ++i) {
-        double y = (perm[i] == j) ? 1.0 : 0.0;
-        for (int k = 0; k < i; ++k) y = fma(-A[i * n + k], Binv[k * n + j], y);
-        Binv[i * n + j] = y;
-      }
-    } else {
-      for (int i = 0; i < n; ++i) Binv[i * n + j] = 0.0;
-    }
-  }
-  for (int i = n - 1; i >= 0; --i) {
-    const double di = __shfl_sync(kFull, dinv, (lane_id() & ~(G - 1)) + i);
-    if (active && glane < n && !singular) {
-      const int j = glane;
-      double x = Binv[i * n + j];
-      for (int k = i + 1; k < n; ++k) x = fma(-A[i * n + k], Binv[k * n + j], x);
-      Binv[i * n + j] = x * di;
-    }
-  }
+struct GroupDet {
+  double mant, trace;
+  int ex, sgn;
+};
 
-  // ln|det| = ln prod |U_ii|: the product of the mantissas (each in [1, 2)) and the sum of the
-  // binary exponents over the group, then one logarithm (no overflow for n <= 32)
-  double mant = 1.0;
-  int ex = 0, neg = 0;
-  if (active && glane < n && !singular) {
-    const double d = A[glane * n + glane];
-    const long long bits = __double_as_longlong(fabs(d));
-    ex = (int)((bits >> 52) & 0x7ff) - 1023;
-    mant = __longlong_as_double((bits & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
-    neg = d < 0.0 ? 1 : 0;
+
+template <int NMAX, class Tb>
+__device__ __forceinline__ GroupDet group_inverse_n(const double* Phi, int ld, const int* idx, int n, int G, bool active,
+                                                    int* perm, double* Bd, float* Bf, double* Bg, const Tb* Lphi,
+                                                    int ldL) {
+  const int lane = lane_id(), gl = lane & (G - 1), gbase = lane & ~(G - 1);
+  const bool mineact = active && gl < n;
+  double a[NMAX];
+  {
+    const int col = mineact ? (idx ? __ldg(idx + gl) : gl) : 0;
+#pragma unroll
+    for (int e = 0; e < NMAX; ++e) a[e] = (mineact && e < n) ? Phi[e * ld + col] : 0.0;
+  }
+  bool used = !mineact, singular = false;
+  unsigned chosen = 0;
+  int par = 0, mine = 0;
+  double piv = 1.0;
+  for (int c = 0; c < n; ++c) {
+    // the largest |a_0| over the lanes not yet chosen, to 15 bits of its mantissa (enough for
+    // stability); ties go to the lowest lane
+    unsigned key = used ? 0u : (0x80000000u | ((unsigned)__double2hiint(a[0]) & 0x7fffffe0u) | (31u - (unsigned)gl));
+    for (int o = G >> 1; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(kFull, key, o, G));
+    const int p = 31 - (int)(key & 31u);
+    const int src = gbase + p;
+    const double pv = __shfl_sync(kFull, a[0], src & 31);
+    const bool zero = (__double_as_longlong(pv) << 1) == 0;
+    singular |= zero;
+    const double ip = zero ? 0.0 : recip_dd(pv);
+    const bool isp = gl == p;
+    const double t = isp ? -ip : a[0] * ip;
+#pragma unroll
+    for (int j = 1; j < NMAX; ++j) {
+      if (j < n) {
+        const double aj = __shfl_sync(kFull, a[j], src & 31);
+        a[j - 1] = fma(-t, aj, isp ? 0.0 : a[j]);
+      } else if (j == n) {
+        a[j - 1] = -t;
+      }
+    }
+    if (n == NMAX) a[NMAX - 1] = -t;
+    if (isp && !used) {
+      mine = c;
+      used = true;
+      piv = pv;
+    }
+    par ^= __popc((chosen >> p) >> 1) & 1;
+    chosen |= 1u << p;
+    if (active && gl == 0) perm[c] = p;
+  }
+  __syncwarp();
+  GroupDet r;
+  // ln|det| later from the product of the pivots' mantissas (each in [1, 2): no overflow for
+  // n <= 32) and the sum of their exponents
+  const long long bits = __double_as_longlong(piv);
+  r.mant = __longlong_as_double((bits & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
+  r.ex = mineact ? (int)((bits >> 52) & 0x7ff) - 1023 : 0;
+  unsigned neg = bits < 0 ? 1u : 0u;
+  double tr = 0.0;
+  if (mineact) {
+#pragma unroll
+    for (int j = 0; j < NMAX; ++j)
+      if (j < n) {
+        const int o = perm[j];
+        const double b = singular ? 0.0 : a[j];
+        const int q = o * n + mine;
+        if (Bd) Bd[q] = b;
+        if (Bf) Bf[q] = (float)b;
+        if (Bg) Bg[q] = b;
+        if (Lphi) tr = fma(b, widen(Lphi[mine * ldL + (idx ? __ldg(idx + o) : o)]), tr);
+      }
   }
   for (int o = G >> 1; o > 0; o >>= 1) {
-    mant *= __shfl_xor_sync(kFull, mant, o, G);
-    ex += __shfl_xor_sync(kFull, ex, o, G);
-    neg += __shfl_xor_sync(kFull, neg, o, G);
+    r.mant *= __shfl_xor_sync(kFull, r.mant, o, G);
+    r.ex += __shfl_xor_sync(kFull, r.ex, o, G);
+    neg ^= __shfl_xor_sync(kFull, neg, o, G);
   }
+  r.trace = Lphi ? group_sum(tr, G) : 0.0;
+  r.sgn = ((neg ^ (unsigned)par) & 1u) ? -1 : 1;
   if (singular) {
-    logdet = -INFINITY;
-    sgn = 0.0;
-  } else {
-    logdet = log(mant) + (double)ex * 0.6931471805599453;
-    sgn = (neg & 1) ? -s : s;
+    r.mant = 1.0;
+    r.ex = 0;
+    r.sgn = 0;
   }
+  __syncwarp();
+  return r;
+}
+
+// The three register sizes behind one call (not inlined: the callers are large and this is a
+// small part of their work).
+template <class Tb>
+__device__ __noinline__ GroupDet group_inverse(const double* Phi, int ld, const int* idx, int n, int G, bool active,
+                                               int* perm, double* Bd, float* Bf, double* Bg, const Tb* Lphi, int ldL) {
+  if (n <= 8) return group_inverse_n<8, Tb>(Phi, ld, idx, n, G, active, perm, Bd, Bf, Bg, Lphi, ldL);
+  if (n <= 16) return group_inverse_n<16, Tb>(Phi, ld, idx, n, G, active, perm, Bd, Bf, Bg, Lphi, ldL);
+  return group_inverse_n<32, Tb>(Phi, ld, idx, n, G, active, perm, Bd, Bf, Bg, Lphi, ldL);
+}
+
+// ln|det| of u = 0..U-1 from the mantissa products (in ldet), exponents and signs: one logarithm
+// per round of 32 determinants.
+__device__ __forceinline__ void finish_logdets(int U, int lane, double* ldet, const int* ex, const double* dsg) {
+  for (int u = lane; u < U; u += 32)
+    ldet[u] = dsg[u] != 0.0 ? log(ldet[u]) + (double)ex[u] * 0.6931471805599453 : -INFINITY;
   __syncwarp();
 }
 
