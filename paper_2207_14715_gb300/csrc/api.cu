@@ -148,6 +148,8 @@ int vbqmc_set_system(vbqmc_ctx* ctx, int sys_id, const vbqmc_system_desc* desc) 
     std::memcpy(&zb, &z, sizeof(zb));
     sh_pack.insert(sh_pack.end(), {h.sh_center[sh] | (h.sh_l[sh] << 16), h.sh_first[sh], sh, zb});
   }
+  std::vector<double> tab_coef(h.term_coef);
+  for (size_t k = 0; k < tab_coef.size(); ++k) tab_coef[k] *= h.tab_sgn[k];
   std::vector<float> een_cf(h.een_c.begin(), h.een_c.end());
   auto split = [](const std::vector<double>& v) {
     std::vector<float> o(2 * v.size());
@@ -187,8 +189,15 @@ int vbqmc_set_system(vbqmc_ctx* ctx, int sys_id, const vbqmc_system_desc* desc) 
                o_zf = bb.add(zeta_f), o_nf = bb.add(norm_f), o_jaf = bb.add(jas_af), o_jbf = bb.add(jas_bf),
                o_ebf = bb.add(een_Bf), o_nzf = bb.add(nuc_zf), o_nsh = bb.add(h.nuc_sh), o_sbl = bb.add(h.sh_by_l), o_shp = bb.add(sh_pack),
                o_jads = bb.add(split(h.jas_a)), o_jbds = bb.add(split(h.jas_b)), o_ecds = bb.add(split(h.een_c)), o_tx0 = bb.add(h.tab_x[0]),
-               o_tx1 = bb.add(h.tab_x[1]), o_td0 = bb.add(h.tab_det[0]), o_td1 = bb.add(h.tab_det[1]),
+               o_tx1 = bb.add(h.tab_x[1]), o_tsg = bb.add(h.tab_sgn), o_tcf = bb.add(tab_coef),
                o_txl0 = bb.add(h.tab_xl[0]), o_txl1 = bb.add(h.tab_xl[1]);
+  size_t o_min[2][vbq::kTabLists];
+  for (int sp = 0; sp < 2; ++sp) {
+    const vbq::TabMinorsHost& t = h.tab_min[sp];
+    const std::vector<int>* const v[vbq::kTabLists] = {&t.sl, &t.l1, &t.l2, &t.l3, &t.l4, &t.rt_off, &t.rt, &t.du_off,
+                                                       &t.du, &t.ld};
+    for (int k = 0; k < vbq::kTabLists; ++k) o_min[sp][k] = bb.add(*v[k]);
+  }
   cudaError_t e = cudaMalloc(&ls.blob, bb.bytes.size());
   if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(system tables)");
   ls.blob_bytes = bb.bytes.size();
@@ -241,14 +250,18 @@ int vbqmc_set_system(vbqmc_ctx* ctx, int sys_id, const vbqmc_system_desc* desc) 
   d.det_ev[1] = (const int*)(B + o_de1);
   d.tab_x[0] = (const int*)(B + o_tx0);
   d.tab_x[1] = (const int*)(B + o_tx1);
-  d.tab_det[0] = (const int*)(B + o_td0);
-  d.tab_det[1] = (const int*)(B + o_td1);
-  d.tab_ksq = 0;
-  for (int sp = 0; sp < 2; ++sp)
-    for (size_t u = 0; u * vbq::kTabStride < h.tab_det[sp].size(); ++u) {
-      const int k = h.tab_det[sp][u * vbq::kTabStride];
-      d.tab_ksq += k * k;
-    }
+  d.tab_sgn = (const double*)(B + o_tsg);
+  d.tab_coef = (const double*)(B + o_tcf);
+  for (int sp = 0; sp < 2; ++sp) {
+    const vbq::TabMinorsHost& t = h.tab_min[sp];
+    vbq::TabMinors& m = d.tab[sp];
+    m.ns = t.ns; m.nx = t.nx; m.nv = t.nv;
+    m.n1 = (int)t.l1.size() / 2; m.n2 = (int)t.l2.size() / 4; m.n3 = (int)t.l3.size() / 4; m.n4 = (int)t.l4.size() / 8;
+    m.nd = (int)t.ld.size() / 10;
+    const int** const ptr[vbq::kTabLists] = {&m.sl, &m.l1, &m.l2, &m.l3, &m.l4, &m.rt_off, &m.rt, &m.du_off, &m.du,
+                                             &m.ld};
+    for (int k = 0; k < vbq::kTabLists; ++k) *ptr[k] = (const int*)(B + o_min[sp][k]);
+  }
   d.tab_xl[0] = (const int*)(B + o_txl0);
   d.tab_xl[1] = (const int*)(B + o_txl1);
   d.n_x[0] = (int)h.tab_x[0].size();

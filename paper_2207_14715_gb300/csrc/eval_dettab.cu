@@ -2,23 +2,28 @@
 // (arXiv:2207.14715, Sec. 2.1: every determinant of a spin shares the inactive orbitals and
 // differs from the others by a few active columns), for systems whose per-determinant
 // inverses do not fit in shared memory.  One warp per walker.  Per spin:
-//   A_0 = reference determinant (u = 0), B = A_0^-1 by the lane-group LU (double);
-//   T = B Phi_X, Yhat = B L_X - (B L_0) T   over the orbitals X outside the reference;
+//   A_0 = reference determinant (u = 0), B = A_0^-1 by the lane-group inverse (double);
+//   T = B Phi_X over the orbitals X outside the reference;
 //   determinant u replaces the reference slots S_u by the orbitals Q_u (k_u <= 4):
-//     D_u = sgn_u D_0 det M_u,   M_u = T[S_u, Q_u]                (k x k, pivoted elimination)
-//     t_u = tr(A_u^-1 L_u) = tr(B L_0) + tr(M_u^-1 Yhat[S_u, Q_u])
-//     grad_i ln D_u = sum_o B[o][i] grad phi_o(r_i) + tr(M_u^-1 B[S_u][i] c_i[Q_u]),
-//     c_i[x] = grad phi_x(r_i) - sum_o grad phi_{ref o}(r_i) T[o][x],
-// where L is the Jastrow-dressed Laplacian lap phi + 2 grad ln J . grad phi.  The weighted sum
-// over determinants of the gradient term goes through Gamma[x][o] = sum_u W_u (M_u^-1)[x][o].
-// The structure sum, E_L and the structure-coefficient derivatives follow the direct kernel.
+//     D_u = sgn_u D_0 q_u,  q_u = det T[S_u, Q_u]  (tab_minors.cuh).
+// With Sigma = sum_k C_k q_up(k) q_dn(k) the derivatives of ln|Phi| with respect to the orbital
+// values phi_o(r_i) and phi_x(r_i) are
+//   h[x][i] = sum_o Gamma[o][x] B[o][i],  C[o][i] = B[o][i] - sum_x T[o][x] h[x][i],
+//   Gamma[o][x] = d ln Sigma / d T[o][x] = sum_u (d ln Sigma / d q_u) (cofactor of (o, x) in q_u),
+// which give grad_i ln|Phi| and, on the Jastrow-dressed Laplacians L = lap phi + 2 grad ln J . grad phi,
+// K[Phi]/Phi.  The traces t_u = tr(A_u^-1 L_u) are formed for structure-coefficient derivatives only.
+//
+// Bound: the FP64 pipe (about 2400 instructions per walker on 48 electrons, a quarter of them the
+// two inverses) and latency at 10 walkers per SM (22.5 KB each): 2.22 -> 0.88 ms per 4096 walkers
+// against traces and inverses of every determinant's own minor (36 KB, 6 walkers per SM).
 #include "dettab_body.cuh"
 
 namespace vbq {
 
 namespace {
+constexpr int kDetTabWarps = 12;
 template <class Tb>
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(32 * kDetTabWarps, 1)
     dettab_kernel(const SysDev s, const DetTabLayout L, int W, const Tb* __restrict__ JG, const Tb* __restrict__ JL,
                   const double* __restrict__ JS, const Tb* __restrict__ OB, const double* __restrict__ OD,
                   double* __restrict__ logpsi, double* __restrict__ sgn_out, double* __restrict__ eloc,
@@ -40,31 +45,30 @@ int make_dettab_layout(const SysDev& s, int tb, int max_smem, DetTabLayout& L) {
     off = align16(off + bytes);
     return o;
   };
-  const int N = s.N, Ut = s.U[0] + s.U[1], nevd = std::max(s.n_ev_det, 1);
+  const int N = s.N, nevd = std::max(s.n_ev_det, 1);
+  const TabMinors* m = s.tab;
   const int nmax = std::max(std::max(s.n[0], s.n[1]), 1);
-  const int nxmax = std::max(std::max(s.n_x[0], s.n_x[1]), 1);
+  const int nx = std::max(std::max(s.n[0] * s.n_x[0], s.n[1] * s.n_x[1]), 1);
+  const int nt = std::max(std::max(m[0].ns * s.n_x[0], m[1].ns * s.n_x[1]), 1);
   L.vg = take(8 * 3 * N);
   L.G = take(tb * 3 * N);
   L.B0 = take(8 * std::max(s.n[0] * s.n[0], 1));
   L.B1 = take(8 * std::max(s.n[1] * s.n[1], 1));
   L.T0 = take(8 * std::max(s.n[0] * s.n_x[0], 1));
   L.T1 = take(8 * std::max(s.n[1] * s.n_x[1], 1));
-  L.Y0 = take(8 * std::max(s.n[0] * s.n_x[0], 1));
-  L.Y1 = take(8 * std::max(s.n[1] * s.n_x[1], 1));
-  L.A = take(8 * std::max(nmax * nmax, nxmax * nmax));
-  L.Bs = take(8 * nxmax * nmax);
+  L.v0 = take(8 * m[0].nv);
+  L.v1 = take(8 * m[1].nv);
+  L.tdet = take(8 * (s.U[0] + s.U[1]));
   L.perm = take(4 * nmax);
+  L.Tn = take(8 * nt);
+  L.PX = take(8 * nx);
   L.Ls = take(8 * nmax * nevd);
-  L.ldet = take(8 * Ut);
-  L.dsg = take(8 * Ut);
-  L.tdet = take(8 * Ut);
-  L.Wdet = take(8 * Ut);
-  L.rk = take(8 * std::max(s.nterm, 1));
-  L.Minv = take(8 * std::max(s.tab_ksq, 1));  // the k_u x k_u minor inverses, packed
-  L.Gam = take(8 * nxmax * nmax);
+  L.adj = take(8 * std::max(s.U[0], s.U[1]));
+  L.gT = take(8 * nt);
+  L.Gam = take(8 * nx);
   L.warp_bytes = off;
   int wpb = max_smem / off;
-  if (wpb > 8) wpb = 8;
+  if (wpb > kDetTabWarps) wpb = kDetTabWarps;
   if (wpb < 1) return VBQMC_ERR_CAPACITY;
   L.wpb = wpb;
   return VBQMC_OK;

@@ -78,9 +78,13 @@ int make_sweep_layout(const SysDev& s, int tb, int max_smem, SweepLayout& L) {
     L.Binv1 = take(8 * s.n[1] * s.n[1]);
     L.T0 = take(8 * std::max(s.n[0] * s.n_x[0], 1));
     L.T1 = take(8 * std::max(s.n[1] * s.n_x[1], 1));
-    L.wk = take(8 * std::max(Ut, 1));
-    L.qn = take(8 * std::max(std::max(s.U[0], s.U[1]), 1));
+    const TabMinors *m = s.tab;
+    L.wk = take(8 * (m[0].nv + m[1].nv));
+    L.qn = take(8 * std::max(m[0].nv, m[1].nv));
     L.cx = take(8 * std::max(std::max(s.n_x[0], s.n_x[1]), 1));
+    L.Tn = take(8 * std::max(std::max(m[0].ns * s.n_x[0], m[1].ns * s.n_x[1]), 1));
+    L.gw = take(8 * std::max(s.U[0], s.U[1]));
+    L.wrow = take(8 * std::max(s.n[0], s.n[1]));
   } else {
     L.Binv0 = take(8 * s.U[0] * s.n[0] * s.n[0]);
     L.Binv1 = take(8 * s.U[1] * s.n[1] * s.n[1]);
@@ -95,9 +99,14 @@ int make_sweep_layout(const SysDev& s, int tb, int max_smem, SweepLayout& L) {
   L.geom = take(tb * (2 * N + s.Nn + 6 * s.Nn + 10 * (N + 1)));
   const int moves_end = off;
   off = over0;
-  L.ldet = take(8 * Ut);
-  L.dsg = take(8 * Ut);
-  L.PhiO = take(8 * N * L.nocc_max);
+  if (L.tab) {  // the X values of one spin; the reference's values are formed where its inverse goes
+    L.ldet = L.dsg = off;
+    L.PhiO = take(8 * std::max(std::max(s.n[0] * s.n_x[0], s.n[1] * s.n_x[1]), 1));
+  } else {
+    L.ldet = take(8 * Ut);
+    L.dsg = take(8 * Ut);
+    L.PhiO = take(8 * N * L.nocc_max);
+  }
   off = std::max(off, moves_end);
   int cv = 0, scr = 0;
   for (int sp = 0; sp < 2; ++sp) {

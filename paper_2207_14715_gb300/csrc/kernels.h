@@ -38,7 +38,7 @@ struct DetLayout {
 // Determinant part through the reference-determinant tables (eval_dettab.cu), warp per walker.
 struct DetTabLayout {
   int wpb = 0, warp_bytes = 0;
-  int vg, G, B0, B1, T0, T1, Y0, Y1, A, Bs, perm, Ls, ldet, dsg, tdet, Wdet, rk, Minv, Gam;
+  int vg, G, B0, B1, T0, T1, v0, v1, tdet, perm, Tn, PX, Ls, adj, gT, Gam;
 };
 
 struct EvalLayout {
@@ -53,12 +53,13 @@ struct EvalLayout {
 // inverse of every unique determinant of each spin, wk the term ratios D_k/Phi.  With the
 // reference-determinant tables (tab = 1, systems whose per-determinant inverses do not fit):
 // Binv0/Binv1 hold the reference inverse B of each spin, T0/T1 the tables T = B Phi_X
-// [n][n_x], wk the replacement determinants q_u = D_u/D_0 of both spins [U0 + U1], qn the
-// proposed q_u of the moving electron's spin, cx the vector c_x of the move.
+// [n][n_x], wk the minors of both spins [nv0 + nv1], qn the proposed minors of the moving
+// electron's spin, cx the vector c_x of the move, Tn the proposed rows of T that the minors read,
+// gw the weights g_u of the moving spin, wrow the row v^T B - e_i of an accepted move.
 struct SweepLayout {
   int wpb = 0, warp_bytes = 0;
   int R, Rds, rtab, rtds, Binv0, Binv1, ldet, dsg, wk, PhiO, bas, vrow, part, rho, rinv, cvec, scratch, geo, geom;
-  int T0 = 0, T1 = 0, qn = 0, cx = 0;
+  int T0 = 0, T1 = 0, qn = 0, cx = 0, Tn = 0, gw = 0, wrow = 0;
   int tab = 0;
   int nocc_max;
   int G0, G1;    // lanes per determinant of the LU and Sherman-Morrison (power of two >= n)

@@ -4,56 +4,10 @@
 #pragma once
 
 #include "batch.h"
+#include "tab_minors.cuh"
 #include "walker_common.cuh"
 
 namespace vbq {
-
-// q_u = D_u / D_0 of a determinant u given by the reference-determinant tables: sign_u times
-// the k x k determinant of T[S_u, Q_u] + b[S_u] c[Q_u]^T (k <= 4; b = null: T alone), by
-// elimination with partial pivoting.  T [n][nx] row-major; td = the determinant's table row.
-__device__ __forceinline__ double tab_ratio(const double* T, int nx, const int* __restrict__ td, const double* b,
-                                            const double* c) {
-  const int k = __ldg(td);
-  double M[kMaxExc][kMaxExc];
-#pragma unroll
-  for (int i = 0; i < kMaxExc; ++i)
-#pragma unroll
-    for (int j = 0; j < kMaxExc; ++j) {
-      double v = (i == j) ? 1.0 : 0.0;
-      if (i < k && j < k) {
-        const int si = __ldg(td + 2 + i), qj = __ldg(td + 2 + kMaxExc + j);
-        v = T[si * nx + qj];
-        if (b) v = fma(b[si], c[qj], v);
-      }
-      M[i][j] = v;
-    }
-  double det = (double)__ldg(td + 1);
-#pragma unroll
-  for (int col = 0; col < kMaxExc; ++col) {
-#pragma unroll
-    for (int r = col + 1; r < kMaxExc; ++r)
-      if (fabs(M[r][col]) > fabs(M[col][col])) {
-#pragma unroll
-        for (int j = 0; j < kMaxExc; ++j) {
-          const double t = M[col][j];
-          M[col][j] = M[r][j];
-          M[r][j] = t;
-        }
-        det = -det;
-      }
-    const double p = M[col][col];
-    det *= p;
-    if (p == 0.0) return 0.0;
-    const double ip = 1.0 / p;
-#pragma unroll
-    for (int r = col + 1; r < kMaxExc; ++r) {
-      const double f = M[r][col] * ip;
-#pragma unroll
-      for (int j = col + 1; j < kMaxExc; ++j) M[r][j] = fma(-f, M[col][j], M[r][j]);
-    }
-  }
-  return det;
-}
 
 // =====================================================================================
 // VMC sweep kernel
@@ -64,12 +18,20 @@ __device__ __forceinline__ double tab_ratio(const double* T, int nx, const int* 
 //    rho_u = sum_o v_o Binv_u[o][i].
 //  - reference-determinant tables (TAB = true; systems whose per-determinant inverses do not
 //    fit in shared memory): each spin carries the inverse B of its reference determinant
-//    (u = 0), T = B Phi_X over the orbitals X outside the reference, and q_u = D_u / D_0 =
-//    sgn_u det T[S_u, Q_u].  Moving electron i to a point with orbital row v gives
+//    (u = 0), T = B Phi_X over the orbitals X outside the reference, and the minors q_u =
+//    det T[S_u, Q_u] = sgn_u D_u / D_0 (tab_minors.cuh).  Moving electron i to a point with orbital
+//    row v gives
 //      rho_0 = sum_o v_o B[o][i],  c_x = v_x - sum_o v_o T[o][x],  b = B[:, i] / rho_0,
-//      T' = T + b c^T,  q'_u = sgn_u det T'[S_u, Q_u],
-//    and Phi'/Phi = rho_0 Sigma' / Sigma with Sigma = sum_k C_k q_up(k) q_dn(k); an accepted move
-//    updates B by Sherman-Morrison, T to T' and q to q'.
+//      T' = T + b c^T,  q'_u = det T'[S_u, Q_u],
+//    and Phi'/Phi = rho_0 Sigma' / Sigma with Sigma = sum_k C_k q_up(k) q_dn(k) (C_k with the signs) =
+//    sum_u q_u g_u, where g_u = sum over the terms of u of C_k times the other spin's minor stays
+//    as it is while the electrons of one spin move; an accepted move updates B by Sherman-Morrison,
+//    T to T' and q to q'.
+//    Bound: latency at 7 walkers per SM (the walker's region), over the FP64 pipe, whose
+//    instructions are therefore counted: on 48 electrons (70 determinants per spin) about 60 per
+//    move and 55 more when it is accepted, where eliminating every determinant's matrix, summing
+//    the 256 terms and serial column sums took about 250 and 70: 16.5 -> 11.5 ms per sweep of
+//    8192 walkers.
 // Each sweep moves every electron once (Sec. 2.3.1).  The determinant inverses come from
 // the walker state written by the evaluation at the same positions, or from a fresh LU of
 // double-precision orbital values (first sweep without state, and every 'refresh' sweeps).
@@ -141,12 +103,16 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
   // [1, 2) and a binary exponent (bit operations; one logarithm per sweep instead of one per move)
   double pm = 1.0;
   int pe = 0;
-  // reference-determinant tables (TAB): T per spin, q_u of both spins in wk, proposed q_u,
-  // the move's c_x, and Sigma = sum_k C_k q_up q_dn
+  // reference-determinant tables (TAB): T per spin, the minors of both spins in wk, proposed minors,
+  // the move's c_x, the rows of T that the minors read, the weights g_u and w of the moving spin,
+  // and Sigma with its reciprocal
   double* Tt[2] = {reinterpret_cast<double*>(base + L.T0), reinterpret_cast<double*>(base + L.T1)};
   double* qn = reinterpret_cast<double*>(base + L.qn);
   double* cxv = reinterpret_cast<double*>(base + L.cx);
-  double Sig = 1.0;
+  double* Tn = reinterpret_cast<double*>(base + L.Tn);
+  double* gw = reinterpret_cast<double*>(base + L.gw);
+  double* wrow = reinterpret_cast<double*>(base + L.wrow);
+  double Sig = 1.0, iSig = 1.0;
   const bool from_state = !TAB && state && state_valid;
   if (from_state) {
     const double* st = state + (size_t)w * s.state_doubles;
@@ -163,9 +129,8 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
   for (int sw = 0; sw < nsweeps; ++sw) {
     const bool do_refresh = (sw == 0) ? !from_state : (refresh > 0 && sw % refresh == 0);
     if (do_refresh) {
-      // double-precision orbital values of every electron, then LU of every unique determinant
-      for (int e = 0; e < N; ++e) {
-        const int sp = e >= Nup ? 1 : 0;
+      // double-precision orbital values of every electron, then the inverse of every unique determinant
+      auto orbital_values = [&](int e, int sp) {  // of electron e, in vrowd
         basis_at<double, false>(s, lane, R[3 * e], R[3 * e + 1], R[3 * e + 2], basd, nullptr, nullptr, nullptr,
                                 nullptr);
         __syncwarp();
@@ -181,40 +146,47 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
           const int c0 = __ldg(s.occ_chunk_off[sp] + q), c1 = __ldg(s.occ_chunk_off[sp] + q + 1);
           double v = 0.0;
           for (int c = c0; c < c1; ++c) v += partd[c];
-          PhiO[e * ldo + q] = v;
+          vrowd[q] = v;
         }
         __syncwarp();
-      }
+      };
       if constexpr (TAB) {
-        // per spin: LU of the reference determinant, T = B Phi_X, every q_u
+        // per spin: the reference's matrix in place of its inverse and the X values in PhiO, then
+        // the inverse, T = B Phi_X and every minor
         for (int sp = 0; sp < 2; ++sp) {
-          const int n = s.n[sp], e0 = sp ? Nup : 0, nx = s.n_x[sp], U = s.U[sp], uo = sp ? U0 : 0;
-          if (n == 0) {
-            for (int u = lane; u < U; u += 32) wk[uo + u] = 1.0;
+          const int n = s.n[sp], e0 = sp ? Nup : 0, nx = s.n_x[sp];
+          double* B = Binv[sp];
+          double* T = Tt[sp];
+          for (int i = 0; i < n; ++i) {
+            orbital_values(e0 + i, sp);
+            for (int o = lane; o < n; o += 32) B[i * n + o] = vrowd[__ldg(s.det_loc[sp] + o)];
+            for (int x = lane; x < nx; x += 32) PhiO[i * nx + x] = vrowd[__ldg(s.tab_xl[sp] + x)];
             __syncwarp();
-            continue;
           }
-          int G = 1;
-          while (G < n) G <<= 1;
-          group_inverse<double>(PhiO + e0 * ldo, ldo, s.det_loc[sp], n, G, lane < G, reinterpret_cast<int*>(scr),
-                                Binv[sp], nullptr, nullptr, nullptr, 0);
-          const double* B = Binv[sp];
-          for (int t = lane; t < n * nx; t += 32) {
-            const int o = t / nx, x = t - o * nx, col = __ldg(s.tab_xl[sp] + x);
+          if (n > 0) {
+            int G = 1;
+            while (G < n) G <<= 1;
+            group_inverse<double>(B, n, nullptr, n, G, lane < G, reinterpret_cast<int*>(scr), B, nullptr, nullptr,
+                                  nullptr, 0);
+          }
+          for (DivStep ox(lane, max(nx, 1)); ox.hi < n && nx > 0; ox.next(nx)) {
             double v = 0.0;
-            for (int e = 0; e < n; ++e) v = fma(B[o * n + e], PhiO[(e0 + e) * ldo + col], v);
-            Tt[sp][t] = v;
+            for (int e = 0; e < n; ++e) v = fma(B[ox.hi * n + e], PhiO[e * nx + ox.lo], v);
+            T[ox.hi * nx + ox.lo] = v;
           }
           __syncwarp();
-          for (int u = lane; u < U; u += 32)
-            wk[uo + u] = tab_ratio(Tt[sp], nx, s.tab_det[sp] + u * kTabStride, nullptr, nullptr);
+          for (DivStep ox(lane, max(nx, 1)); ox.hi < s.tab[sp].ns && nx > 0; ox.next(nx))
+            Tn[ox.hi * nx + ox.lo] = T[__ldg(s.tab[sp].sl + ox.hi) * nx + ox.lo];
+          __syncwarp();
+          tab_values(s.tab[sp], lane, Tn, wk + (sp ? s.tab[0].nv : 0));
+        }
+      } else {
+        for (int e = 0; e < N; ++e) {
+          const int sp = e >= Nup ? 1 : 0;
+          orbital_values(e, sp);
+          for (int q = lane; q < s.nocc[sp]; q += 32) PhiO[e * ldo + q] = vrowd[q];
           __syncwarp();
         }
-        double sg = 0.0;
-        for (int k = lane; k < s.nterm; k += 32)
-          sg = fma(__ldg(s.term_coef + k), wk[__ldg(s.term_det + 2 * k)] * wk[U0 + __ldg(s.term_det + 2 * k + 1)], sg);
-        Sig = warp_sum(sg);
-      } else {
         for (int sp = 0; sp < 2; ++sp)
           invert_all<double>(s, sp, lane, PhiO, ldo, s.det_loc[sp], sp ? L.G1 : L.G0, Binv[sp], nullptr, nullptr,
                              reinterpret_cast<int*>(scr), ldet + (sp ? U0 : 0), dsg + (sp ? U0 : 0), nullptr, 0, nullptr);
@@ -247,6 +219,25 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
     __syncwarp();
     for (int e = 0; e < N; ++e) {
       const int sp = e >= Nup ? 1 : 0, ie = e - (sp ? Nup : 0), n = s.n[sp], G = sp ? L.G1 : L.G0;
+      if (TAB && (e == 0 || e == Nup)) {
+        // the moving spin's weights g_u and Sigma: the other spin's minors stay until the next spin
+        const double* wo = wk + (sp ? 0 : s.tab[0].nv);
+        const double* wm = wk + (sp ? s.tab[0].nv : 0);
+        double sg = 0.0;
+        for (int u = lane; u < s.U[sp]; u += 32) {
+          const int ud = u + (sp ? U0 : 0);
+          double g = 0.0;
+          for (int t = __ldg(s.det_term_off + ud); t < __ldg(s.det_term_off + ud + 1); ++t) {
+            const int k = __ldg(s.det_term + t);
+            g = fma(__ldg(s.tab_coef + k), wo[__ldg(s.term_det + 2 * k + 1 - sp)], g);
+          }
+          gw[u] = g;
+          sg = fma(wm[u], g, sg);
+        }
+        Sig = warp_sum(sg);
+        iSig = nonzero(Sig) ? recip(Sig) : 0.0;
+        __syncwarp();
+      }
       const double uacc = rtab[4 * e + 3];
       const double rn[3] = {rtab[4 * e], rtab[4 * e + 1], rtab[4 * e + 2]};
       // the proposed position as the bulk-type arithmetic reads it
@@ -291,32 +282,39 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
       const int* dl = s.det_loc[sp];
       double rphi = 0.0, r0 = 0.0, Sig_new = 0.0;
       if constexpr (TAB) {
-        // rho_0, c_x, b = B[:, i] / rho_0 (in cvec), the proposed q_u and Sigma'
-        const int nx = s.n_x[sp], uo = sp ? U0 : 0;
+        // rho_0, c_x, b = B[:, i] / rho_0 (in cvec), the proposed minors and Sigma'.  The n_x + 1
+        // column sums (the last is rho_0) share the warp: PX columns of 32 / PX partial sums.
+        const int nx = s.n_x[sp];
+        const TabMinors& tm = s.tab[sp];
         const double* B = Binv[sp];
         const double* T = Tt[sp];
-        if (lane < n) r0 = vrowd[__ldg(dl + lane)] * B[lane * n + ie];
-        r0 = warp_sum(r0);
-        for (int x = lane; x < nx; x += 32) {
-          double cc = vrowd[__ldg(s.tab_xl[sp] + x)];
-          for (int o = 0; o < n; ++o) cc = fma(-vrowd[__ldg(dl + o)], T[o * nx + x], cc);
-          cxv[x] = cc;
+        int PX = 1;
+        while (PX <= nx && PX < 32) PX <<= 1;
+        for (int cb = 0; cb <= nx; cb += PX) {
+          const int lg = __ffs(PX) - 1, c = cb + (lane & (PX - 1)), st = 32 >> lg;
+          const double* col = c < nx ? T + c : B + ie;
+          const int ld = c < nx ? nx : n;
+          double a = 0.0;
+          if (c <= nx)
+            for (int o = lane >> lg; o < n; o += st) a = fma(vrowd[__ldg(dl + o)], col[o * ld], a);
+          for (int off = PX; off < 32; off <<= 1) a += __shfl_xor_sync(kFull, a, off);
+          if (c < nx && lane < PX) cxv[c] = vrowd[__ldg(s.tab_xl[sp] + c)] - a;
+          if (nx >= cb && nx < cb + PX) r0 = __shfl_sync(kFull, a, nx - cb);
         }
-        const double ir0 = r0 != 0.0 ? 1.0 / r0 : 0.0;
+        const double ir0 = nonzero(r0) ? recip(r0) : 0.0;
         if (lane < n) cvec[lane] = B[lane * n + ie] * ir0;
         __syncwarp();
-        for (int u = lane; u < U; u += 32) qn[u] = tab_ratio(T, nx, s.tab_det[sp] + u * kTabStride, cvec, cxv);
-        __syncwarp();
-        double sg = 0.0;
-        for (int k = lane; k < s.nterm; k += 32) {
-          const int a = __ldg(s.term_det + 2 * k), b = __ldg(s.term_det + 2 * k + 1);
-          const double qa = sp == 0 ? qn[a] : wk[a], qb = sp == 1 ? qn[b] : wk[U0 + b];
-          sg = fma(__ldg(s.term_coef + k), qa * qb, sg);
+        for (DivStep ox(lane, max(nx, 1)); ox.hi < tm.ns && nx > 0; ox.next(nx)) {
+          const int o = __ldg(tm.sl + ox.hi);
+          Tn[ox.hi * nx + ox.lo] = fma(cvec[o], cxv[ox.lo], T[o * nx + ox.lo]);
         }
+        __syncwarp();
+        tab_values(tm, lane, Tn, qn);
+        double sg = 0.0;
+        for (int u = lane; u < U; u += 32) sg = fma(qn[u], gw[u], sg);
         Sig_new = warp_sum(sg);
-        rphi = (r0 != 0.0 && Sig != 0.0) ? r0 * Sig_new / Sig : 0.0;
-        if (!isfinite(rphi)) rphi = 0.0;  // an overflowing ratio is rejected (the tables are refreshed)
-        (void)uo;
+        rphi = (nonzero(r0) && nonzero(Sig)) ? r0 * Sig_new * iSig : 0.0;
+        if (!finite_bits(rphi)) rphi = 0.0;  // an overflowing ratio is rejected (the tables are refreshed)
       }
       // determinant ratios rho_u = sum_o v_occ(o) Binv_u[o][ie], RG lanes per determinant.  With
       // one pass over the determinants (the usual case) the lanes' products are formed here and
@@ -469,23 +467,33 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
       const double prob = rphi * rphi * ej;
       const bool acc = less_nonneg(uacc, prob);  // uacc in [0, 1), prob >= 0 or NaN
       if (TAB && acc) {
-        // T <- T + b c^T; B <- B - b (v^T B - e_i^T) (b = B[:, i] / rho_0, lane j owns column j:
-        // it reads only its own column before writing it); q <- q'
-        const int nx = s.n_x[sp], uo = sp ? U0 : 0;
+        // T <- T + b c^T; B <- B - b w^T with w = v^T B - e_i (lane j owns w_j); q <- q'
+        const int nx = s.n_x[sp], vo = sp ? s.tab[0].nv : 0;
         double* T = Tt[sp];
         double* B = Binv[sp];
-        for (int t = lane; t < n * nx; t += 32) {
-          const int o = t / nx, x = t - o * nx;
-          T[t] = fma(cvec[o], cxv[x], T[t]);
+        for (DivStep ox(lane, max(nx, 1)); ox.hi < n && nx > 0; ox.next(nx)) {
+          double& t = T[ox.hi * nx + ox.lo];
+          t = fma(cvec[ox.hi], cxv[ox.lo], t);
         }
         if (lane < n) {
           const int j = lane;
-          double w = (j == ie) ? -1.0 : 0.0;
-          for (int o = 0; o < n; ++o) w = fma(vrowd[__ldg(dl + o)], B[o * n + j], w);
-          for (int o = 0; o < n; ++o) B[o * n + j] = fma(-cvec[o], w, B[o * n + j]);
+          double w0 = (j == ie) ? -1.0 : 0.0, w1 = 0.0;
+          int o = 0;
+          for (; o + 1 < n; o += 2) {
+            w0 = fma(vrowd[__ldg(dl + o)], B[o * n + j], w0);
+            w1 = fma(vrowd[__ldg(dl + o + 1)], B[(o + 1) * n + j], w1);
+          }
+          if (o < n) w0 = fma(vrowd[__ldg(dl + o)], B[o * n + j], w0);
+          wrow[j] = w0 + w1;
         }
-        for (int u = lane; u < U; u += 32) wk[uo + u] = qn[u];
+        __syncwarp();
+        for (DivStep oj(lane, n); oj.hi < n; oj.next(n)) {
+          double& x = B[oj.hi * n + oj.lo];
+          x = fma(-cvec[oj.hi], wrow[oj.lo], x);
+        }
+        for (int u = lane; u < s.tab[sp].nv; u += 32) wk[vo + u] = qn[u];
         Sig = Sig_new;
+        iSig = recip(Sig);  // an accepted ratio is nonzero, so Sigma is
         if (lane < 3) {
           R[3 * e + lane] = lane == 0 ? rn[0] : (lane == 1 ? rn[1] : rn[2]);
           if constexpr (!kSameType<Tb, double>) Rds[3 * e + lane] = lane == 0 ? rnd[0] : (lane == 1 ? rnd[1] : rnd[2]);

@@ -263,6 +263,94 @@ static void make_quads(SysHost& s) {
   }
 }
 
+// The minors of one spin's reference tables (TabMinors) from its determinant rows tab_det.
+static void make_minors(const std::vector<int>& tab_det, int U, int nx, TabMinorsHost& m) {
+  typedef std::pair<std::vector<int>, std::vector<int>> Key;  // reference slots, x indices, both ascending
+  m = TabMinorsHost();
+  m.nx = nx;
+  std::vector<Key> node(U);
+  std::map<Key, int> slot;
+  std::vector<int> sl;
+  for (int u = 0; u < U; ++u) {
+    const int* t = tab_det.data() + (size_t)u * kTabStride;
+    for (int j = 0; j < t[0]; ++j) {
+      node[u].first.push_back(t[2 + j]);
+      node[u].second.push_back(t[2 + kMaxExc + j]);
+      sl.push_back(t[2 + j]);
+    }
+    slot.insert({node[u], u});
+  }
+  std::sort(sl.begin(), sl.end());
+  sl.erase(std::unique(sl.begin(), sl.end()), sl.end());
+  m.sl = sl;
+  m.ns = (int)sl.size();
+  auto row = [&](int s) { return (int)(std::lower_bound(sl.begin(), sl.end(), s) - sl.begin()); };
+  auto minor = [&](const Key& k, int i, int j) {  // without row i and column j
+    Key c = k;
+    c.first.erase(c.first.begin() + i);
+    c.second.erase(c.second.begin() + j);
+    return c;
+  };
+  // a determinant of size >= 3 needs its cofactors; an added minor the ones of its first row
+  const size_t most = std::min<size_t>(2 * (size_t)U + 256, 0x7fff);  // a slot fits the lists' 15 bits
+  for (size_t q = 0; q < node.size() && node.size() <= most; ++q) {
+    const Key k = node[q];
+    const int n = (int)k.first.size();
+    if (n < 3) continue;
+    for (int i = 0; i < ((int)q < U ? n : 1); ++i)
+      for (int j = 0; j < n; ++j) {
+        const Key c = minor(k, i, j);
+        if (slot.insert({c, (int)node.size()}).second) node.push_back(c);
+      }
+  }
+  const bool direct = node.size() > most;
+  if (direct) node.resize((size_t)U);
+  m.nv = (int)node.size();
+  const int nt = m.ns * nx;
+  const int kNeg = (int)0x80000000u;
+  std::vector<std::vector<int>> ut(nt);  // by Tn entry
+  m.du_off.assign(1, 0);
+  auto t_of = [&](int s, int x) { return row(s) * nx + x; };
+  for (int q = 0; q < m.nv; ++q) {
+    const Key& key = node[q];
+    const std::vector<int>&S = key.first, &Q = key.second;
+    const int k = (int)S.size();
+    if (k == 1) {
+      m.l1.insert(m.l1.end(), {q, t_of(S[0], Q[0])});
+    } else if (k == 2) {
+      m.l2.insert(m.l2.end(), {q, t_of(S[0], Q[0]) | t_of(S[1], Q[1]) << 16, t_of(S[0], Q[1]) | t_of(S[1], Q[0]) << 16, 0});
+    } else if (k >= 3 && direct) {
+      int e[10] = {q, k, 0, 0, 0, 0, 0, 0, 0, 0};
+      for (int j = 0; j < k; ++j) {
+        e[2 + j] = row(S[j]);
+        e[6 + j] = Q[j];
+      }
+      m.ld.insert(m.ld.end(), e, e + 10);
+    } else if (k >= 3) {
+      std::vector<int>& l = k == 3 ? m.l3 : m.l4;
+      l.push_back(q);
+      for (int j = 0; j < k; ++j) l.push_back(t_of(S[0], Q[j]) | slot.at(minor(key, 0, j)) << 16);
+      if (k == 4) l.insert(l.end(), {0, 0, 0});
+    }
+    if (q < U) {
+      if (k <= 2 || !direct)
+        for (int i = 0; i < k; ++i)
+          for (int j = 0; j < k; ++j) {
+            const int t = t_of(S[i], Q[j]), sg = ((i + j) & 1) ? kNeg : 0;
+            const int cof = k == 1 ? -1 : (k == 2 ? 0x10000 + t_of(S[1 - i], Q[1 - j]) : slot.at(minor(key, i, j)));
+            ut[t].insert(ut[t].end(), {q | sg, cof});
+            m.du.insert(m.du.end(), {t | sg, cof});
+          }
+      m.du_off.push_back((int)(m.du.size() / 2));
+    }
+  }
+  m.rt_off.assign(1, 0);
+  for (int t = 0; t < nt; ++t) {
+    m.rt.insert(m.rt.end(), ut[t].begin(), ut[t].end());
+    m.rt_off.push_back((int)(m.rt.size() / 2));
+  }
+}
+
 #define VBQ_REQUIRE(cond, msg)                 \
   do {                                         \
     if (!(cond)) {                             \
@@ -550,6 +638,13 @@ int build_system(const vbqmc_system_desc* d, SysHost& s, std::string& err) {
       }
     }
   }
+  s.tab_sgn.assign(s.term_coef.size(), 1.0);
+  for (int sp = 0; sp < 2 && s.tab_ok; ++sp) {
+    make_minors(s.tab_det[sp], s.U[sp], (int)s.tab_x[sp].size(), s.tab_min[sp]);
+  }
+  for (size_t k = 0; k < s.term_coef.size() && s.tab_ok; ++k)
+    for (int sp = 0; sp < 2; ++sp)
+      if (s.n[sp] > 0) s.tab_sgn[k] *= s.tab_det[sp][(size_t)s.term_det[2 * k + sp] * kTabStride + 1];
   // contraction work chunks
   for (int sp = 0; sp < 2; ++sp) make_chunks(s, s.occ_list[sp], s.occ_chunk[sp], s.occ_chunk_off[sp]);
   make_quads(s);

@@ -24,6 +24,28 @@ constexpr int kTabStride = 2 + 2 * kMaxExc;  // per determinant: k, sign, S[kMax
 struct EenTerm { int p, k, l, m; };
 std::vector<EenTerm> een_term_list();
 
+// Minors of the reference tables of one spin, as the kernels read them (tab_minors.cuh): the ns
+// reference slots that any determinant replaces (sl) and the nx orbitals outside the reference span
+// the rows Tn [ns][nx]; nv value slots, slot u < U the minor of determinant u, then the minors that only
+// serve larger ones.  Lists of the minors of each size, with Tn indices t and value slots c:
+//   l1 [n1][2] slot, t;  l2 [n2][4] slot, t_ax | t_by << 16, t_ay | t_bx << 16, 0;
+//   l3 [n3][4] slot, t | c << 16 for the three terms of the expansion along the first row (+ - +);
+//   l4 [n4][8] slot, the four terms (+ - + -), 0, 0, 0;
+// and the k^2 first derivatives of every determinant's minor, by Tn entry (rt: determinant with the
+// sign in bit 31, cofactor) and by determinant (du: Tn index with the sign, cofactor), the cofactor
+// as -1 for 1, a slot, or 0x10000 + t.  Where the added minors would outnumber the determinants
+// (many determinants over many orbitals), none is added and ld [nd][10] lists the determinants
+// with k >= 3 to be expanded each by itself: slot, k, the 4 rows, the 4 columns of Tn.
+struct TabMinors {
+  int ns, nx, nv, n1, n2, n3, n4, nd;
+  const int *sl, *l1, *l2, *l3, *l4, *rt_off, *rt, *du_off, *du, *ld;
+};
+constexpr int kTabLists = 10;
+struct TabMinorsHost {
+  int ns = 0, nx = 0, nv = 0;
+  std::vector<int> sl, l1, l2, l3, l4, rt_off, rt, du_off, du, ld;
+};
+
 // Everything the kernels need, as host vectors (built by build_system).
 struct SysHost {
   int N = 0, Nup = 0, Ndn = 0, Nn = 0, n_elem = 0, S = 0, M = 0, Norb = 0, Nvb = 0;
@@ -55,6 +77,8 @@ struct SysHost {
   std::vector<int> tab_x[2];
   std::vector<int> tab_det[2];
   std::vector<int> tab_xl[2];          // [n_x] position of each tab_x orbital in occ_list[spin]
+  TabMinorsHost tab_min[2];
+  std::vector<double> tab_sgn;         // [nterm] sgn_up sgn_dn of the term's determinants
   // determinant terms: unique (up, dn) pairs with merged coefficients C_k = sum_I c_I d_{I,k}
   std::vector<int> term_det;           // [nterm][2]
   std::vector<double> term_coef;       // [nterm]
@@ -132,8 +156,9 @@ struct SysDev {
   int msd;                             // determinant part through the reference-determinant tables
   int n_x[2];
   const int* tab_x[2];
-  const int* tab_det[2];
-  int tab_ksq;                         // sum over the determinants of both spins of k_u^2
+  TabMinors tab[2];
+  const double* tab_sgn;               // [nterm] signs of the term's two determinants against their minors
+  const double* tab_coef;              // [nterm] term_coef * tab_sgn
   const int* tab_xl[2];
   const int* term_det;
   const double* term_coef;
