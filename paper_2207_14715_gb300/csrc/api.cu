@@ -1,5 +1,6 @@
 // C ABI of the VB-QMC library (declared in include/vbqmc.h): context, system upload and
 // the walker entry points.
+#include <algorithm>
 #include <cstring>
 #include <string>
 #include <utility>
@@ -232,6 +233,8 @@ int vbqmc_set_system(vbqmc_ctx* ctx, int sys_id, const vbqmc_system_desc* desc) 
   d.sh_first = (const int*)(B + o_sh_first);
   d.nuc_sh = (const int*)(B + o_nsh);
   d.sh_by_l = (const int*)(B + o_sbl);
+  for (int l = 0; l < 3; ++l)
+    d.sh_l_off[l] = (int)std::count_if(h.sh_l.begin(), h.sh_l.end(), [&](int x) { return x < l; });
   d.sh_pack_f = (const int*)(B + o_shp);
   d.max_nuc_mu = h.max_nuc_mu;
   d.sh_zeta = (const double*)(B + o_sh_zeta);

@@ -166,7 +166,7 @@ int build_fused_plan(vbqmc_batch* b) {
       if (bytes[q] > smem) return fail(VBQMC_ERR_CAPACITY, "per-walker region of a batched system");
       s.cw[q] = std::max(1, std::min(T, smem / std::max(bytes[q], 1)));
     }
-    if (warps * s.lay.orb.warp_bytes > smem) return fail(VBQMC_ERR_CAPACITY, "orbital tables of a batched system");
+    if (warps * s.lay.orb.table_bytes > smem) return fail(VBQMC_ERR_CAPACITY, "orbital tables of a batched system");
     per[k] = T;
   }
   struct It {

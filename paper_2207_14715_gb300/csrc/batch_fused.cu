@@ -3,7 +3,7 @@
 // step on its tile in turn (Sec. 2.3.1: sweep of single-electron Metropolis moves, then the
 // evaluation of ln|Psi|, E_L and the parameter derivatives), with block barriers between the
 // phases: the VMC sweep (warp per walker), the Jastrow factor (warp per walker), the orbitals
-// (warps over the tile's (walker, electron) pairs), the determinant part (warp per walker) and
+// (groups of the tile's (walker, electron) points, the whole block on each), the determinant part (warp per walker) and
 // the Jastrow-parameter derivatives (warp per walker); systems on reference-determinant tables
 // take the table forms of the sweep and of the determinant part.  The phases exchange their results
 // through the systems' evaluation workspaces in global memory, written and read by the same
@@ -65,10 +65,11 @@ __global__ void __launch_bounds__(MAXT, 1) batch_fused_kernel(const BatchSys* __
                          static_cast<Tb*>(b.JG), static_cast<Tb*>(b.JL), b.JS);
     __syncthreads();
     const int npair = item.count * b.dev.N;
-    if (wl < co)
-      for (int p = wl; p < npair; p += co)
-        orbital_body<Tb>(b.dev, b.lay.orb, (long long)item.first * b.dev.N + p, smem + wl * b.lay.orb.warp_bytes,
-                         b.R, static_cast<Tb*>(b.OB), b.OD);
+    for (int p = 0; p < npair; p += co) {
+      if (p) __syncthreads();  // the previous group's regions have been read
+      orbital_block<Tb>(b.dev, b.lay.orb, (long long)item.first * b.dev.N + p, min(co, npair - p), smem, b.R,
+                        static_cast<Tb*>(b.OB), b.OD);
+    }
     __syncthreads();
     const bool d = derivs && b.O && b.dev.P > 0;
     if (wl < cd)

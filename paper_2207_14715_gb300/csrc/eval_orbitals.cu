@@ -1,7 +1,7 @@
 // Orbitals at every electron (arXiv:2207.14715, Sec. 2.1: phi_p = sum_mu lambda_{p mu} chi_mu):
 // basis functions with gradients and Laplacians, then the contraction in balanced chunks of
-// the nonzero coefficients, four orbitals of equal coefficient range at a time.  One warp per (walker, electron), so that many warps share each
-// SM; results go to the evaluation workspace:
+// the nonzero coefficients, four orbitals of equal coefficient range at a time.  One block per eight
+// (walker, electron) points; results go to the evaluation workspace:
 //   OB [W][N][5][n_ev] bulk type: phi, d/dx, d/dy, d/dz, lap phi of the evaluated orbitals
 //   OD [W][N][n_det_ev] double: values of the orbitals that enter determinants; in the mixed
 //      form these come from float-float basis values and coefficients, and OB holds them
@@ -17,25 +17,20 @@ __global__ void __launch_bounds__(32 * kOrbWarps, 4) orbital_kernel(const SysDev
                                                                      const double* __restrict__ Rg,
                                                                      Tb* __restrict__ OB, double* __restrict__ OD) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int wl = threadIdx.x >> 5;
-  const long long gw = (long long)blockIdx.x * kOrbWarps + wl;
-  if (gw >= (long long)W * s.N) return;
-  orbital_body<Tb>(s, L, gw, smem + wl * L.warp_bytes, Rg, OB, OD);
+  const long long gw0 = (long long)blockIdx.x * L.wpb;
+  orbital_block<Tb>(s, L, gw0, (int)min((long long)L.wpb, (long long)W * s.N - gw0), smem, Rg, OB, OD);
 }
 
 template <class Tb>
 __global__ void __launch_bounds__(32 * kOrbWarps, 4)
     orbital_batch_kernel(const BatchSys* __restrict__ sys, const BatchItem* __restrict__ items, int nitems) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int wl = threadIdx.x >> 5;
   for (int it = blockIdx.x; it < nitems; it += gridDim.x) {
-    // the warps' shared-memory regions depend on the item's system: start together
+    // the points' shared-memory regions depend on the item's system: start together
     __syncthreads();
     const BatchItem item = items[it];
-    if (wl >= item.count) continue;
     const BatchSys& b = sys[item.sys];
-    orbital_body<Tb>(b.dev, b.lay.orb, (long long)item.first + wl, smem + wl * b.lay.orb.warp_bytes, b.R,
-                     static_cast<Tb*>(b.OB), b.OD);
+    orbital_block<Tb>(b.dev, b.lay.orb, item.first, item.count, smem, b.R, static_cast<Tb*>(b.OB), b.OD);
   }
 }
 
@@ -54,21 +49,25 @@ int make_orb_layout(const SysDev& s, int tb, int max_smem, OrbLayout& L) {
   L.ctab = take(tb == 4 ? 8 * 4 * s.Nn : 16);
   L.part = take(5 * s.evq_width * tb * std::max(s.n_evq_chunk, 1));
   L.partd = take(tb == 4 ? 8 * std::max(s.n_det_chunk, 1) : 16);
+  L.table_bytes = off;
+  if (kOrbWarps * off > max_smem) return VBQMC_ERR_CAPACITY;  // the limit on the size of a system
+  L.r3 = take(8 * 3);
+  L.dis = take(tb * 3 * s.Nn);
+  // consecutive points 16 bytes apart in the banks: lanes on different points store side by side
+  while (off % 128 != 16) off += 16;
   L.warp_bytes = off;
-  L.wpb = kOrbWarps;
-  if (kOrbWarps * off > max_smem) return VBQMC_ERR_CAPACITY;
+  L.wpb = std::min(kOrbWarps, max_smem / off);
   return VBQMC_OK;
 }
 
 template <class Tb>
 cudaError_t launch_orbitals(const SysDev& s, const OrbLayout& L, int W, const double* R, Tb* OB, double* OD,
                             cudaStream_t st) {
-  const int smem = kOrbWarps * L.warp_bytes;
+  const int smem = L.wpb * L.warp_bytes;
   cudaError_t e = cudaFuncSetAttribute(orbital_kernel<Tb>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const long long warps = (long long)W * s.N;
-  orbital_kernel<Tb><<<(unsigned)((warps + kOrbWarps - 1) / kOrbWarps), 32 * kOrbWarps, smem, st>>>(s, L, W, R, OB,
-                                                                                                    OD);
+  const long long points = (long long)W * s.N;
+  orbital_kernel<Tb><<<(unsigned)((points + L.wpb - 1) / L.wpb), 32 * kOrbWarps, smem, st>>>(s, L, W, R, OB, OD);
   return cudaGetLastError();
 }
 

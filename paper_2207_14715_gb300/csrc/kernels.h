@@ -9,7 +9,7 @@ namespace vbq {
 
 // The evaluation runs as four kernels, each with the occupancy its own working set allows:
 //   jastrow     warp per walker: geometry tables, ln J, grad_i ln J, lap_i ln J, potential
-//   orbitals    warp per (walker, electron): basis functions and orbital values/derivatives
+//   orbitals    block per 8 (walker, electron) points: basis functions and orbital values/derivatives
 //   det         warp per walker: Slater LU + inverses, structure sum, E_L, grad ln|Psi|,
 //               structure-coefficient and orbital-excitation derivatives, walker state
 //   jastrow_d   warp per walker: Jastrow-parameter derivatives (needs grad ln|Psi|)
@@ -24,9 +24,10 @@ struct JasLayout {
   int nw = 1, wide_bytes = 0, wred = 0, wred2 = 0;
 };
 
+// wpb points per block, warp_bytes per point (table_bytes without the coordinates and padding).
 struct OrbLayout {
-  int wpb = 0, warp_bytes = 0;
-  int bas, bds, ctab, part, partd;
+  int wpb = 0, warp_bytes = 0, table_bytes = 0;
+  int bas, bds, ctab, part, partd, r3, dis;
 };
 
 struct DetLayout {

@@ -139,6 +139,7 @@ struct SysDev {
   const int* sh_l;
   const int* sh_first;
   const int* sh_by_l;
+  int sh_l_off[3];                     // first shell of each l in sh_by_l
   const int* sh_pack_f;                // [S][4] in the order of sh_by_l: center | l << 16, first function, shell, float bits of zeta
   const int* nuc_sh;                   // [Nn][4], see SysHost
   int max_nuc_mu;

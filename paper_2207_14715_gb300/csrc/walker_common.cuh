@@ -61,9 +61,7 @@ __device__ __forceinline__ dsf nuc_coord_ds(const SysDev& s, int a, int d) {
   const float2 v = __ldg(reinterpret_cast<const float2*>(s.nuc_ds) + 3 * a + d);
   return dsf{v.x, v.y};
 }
-// PACK4 (with DERIV): value and gradient of function mu as the float4 bv[4 mu .. 4 mu + 3],
-// Laplacian at bl[mu] (bx, by, bz and cs unused).
-template <bool DERIV, bool PACK4 = false>
+template <bool DERIV>
 __device__ __forceinline__ void basis_at_f(const SysDev& s, int lane, const dsf* r3, float* bv, float* bx, float* by,
                                            float* bz, float* bl, int cs = 1) {
   // the displacement from each nucleus once (lane a: nucleus a), shared by shuffles with the
@@ -92,61 +90,49 @@ __device__ __forceinline__ void basis_at_f(const SysDev& s, int lane, const dsf*
       dz = ds_diff_f(r3[2], nuc_coord_ds(s, c, 2));
     }
     if (act) {
-      if constexpr (PACK4)  // value and gradient of function f + c as one 16-byte store
-        gto_shell_emit<float, true>(l, __int_as_float(p.w), s.sh_norm_f + 6 * sh, dx, dy, dz,
-                                    [&](int c, float v, float x, float y, float w, float lp) {
-                                      reinterpret_cast<float4*>(bv)[f + c] = make_float4(v, x, y, w);
-                                      bl[f + c] = lp;
-                                    });
-      else
-        gto_shell<float, DERIV>(l, __int_as_float(p.w), s.sh_norm_f + 6 * sh, dx, dy, dz,
-                                bv + f * cs, DERIV ? bx + f * cs : nullptr, DERIV ? by + f * cs : nullptr,
-                                DERIV ? bz + f * cs : nullptr, DERIV ? bl + f : nullptr, cs);
+      gto_shell<float, DERIV>(l, __int_as_float(p.w), s.sh_norm_f + 6 * sh, dx, dy, dz, bv + f * cs,
+                              DERIV ? bx + f * cs : nullptr, DERIV ? by + f * cs : nullptr,
+                              DERIV ? bz + f * cs : nullptr, DERIV ? bl + f : nullptr, cs);
     }
   }
 }
 
-// Values of all basis functions at the point r3 (float-float) in float-float (mixed form).
-// Per center the displacement and r^2 are float-float; per shell exp(-zeta r^2) and the
-// cartesian factors are float-float.  ctab: [Nn][4] scratch (dx, dy, dz, r^2).
-__device__ __forceinline__ void basis_values_ds(const SysDev& s, int lane, const dsf* r3, dsf* ctab, dsf* out) {
-  for (int c = lane; c < s.Nn; c += 32) {
-    const dsf dx = ds_add(r3[0], ds_neg(nuc_coord_ds(s, c, 0)));
-    const dsf dy = ds_add(r3[1], ds_neg(nuc_coord_ds(s, c, 1)));
-    const dsf dz = ds_add(r3[2], ds_neg(nuc_coord_ds(s, c, 2)));
-    ctab[4 * c] = dx;
-    ctab[4 * c + 1] = dy;
-    ctab[4 * c + 2] = dz;
-    ctab[4 * c + 3] = ds_add_nc(ds_add_nc(ds_mul(dx, dx), ds_mul(dy, dy)), ds_mul(dz, dz));
-  }
-  __syncwarp();
-  for (int t = lane; t < s.S; t += 32) {
-    const int sh = __ldg(s.sh_by_l + t);
-    const int c = __ldg(s.sh_center + sh), l = __ldg(s.sh_l + sh), f = __ldg(s.sh_first + sh);
-    const float2 zt = __ldg(reinterpret_cast<const float2*>(s.sh_zeta_ds) + sh);
-    dsf e = {1.0f, 0.0f};
-    if (zt.x < 0.0f)  // Slater shell: exp(-zeta r), zeta = -z
-      e = ds_exp_neg(ds_mul(ds_sqrt(ctab[4 * c + 3]), dsf{-zt.x, -zt.y}));
-    else if (zt.x != 0.0f)
-      e = ds_exp_neg(ds_mul(ctab[4 * c + 3], dsf{zt.x, zt.y}));
-    const float2* nr = reinterpret_cast<const float2*>(s.sh_norm_ds) + 6 * sh;
-    if (l == 0) {
-      const float2 n0 = __ldg(nr);
-      out[f] = ds_mul(dsf{n0.x, n0.y}, e);
-    } else if (l == 1) {
+// Displacement of the point r3 from nucleus c and its square in float-float: ctab[4 c .. 4 c + 3].
+__device__ __forceinline__ void center_ds(const SysDev& s, int c, const dsf* r3, dsf* ctab) {
+  const dsf dx = ds_add(r3[0], ds_neg(nuc_coord_ds(s, c, 0)));
+  const dsf dy = ds_add(r3[1], ds_neg(nuc_coord_ds(s, c, 1)));
+  const dsf dz = ds_add(r3[2], ds_neg(nuc_coord_ds(s, c, 2)));
+  ctab[4 * c] = dx;
+  ctab[4 * c + 1] = dy;
+  ctab[4 * c + 2] = dz;
+  ctab[4 * c + 3] = ds_add_nc(ds_add_nc(ds_mul(dx, dx), ds_mul(dy, dy)), ds_mul(dz, dz));
+}
+// Values of the functions of shell sh (center c, angular momentum l, first function f) in
+// float-float (mixed form): exp(-zeta r^2) and the cartesian factors are float-float.
+__device__ __forceinline__ void shell_values_ds(const SysDev& s, int sh, int c, int l, int f, const dsf* ctab, dsf* out) {
+  const float2 zt = __ldg(reinterpret_cast<const float2*>(s.sh_zeta_ds) + sh);
+  dsf e = {1.0f, 0.0f};
+  if (zt.x < 0.0f)  // Slater shell: exp(-zeta r), zeta = -z
+    e = ds_exp_neg(ds_mul(ds_sqrt(ctab[4 * c + 3]), dsf{-zt.x, -zt.y}));
+  else if (zt.x != 0.0f)
+    e = ds_exp_neg(ds_mul(ctab[4 * c + 3], dsf{zt.x, zt.y}));
+  const float2* nr = reinterpret_cast<const float2*>(s.sh_norm_ds) + 6 * sh;
+  if (l == 0) {
+    const float2 n0 = __ldg(nr);
+    out[f] = ds_mul(dsf{n0.x, n0.y}, e);
+  } else if (l == 1) {
 #pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        const float2 nq = __ldg(nr + q);
-        out[f + q] = ds_mul(ds_mul(dsf{nq.x, nq.y}, ctab[4 * c + q]), e);
-      }
-    } else {
-      const int ia[6] = {0, 1, 2, 0, 0, 1};
-      const int ib[6] = {0, 1, 2, 1, 2, 2};
+    for (int q = 0; q < 3; ++q) {
+      const float2 nq = __ldg(nr + q);
+      out[f + q] = ds_mul(ds_mul(dsf{nq.x, nq.y}, ctab[4 * c + q]), e);
+    }
+  } else {
+    const int ia[6] = {0, 1, 2, 0, 0, 1};
+    const int ib[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
-      for (int q = 0; q < 6; ++q) {
-        const float2 nq = __ldg(nr + q);
-        out[f + q] = ds_mul(ds_mul(dsf{nq.x, nq.y}, ds_mul(ctab[4 * c + ia[q]], ctab[4 * c + ib[q]])), e);
-      }
+    for (int q = 0; q < 6; ++q) {
+      const float2 nq = __ldg(nr + q);
+      out[f + q] = ds_mul(ds_mul(dsf{nq.x, nq.y}, ds_mul(ctab[4 * c + ia[q]], ctab[4 * c + ib[q]])), e);
     }
   }
 }
