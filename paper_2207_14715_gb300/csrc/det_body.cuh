@@ -120,7 +120,7 @@ __device__ __forceinline__ void det_body(const SysDev& s, const DetLayout& L, in
       if constexpr (kSameType<Tb, double>) Bd = Bt[sp];
       else Bf = Bt[sp];
       invert_all<Tb>(s, sp, lane, PhiD, nevd, s.det_ev[sp], sp ? L.G1 : L.G0, Bd, Bf, st ? st + (sp ? nb0 : 0) : nullptr,
-                     reinterpret_cast<int*>(scr), ldet + uo, dsg + uo, Lphi, nev, tdet + uo);
+                     reinterpret_cast<double*>(scr), ldet + uo, dsg + uo, Lphi, nev, tdet + uo);
     }
     term_ratios(s, lane, ldet, dsg, rk, lnPhi, sgnPhi);
     if (st) {

@@ -44,17 +44,14 @@ __device__ __forceinline__ void dettab_body(const SysDev& s, const DetTabLayout&
     const int n = s.n[sp], e0 = sp ? Nup : 0, nx = s.n_x[sp];
     const TabMinors& tm = s.tab[sp];
     if (n > 0) {
-      int Gs = 1;
-      while (Gs < n) Gs <<= 1;
       const double* od = OD + ((size_t)w * N + e0) * nevd;
       for (DivStep ex(lane, max(nx, 1)); ex.hi < n && nx > 0; ex.next(nx))
         PX[ex.hi * nx + ex.lo] = od[ex.hi * nevd + __ldg(s.tab_x[sp] + ex.lo)];
       double* B = Bd[sp];
-      const GroupDet d =
-          group_inverse<Tb>(od, nevd, s.det_ev[sp], n, Gs, lane < Gs, perm, B, nullptr, nullptr, nullptr, 0);
-      const int sg = __shfl_sync(kFull, d.sgn, 0);
+      const GroupDet d = warp_inverse(od, nevd, s.det_ev[sp], n, perm, B);
+      const int sg = d.sgn;
       sg0 *= sg;
-      lg0 += sg != 0 ? log(__shfl_sync(kFull, d.mant, 0)) + (double)__shfl_sync(kFull, d.ex, 0) * 0.6931471805599453
+      lg0 += sg != 0 ? log(d.mant) + (double)d.ex * 0.6931471805599453
                      : 0.0;
       double* T = TX[sp];  // T = B Phi_X
       for (DivStep ox(lane, max(nx, 1)); ox.hi < n && nx > 0; ox.next(nx)) {

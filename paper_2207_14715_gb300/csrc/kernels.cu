@@ -112,7 +112,7 @@ int make_sweep_layout(const SysDev& s, int tb, int max_smem, SweepLayout& L) {
   for (int sp = 0; sp < 2; ++sp) {
     const int n = s.n[sp], G = sp ? L.G1 : L.G0, ng = L.tab ? 1 : 32 / G;
     cv = std::max(cv, 8 * (L.tab ? 1 : 2) * ng * n);  // Sherman-Morrison stages two passes' columns
-    scr = std::max(scr, inverse_scratch_bytes(n, L.tab ? 0 : s.U[sp], G));
+    scr = std::max(scr, L.tab ? 4 * n + 16 : inverse_scratch_bytes(n, s.U[sp], G));
   }
   // the LU scratch of a refactorisation shares its space with the buffers of the moves (the
   // basis values and partial sums that build PhiO are consumed before the LU starts)

@@ -164,10 +164,7 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
             __syncwarp();
           }
           if (n > 0) {
-            int G = 1;
-            while (G < n) G <<= 1;
-            group_inverse<double>(B, n, nullptr, n, G, lane < G, reinterpret_cast<int*>(scr), B, nullptr, nullptr,
-                                  nullptr, 0);
+            warp_inverse(B, n, nullptr, n, reinterpret_cast<int*>(scr), B);
           }
           for (DivStep ox(lane, max(nx, 1)); ox.hi < n && nx > 0; ox.next(nx)) {
             double v = 0.0;
@@ -189,7 +186,7 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
         }
         for (int sp = 0; sp < 2; ++sp)
           invert_all<double>(s, sp, lane, PhiO, ldo, s.det_loc[sp], sp ? L.G1 : L.G0, Binv[sp], nullptr, nullptr,
-                             reinterpret_cast<int*>(scr), ldet + (sp ? U0 : 0), dsg + (sp ? U0 : 0), nullptr, 0, nullptr);
+                             scr, ldet + (sp ? U0 : 0), dsg + (sp ? U0 : 0), nullptr, 0, nullptr);
       }
     }
     if (!TAB && do_refresh) {

@@ -220,12 +220,14 @@ __device__ __forceinline__ void pade_eval(const PadeCoef& c, Tb r, Tb kap, Tb& f
 // Phi[(e0 + e) * ld + idx[u][o]]: ldet[u], dsg[u], and each where given Bd[u], Bg[u] (double) and
 // Bf[u] (float), and t[u] = tr(A_u^-1 L) with L read at Lphi[(e0 + e) * ldL + idx[u][o]].
 // scr: inverse_scratch_bytes.
-__host__ __device__ inline int inverse_scratch_bytes(int n, int U, int G) { return 4 * ((32 / G) * n + U) + 16; }
+__host__ __device__ inline int inverse_scratch_bytes(int n, int U, int G) {
+  return (32 / G) * (8 * n * (n | 1) * (n > 16 ? 2 : 1) + 4 * n) + 4 * U + 16;
+}
 template <class Tb>
 __device__ __forceinline__ void invert_all(const SysDev& s, int sp, int lane, const double* Phi, int ld, const int* idx,
-                                           int G, double* Bd, float* Bf, double* Bg, int* scr, double* ldet,
+                                           int G, double* Bd, float* Bf, double* Bg, double* scr, double* ldet,
                                            double* dsg, const Tb* Lphi, int ldL, double* tdet) {
-  const int n = s.n[sp], U = s.U[sp], e0 = sp ? s.Nup : 0;
+  const int n = s.n[sp], U = s.U[sp], e0 = sp ? s.Nup : 0, lda = n | 1;
   if (n == 0) {
     for (int u = lane; u < U; u += 32) {
       ldet[u] = 0.0;
@@ -236,20 +238,43 @@ __device__ __forceinline__ void invert_all(const SysDev& s, int sp, int lane, co
     return;
   }
   const LaneGroup lgp(lane, G);
-  const int ng = lgp.ng, g = lgp.g;
-  int* ex = scr + ng * n;
+  const int ng = lgp.ng, g = lgp.g, gl = lgp.gl;
+  double* A = scr + g * n * lda;
+  double* end = scr + ng * n * lda;
+  double* B = end;  // n > 16 only
+  if (n > 16) end += n * lda;
+  int* perm = reinterpret_cast<int*>(end) + g * n;
+  int* ex = reinterpret_cast<int*>(end) + ng * n;
   for (int u0 = 0; u0 < U; u0 += ng) {
     const int u = u0 + g;
     const bool act = u < U;
-    const int o = (act ? u : 0) * n * n;
-    const GroupDet d = group_inverse<Tb>(Phi + e0 * ld, ld, idx + (act ? u : 0) * n, n, G, act, scr + g * n,
-                                         Bd ? Bd + o : nullptr, Bf ? Bf + o : nullptr, Bg ? Bg + o : nullptr,
-                                         Lphi ? Lphi + e0 * ldL : nullptr, ldL);
-    if (act && lgp.gl == 0) {
-      ldet[u] = d.mant;
-      ex[u] = d.ex;
-      dsg[u] = (double)d.sgn;
-      if (tdet) tdet[u] = d.trace;
+    const int* iu = idx + (act ? u : 0) * n;
+    const double* P = Phi + e0 * ld;
+    const GroupDet d = n <= 8    ? group_lu8(P, ld, iu, n, G, act, A, perm)
+                       : n <= 16 ? group_lu16(P, ld, iu, n, G, act, A, perm)
+                                 : group_lu_smem(P, ld, iu, n, G, act, A, B, perm);
+    double t = 0.0;
+    if (tdet && act && gl < n) {
+      const int col = __ldg(iu + gl);
+      for (int e = 0; e < n; ++e) t = fma(A[gl * lda + e], widen(Lphi[(e0 + e) * ldL + col]), t);
+    }
+    if (tdet) t = group_sum(t, G);
+    if (act) {
+      // the group's lanes over the rows of the inverse, a row at a time
+      if (gl < n)
+        for (int o = 0; o < n; ++o) {
+          const double b = A[o * lda + gl];
+          const int q = (u * n + o) * n + gl;
+          if (Bd) Bd[q] = b;
+          if (Bf) Bf[q] = (float)b;
+          if (Bg) Bg[q] = b;
+        }
+      if (gl == 0) {
+        ldet[u] = d.mant;
+        ex[u] = d.ex;
+        dsg[u] = (double)d.sgn;
+        if (tdet) tdet[u] = t;
+      }
     }
     __syncwarp();
   }

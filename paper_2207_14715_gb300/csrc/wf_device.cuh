@@ -169,129 +169,288 @@ __device__ __forceinline__ bool less_nonneg(double a, double b) {
 }
 
 // ------------------------------------------------------------------------------------
-// Lane-group inverse of a Slater matrix, in registers.
-// A group of G lanes (G = power of two >= n, n <= 32) inverts one n x n matrix A (rows =
-// electrons, columns = orbital slots): lane o holds column o of A, that is row o of A^T, and A^T
-// is inverted in place by Gauss-Jordan elimination with partial pivoting over the lanes.  Step c
-// eliminates electron c: the pivot lane p is the one, among those not yet chosen, with the
-// largest |a_c|; its row is broadcast by shuffles and every lane subtracts its multiple.  The
-// registers move down by one per step (the finished column enters at the end), so that the loop
-// over c stays rolled with every register index a constant.  After n steps lane p(i), i its own
-// step, holds A^-1[p(j)][i] in register j.
+// Lane-group LU with partial pivoting and explicit inverse.
+// A group of G lanes (G = power of two >= n) inverts one n x n matrix A (rows = electrons, columns
+// = orbital slots); every lane of the warp calls this with the same n and G (inactive groups pass
+// active = false).  Phi [n][ld] holds the orbital values of the spin's electrons, idx [n] the column
+// of each slot.  Pivot ties go to the lowest row.  A: group scratch of n (n | 1) doubles, perm: n
+// ints.  det A = sgn * mant * 2^ex; a zero pivot gives sgn = 0, mant = 1 and a zero inverse.
 //
-// Bound: the FP64 pipe (64 cycles per warp instruction of an SM sub-partition, whatever its active
-// lanes): n + 4 instructions per step (a reciprocal, the multiplier, n - 1 updates).  The
-// factorisation in shared memory that this replaces issued about as many but waited for them: each
-// lane walked its own row serially, with the rows of a group 8 n bytes apart (16-way bank
-// conflicts at n = 8).
-//
-// Every lane of the warp calls this with the same n and G (inactive groups pass active = false).
-// Phi [n][ld] holds the orbital values of the spin's electrons, idx [n] the column of each slot (null:
-// column o).  Bd may be Phi itself (ld = n): the values are read first.
-// Outputs, row-major [slot][electron], each may be null: Bd, Bg in double, Bf in float.  perm: n
-// ints per group.  If Lphi is given, 'trace' returns tr(A^-1 L), L read at Lphi[e * ldL + idx[o]].
-// det A = sgn * mant * 2^ex; a zero pivot gives sgn = 0, mant = 1 and a zero inverse.
+// n <= NMAX: lane r keeps row r in registers through the elimination (the pivot row comes by
+// shuffles; the registers move down by one per column, so that the loop stays rolled with constant
+// register indices), writes its row of factors once, and as lane j solves for column j of the
+// inverse in registers, reading the factors by broadcast.  A then holds the inverse, row-major
+// [slot][electron] with rows of n | 1 doubles: lanes on consecutive rows read different banks
+// (rows of n = 8 doubles were 16-way conflicts, and every step waited for its stores).
+// Bound: the FP64 pipe (64 cycles per warp instruction whatever its active lanes).
 // ------------------------------------------------------------------------------------
 struct GroupDet {
-  double mant, trace;
+  double mant;
   int ex, sgn;
 };
 
+// mantissa product, exponent sum and sign from each lane's U diagonal d (1 outside the matrix)
+__device__ __forceinline__ GroupDet group_det(double d, bool in, int swaps, bool singular, int G) {
+  GroupDet r;
+  const long long bits = __double_as_longlong(d);
+  r.mant = in && !singular ? __longlong_as_double((bits & 0x000fffffffffffffll) | 0x3ff0000000000000ll) : 1.0;
+  r.ex = in && !singular ? (int)((bits >> 52) & 0x7ff) - 1023 : 0;
+  int neg = in && bits < 0 ? 1 : 0;
+  for (int o = G >> 1; o > 0; o >>= 1) {
+    r.mant *= __shfl_xor_sync(kFull, r.mant, o, G);
+    r.ex += __shfl_xor_sync(kFull, r.ex, o, G);
+    neg += __shfl_xor_sync(kFull, neg, o, G);
+  }
+  r.sgn = singular ? 0 : (((neg + swaps) & 1) ? -1 : 1);
+  return r;
+}
 
-template <int NMAX, class Tb>
-__device__ __forceinline__ GroupDet group_inverse_n(const double* Phi, int ld, const int* idx, int n, int G, bool active,
-                                                    int* perm, double* Bd, float* Bf, double* Bg, const Tb* Lphi,
-                                                    int ldL) {
-  const int lane = lane_id(), gl = lane & (G - 1), gbase = lane & ~(G - 1);
-  const bool mineact = active && gl < n;
+template <int NMAX>
+__device__ __forceinline__ GroupDet group_lu_n(const double* Phi, int ld, const int* idx, int n, int G, bool active,
+                                               double* A, int* perm) {
+  const int lane = lane_id(), gl = lane & (G - 1), gbase = lane & ~(G - 1), lda = n | 1;
+  const bool in = active && gl < n;
+  double a[NMAX];
+#pragma unroll
+  for (int o = 0; o < NMAX; ++o) a[o] = (in && o < n) ? Phi[gl * ld + __ldg(idx + o)] : 0.0;
+  int pos = gl, swaps = 0;  // this lane's row stands at position pos
+  bool singular = false;
+  for (int c = 0; c < n; ++c) {
+    // largest |a_c| over the rows at positions >= c (compared as integers: bit order is value order)
+    unsigned long long v = in && pos >= c ? (unsigned long long)__double_as_longlong(a[0]) & 0x7fffffffffffffffull : 0;
+    int at = in && pos >= c ? pos : 64, who = gl;
+    for (int o = G >> 1; o > 0; o >>= 1) {
+      const unsigned long long ov = __shfl_xor_sync(kFull, v, o, G);
+      const int oat = __shfl_xor_sync(kFull, at, o, G), ow = __shfl_xor_sync(kFull, who, o, G);
+      if (ov > v || (ov == v && oat < at)) { v = ov; at = oat; who = ow; }
+    }
+    if (v == 0) singular = true;
+    if (at != c) {
+      ++swaps;
+      if (in) {
+        if (pos == c) pos = at;
+        else if (gl == who) pos = c;
+      }
+    }
+    const int src = (gbase + who) & 31;
+    const double pv = __shfl_sync(kFull, a[0], src);
+    const double ip = singular ? 0.0 : recip_dd(pv);
+    const bool below = in && pos > c && !singular;
+    const double l = a[0] * ip;
+#pragma unroll
+    for (int j = 1; j < NMAX; ++j) {
+      if (j < n - c) {
+        const double u = __shfl_sync(kFull, a[j], src);
+        const double x = fma(-l, u, a[j]);
+        a[j] = below ? x : a[j];
+      }
+    }
+    const double head = below ? l : a[0];  // the factor, or U's own entry
+#pragma unroll
+    for (int j = 1; j < NMAX; ++j) {
+      if (j < n) a[j - 1] = a[j];
+      else if (j == n) a[j - 1] = head;
+    }
+    if (n == NMAX) a[NMAX - 1] = head;
+  }
+  if (in) {
+    perm[pos] = gl;
+#pragma unroll
+    for (int j = 0; j < NMAX; ++j)
+      if (j < n) A[pos * lda + j] = a[j];
+  }
+  __syncwarp();
+  // lane i holds 1 / U_ii; the solves multiply by it (broadcast by shuffle)
+  const double diag = in ? A[gl * lda + gl] : 1.0;
+  const double dinv = in && !singular ? recip_dd(diag) : 0.0;
+  // column gl of the inverse: L y = P e, U x = y
+#pragma unroll
+  for (int i = 0; i < NMAX; ++i)
+    if (i < n) {
+      double y = (in && perm[i] == gl) ? 1.0 : 0.0;
+#pragma unroll
+      for (int k = 0; k < NMAX; ++k)
+        if (k < i) y = fma(-A[i * lda + k], a[k], y);
+      a[i] = y;
+    }
+#pragma unroll
+  for (int i = NMAX - 1; i >= 0; --i)
+    if (i < n) {
+      const double di = __shfl_sync(kFull, dinv, (gbase + i) & 31);
+      double x = a[i];
+#pragma unroll
+      for (int k = 0; k < NMAX; ++k)
+        if (k > i && k < n) x = fma(-A[i * lda + k], a[k], x);
+      a[i] = x * di;
+    }
+  __syncwarp();
+  if (in)
+#pragma unroll
+    for (int i = 0; i < NMAX; ++i)
+      if (i < n) A[i * lda + gl] = singular ? 0.0 : a[i];
+  __syncwarp();
+  return group_det(diag, in, swaps, singular, G);
+}
+
+// the same with the matrix in shared memory (16 < n <= 32: one group); B: n (n | 1) doubles more
+static __device__ __noinline__ GroupDet group_lu_smem(const double* Phi, int ld, const int* idx, int n, int G, bool active,
+                                                      double* A, double* B, int* perm) {
+  const int lane = lane_id(), gl = lane & (G - 1), gbase = lane & ~(G - 1), lda = n | 1;
+  const bool in = active && gl < n;
+  if (in) {
+    perm[gl] = gl;
+    const int col = __ldg(idx + gl);
+    for (int e = 0; e < n; ++e) A[e * lda + gl] = Phi[e * ld + col];
+  }
+  __syncwarp();
+  int swaps = 0;
+  bool singular = false;
+  for (int c = 0; c < n; ++c) {
+    unsigned long long v = in && gl >= c ? (unsigned long long)__double_as_longlong(A[gl * lda + c]) & 0x7fffffffffffffffull : 0;
+    int at = in && gl >= c ? gl : 64;
+    for (int o = G >> 1; o > 0; o >>= 1) {
+      const unsigned long long ov = __shfl_xor_sync(kFull, v, o, G);
+      const int oat = __shfl_xor_sync(kFull, at, o, G);
+      if (ov > v || (ov == v && oat < at)) { v = ov; at = oat; }
+    }
+    if (v == 0) singular = true;
+    if (at != c && !singular) {
+      ++swaps;
+      if (in) {
+        const double t = A[c * lda + gl];
+        A[c * lda + gl] = A[at * lda + gl];
+        A[at * lda + gl] = t;
+        if (gl == 0) {
+          const int q = perm[c];
+          perm[c] = perm[at];
+          perm[at] = q;
+        }
+      }
+    }
+    __syncwarp();
+    double ip = 0.0;
+    if (in && !singular && gl == c) ip = recip_dd(A[c * lda + c]);
+    ip = __shfl_sync(kFull, ip, (gbase + c) & 31);
+    if (in && !singular && gl > c) {
+      const double l = A[gl * lda + c] * ip;
+      A[gl * lda + c] = l;
+#pragma unroll 4
+      for (int j = c + 1; j < n; ++j) A[gl * lda + j] = fma(-l, A[c * lda + j], A[gl * lda + j]);
+    }
+    __syncwarp();
+  }
+  const double diag = in ? A[gl * lda + gl] : 1.0;
+  const double dinv = in && !singular ? recip_dd(diag) : 0.0;
+  for (int i = 0; i < n; ++i) {
+    double y = in && perm[i] == gl ? 1.0 : 0.0;
+    if (in)
+      for (int k = 0; k < i; ++k) y = fma(-A[i * lda + k], B[k * lda + gl], y);
+    if (in) B[i * lda + gl] = y;
+  }
+  for (int i = n - 1; i >= 0; --i) {
+    const double di = __shfl_sync(kFull, dinv, (gbase + i) & 31);
+    if (in) {
+      double x = B[i * lda + gl];
+      for (int k = i + 1; k < n; ++k) x = fma(-A[i * lda + k], B[k * lda + gl], x);
+      B[i * lda + gl] = x * di;
+    }
+  }
+  __syncwarp();
+  if (in)
+    for (int i = 0; i < n; ++i) A[i * lda + gl] = singular ? 0.0 : B[i * lda + gl];
+  __syncwarp();
+  return group_det(diag, in, swaps, singular, G);
+}
+
+// not inlined: the callers are large and this is a small part of their work
+static __device__ __noinline__ GroupDet group_lu8(const double* Phi, int ld, const int* idx, int n, int G, bool active,
+                                                  double* A, int* perm) {
+  return group_lu_n<8>(Phi, ld, idx, n, G, active, A, perm);
+}
+static __device__ __noinline__ GroupDet group_lu16(const double* Phi, int ld, const int* idx, int n, int G, bool active,
+                                                   double* A, int* perm) {
+  return group_lu_n<16>(Phi, ld, idx, n, G, active, A, perm);
+}
+
+// ------------------------------------------------------------------------------------
+// Inverse of one Slater matrix by the whole warp, in registers (the reference of the tables).
+// Lane o < n <= 32 holds column o of A, that is row o of A^T, and A^T is inverted in place by
+// Gauss-Jordan elimination with partial pivoting over the lanes.  Step c eliminates electron c: the
+// pivot lane p is the one, among those not yet chosen, with the largest |a_c|; its row is broadcast
+// by shuffles and every lane subtracts its multiple.  The registers move down by one per step (the
+// finished column enters at the end), so that the loop over c stays rolled with every register
+// index a constant.  After n steps lane p(i), i its own step, holds A^-1[p(j)][i] in register j.
+//
+// Bound: the FP64 pipe: n + 4 instructions per step (a reciprocal, the multiplier, n - 1 updates).
+// The factorisation in shared memory issued half as many again for the factors and the solves of
+// n = 24 and waited for its stores.
+//
+// Phi [n][ld] holds the orbital values of the spin's electrons, idx [n] the column of each slot (null:
+// column o).  Bd [slot][electron] receives the inverse and may be Phi itself (ld = n): the values are
+// read first.  perm: n ints.  det A = sgn * mant * 2^ex; a zero pivot gives sgn = 0, mant = 1
+// and a zero inverse.
+// ------------------------------------------------------------------------------------
+template <int NMAX>
+__device__ __forceinline__ GroupDet warp_inverse_n(const double* Phi, int ld, const int* idx, int n, int* perm,
+                                                   double* Bd) {
+  const int lane = lane_id();
+  const bool in = lane < n;
   double a[NMAX];
   {
-    const int col = mineact ? (idx ? __ldg(idx + gl) : gl) : 0;
+    const int col = in ? (idx ? __ldg(idx + lane) : lane) : 0;
 #pragma unroll
-    for (int e = 0; e < NMAX; ++e) a[e] = (mineact && e < n) ? Phi[e * ld + col] : 0.0;
+    for (int e = 0; e < NMAX; ++e) a[e] = (in && e < n) ? Phi[e * ld + col] : 0.0;
   }
-  bool used = !mineact, singular = false;
+  bool used = !in, singular = false;
   unsigned chosen = 0;
   int par = 0, mine = 0;
   double piv = 1.0;
   for (int c = 0; c < n; ++c) {
     // the largest |a_0| over the lanes not yet chosen, to 15 bits of its mantissa (enough for
     // stability); ties go to the lowest lane
-    unsigned key = used ? 0u : (0x80000000u | ((unsigned)__double2hiint(a[0]) & 0x7fffffe0u) | (31u - (unsigned)gl));
-    for (int o = G >> 1; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(kFull, key, o, G));
+    unsigned key = used ? 0u : (0x80000000u | ((unsigned)__double2hiint(a[0]) & 0x7fffffe0u) | (31u - (unsigned)lane));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(kFull, key, o));
     const int p = 31 - (int)(key & 31u);
-    const int src = gbase + p;
-    const double pv = __shfl_sync(kFull, a[0], src & 31);
-    const bool zero = (__double_as_longlong(pv) << 1) == 0;
+    const double pv = __shfl_sync(kFull, a[0], p);
+    const bool zero = !nonzero(pv);
     singular |= zero;
     const double ip = zero ? 0.0 : recip_dd(pv);
-    const bool isp = gl == p;
+    const bool isp = lane == p;
     const double t = isp ? -ip : a[0] * ip;
 #pragma unroll
     for (int j = 1; j < NMAX; ++j) {
       if (j < n) {
-        const double aj = __shfl_sync(kFull, a[j], src & 31);
+        const double aj = __shfl_sync(kFull, a[j], p);
         a[j - 1] = fma(-t, aj, isp ? 0.0 : a[j]);
       } else if (j == n) {
         a[j - 1] = -t;
       }
     }
     if (n == NMAX) a[NMAX - 1] = -t;
-    if (isp && !used) {
+    if (isp) {
       mine = c;
       used = true;
       piv = pv;
     }
     par ^= __popc((chosen >> p) >> 1) & 1;
     chosen |= 1u << p;
-    if (active && gl == 0) perm[c] = p;
+    if (lane == 0) perm[c] = p;
   }
   __syncwarp();
-  GroupDet r;
-  // ln|det| later from the product of the pivots' mantissas (each in [1, 2): no overflow for
-  // n <= 32) and the sum of their exponents
-  const long long bits = __double_as_longlong(piv);
-  r.mant = __longlong_as_double((bits & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
-  r.ex = mineact ? (int)((bits >> 52) & 0x7ff) - 1023 : 0;
-  unsigned neg = bits < 0 ? 1u : 0u;
-  double tr = 0.0;
-  if (mineact) {
+  if (in) {
 #pragma unroll
     for (int j = 0; j < NMAX; ++j)
-      if (j < n) {
-        const int o = perm[j];
-        const double b = singular ? 0.0 : a[j];
-        const int q = o * n + mine;
-        if (Bd) Bd[q] = b;
-        if (Bf) Bf[q] = (float)b;
-        if (Bg) Bg[q] = b;
-        if (Lphi) tr = fma(b, widen(Lphi[mine * ldL + (idx ? __ldg(idx + o) : o)]), tr);
-      }
-  }
-  for (int o = G >> 1; o > 0; o >>= 1) {
-    r.mant *= __shfl_xor_sync(kFull, r.mant, o, G);
-    r.ex += __shfl_xor_sync(kFull, r.ex, o, G);
-    neg ^= __shfl_xor_sync(kFull, neg, o, G);
-  }
-  r.trace = Lphi ? group_sum(tr, G) : 0.0;
-  r.sgn = ((neg ^ (unsigned)par) & 1u) ? -1 : 1;
-  if (singular) {
-    r.mant = 1.0;
-    r.ex = 0;
-    r.sgn = 0;
+      if (j < n) Bd[perm[j] * n + mine] = singular ? 0.0 : a[j];
   }
   __syncwarp();
-  return r;
+  return group_det(piv, in, par, singular, 32);
 }
-
-// The three register sizes behind one call (not inlined: the callers are large and this is a
-// small part of their work).
-template <class Tb>
-__device__ __noinline__ GroupDet group_inverse(const double* Phi, int ld, const int* idx, int n, int G, bool active,
-                                               int* perm, double* Bd, float* Bf, double* Bg, const Tb* Lphi, int ldL) {
-  if (n <= 8) return group_inverse_n<8, Tb>(Phi, ld, idx, n, G, active, perm, Bd, Bf, Bg, Lphi, ldL);
-  if (n <= 16) return group_inverse_n<16, Tb>(Phi, ld, idx, n, G, active, perm, Bd, Bf, Bg, Lphi, ldL);
-  return group_inverse_n<32, Tb>(Phi, ld, idx, n, G, active, perm, Bd, Bf, Bg, Lphi, ldL);
+static __device__ __noinline__ GroupDet warp_inverse(const double* Phi, int ld, const int* idx, int n, int* perm,
+                                                     double* Bd) {
+  if (n <= 8) return warp_inverse_n<8>(Phi, ld, idx, n, perm, Bd);
+  if (n <= 16) return warp_inverse_n<16>(Phi, ld, idx, n, perm, Bd);
+  return warp_inverse_n<32>(Phi, ld, idx, n, perm, Bd);
 }
 
 // ln|det| of u = 0..U-1 from the mantissa products (in ldet), exponents and signs: one logarithm
