@@ -285,6 +285,7 @@ int vbqmc_set_system(vbqmc_ctx* ctx, int sys_id, const vbqmc_system_desc* desc) 
   d.een_cf = (const float*)(B + o_een_cf);
   d.een_B = (const double*)(B + o_een_B);
   d.kap_x = (const int*)(B + o_kx);
+  d.same_occ = h.occ_list[0] == h.occ_list[1] ? 1 : 0;
   for (int sp = 0; sp < 2; ++sp) d.n_occ_chunk[sp] = (int)(h.occ_chunk[sp].size() / 4);
   d.n_evq_chunk = (int)(h.evq_chunk.size() / 4);
   d.evq_width = h.evq_width;

@@ -50,10 +50,10 @@ __global__ void __launch_bounds__(MAXT, 1) batch_fused_kernel(const BatchSys* __
       for (int r = wl; r < item.count; r += cs) {
         const int w = item.first + r;
         if (b.dev.msd)
-          sweep_body<Tb, true>(b.dev, b.sweep, w, smem + wl * b.sweep.warp_bytes, b.R, call->nsweeps, call->refresh,
+          sweep_body<Tb, true, true>(b.dev, b.sweep, w, smem + wl * b.sweep.warp_bytes, b.R, call->nsweeps, call->refresh,
                                nullptr, 0, call->step, call->seed, call->step0, b.tag, 0u, b.nacc);
         else
-          sweep_body<Tb, false>(b.dev, b.sweep, w, smem + wl * b.sweep.warp_bytes, b.R, call->nsweeps,
+          sweep_body<Tb, false, true>(b.dev, b.sweep, w, smem + wl * b.sweep.warp_bytes, b.R, call->nsweeps,
                                 call->refresh, b.state, call->state_valid, call->step, call->seed, call->step0, b.tag,
                                 0u, b.nacc);
       }

@@ -17,7 +17,7 @@ __global__ void __launch_bounds__(512, 1) sweep_kernel(const SysDev s, const Swe
   const int wl = threadIdx.x >> 5;
   const int w = blockIdx.x * L.wpb + wl;
   if (w >= W) return;
-  sweep_body<Tb, TAB>(s, L, w, smem + wl * L.warp_bytes, Rg, nsweeps, refresh, state, state_valid, step, seed, step0,
+  sweep_body<Tb, TAB, false>(s, L, w, smem + wl * L.warp_bytes, Rg, nsweeps, refresh, state, state_valid, step, seed, step0,
                       tag, woff, nacc);
 }
 
@@ -34,9 +34,9 @@ __global__ void __launch_bounds__(512, 1) sweep_batch_kernel(const BatchSys* __r
     const BatchItem item = items[it];
     if (wl >= item.count) continue;
     const BatchSys& b = sys[item.sys];
-    sweep_body<Tb, false>(b.dev, b.sweep, item.first + wl, smem + wl * b.sweep.warp_bytes, b.R, call->nsweeps,
-                          call->refresh,
-                   b.state, call->state_valid, call->step, call->seed, call->step0, b.tag, 0u, b.nacc);
+    sweep_body<Tb, false, true>(b.dev, b.sweep, item.first + wl, smem + wl * b.sweep.warp_bytes, b.R, call->nsweeps,
+                                call->refresh, b.state, call->state_valid, call->step, call->seed, call->step0, b.tag,
+                                0u, b.nacc);
   }
 }
 
@@ -71,8 +71,7 @@ int make_sweep_layout(const SysDev& s, int tb, int max_smem, SweepLayout& L) {
   L.RG0 = ratio_group(s.n[0], s.U[0], L.G0);
   L.RG1 = ratio_group(s.n[1], s.U[1], L.G1);
   L.nocc_max = std::max(std::max(s.nocc[0], s.nocc[1]), 1);
-  L.R = take(8 * 3 * N);
-  L.Rds = take(tb == 4 ? 8 * 3 * N : 16);
+  L.R = take(8 * 3 * N);  // double, or float pairs
   if (L.tab) {  // reference inverse and tables per spin, q_u of both spins, proposed q_u, c_x
     L.Binv0 = take(8 * s.n[0] * s.n[0]);
     L.Binv1 = take(8 * s.n[1] * s.n[1]);
@@ -90,42 +89,70 @@ int make_sweep_layout(const SysDev& s, int tb, int max_smem, SweepLayout& L) {
     L.Binv1 = take(8 * s.U[1] * s.n[1] * s.n[1]);
     L.wk = take(8 * s.nterm);
   }
-  // a refactorisation's ln|det|, signs and orbital matrix overlay the sweep's proposals and
-  // the move-only geometry (the refactorisation runs before the proposals are formed, and its
-  // outputs are consumed by the term ratios before the moves start)
-  const int over0 = off;
-  L.rtab = take(8 * 4 * N);
-  L.rtds = take(tb == 4 ? 8 * 3 * N : 16);
-  L.geom = take(tb * (2 * N + s.Nn + 6 * s.Nn + 10 * (N + 1)));
-  const int moves_end = off;
-  off = over0;
-  if (L.tab) {  // the X values of one spin; the reference's values are formed where its inverse goes
-    L.ldet = L.dsg = off;
-    L.PhiO = take(8 * std::max(std::max(s.n[0] * s.n_x[0], s.n[1] * s.n_x[1]), 1));
-  } else {
-    L.ldet = take(8 * Ut);
-    L.dsg = take(8 * Ut);
-    L.PhiO = take(8 * N * L.nocc_max);
-  }
-  off = std::max(off, moves_end);
+  L.vrow = take(8 * L.nocc_max);
+  L.ke = tb == 8 ? 1 : (4 * s.Nn <= 32 ? 4 : (2 * s.Nn <= 32 ? 2 : 1));
+  const int nmax = std::max(s.n[0], s.n[1]), nch = std::max(std::max(s.n_occ_chunk[0], s.n_occ_chunk[1]), 1);
   int cv = 0, scr = 0;
   for (int sp = 0; sp < 2; ++sp) {
     const int n = s.n[sp], G = sp ? L.G1 : L.G0, ng = L.tab ? 1 : 32 / G;
     cv = std::max(cv, 8 * (L.tab ? 1 : 2) * ng * n);  // Sherman-Morrison stages two passes' columns
     scr = std::max(scr, L.tab ? 4 * n + 16 : inverse_scratch_bytes(n, s.U[sp], G));
   }
-  // the LU scratch of a refactorisation shares its space with the buffers of the moves (the
-  // basis values and partial sums that build PhiO are consumed before the LU starts)
-  const int shared0 = off;
-  L.bas = take(8 * s.M);
-  L.vrow = take(8 * L.nocc_max);
-  L.part = take(8 * std::max(std::max(s.n_occ_chunk[0], s.n_occ_chunk[1]), 1));
-  L.rho = take(8 * std::max(s.U[0], s.U[1]));
-  L.rinv = take(8 * (std::max(s.U[0], s.U[1]) + 1));
-  L.cvec = take(std::max(cv, 8));
-  L.scratch = shared0;
-  off = std::max(off, align16(shared0 + std::max(scr, 16)));
-  L.geo = take(tb * (N * s.Nn + (N + 1) * s.Nn));
+  // What the moves keep (tables of the current positions, proposals) shares its place with a
+  // refactorisation's ln|det|, signs and orbital matrix, consumed by the term ratios before the tables
+  // are formed.  Then come the basis values and partial sums of either, over them the buffers of a
+  // move, and over all of these the scratch of the inverses (past the orbital matrix).
+  const int over0 = off;
+  auto place = [&](bool all, bool tri, bool rows) {  // end of the walker's region
+    off = over0;
+    const int np = all ? N : nmax;
+    L.all = all ? 1 : 0;
+    L.rows = rows ? 1 : 0;
+    L.tri = tri ? 1 : 0;
+    L.rtab = take(8 * 3 * np);
+    L.rtds = take(tb == 4 ? 8 * 3 * np : 16);
+    L.svn = take(tb * np * s.Nn);
+    L.den = take(tb * np * s.Nn);
+    L.vrows = take(tb * (rows ? N : nmax) * L.nocc_max);
+    L.Sv = take(tb * (N + 1) * s.Nn);
+    L.ut = take(tri ? tb * (N * (N - 1) / 2 + 1) : 0);
+    L.ft = take(tri ? tb * (N * (N - 1) / 2 + 1) : 0);
+    const int moves_end = off;
+    off = over0;
+    if (L.tab) {  // the X values of one spin; the reference's values are formed where its inverse goes
+      L.ldet = L.dsg = off;
+      L.PhiO = take(8 * std::max(std::max(s.n[0] * s.n_x[0], s.n[1] * s.n_x[1]), 1));
+    } else {
+      L.ldet = take(8 * Ut);
+      L.dsg = take(8 * Ut);
+      L.PhiO = take(8 * N * L.nocc_max);
+    }
+    L.scratch = off;
+    const int scr_end = align16(off + std::max(scr, 16));
+    const int shared0 = off = std::max(off, moves_end);
+    L.bas = take(std::max(8 * s.M, tb * L.ke * s.M));
+    L.alias = nch <= 32 ? 1 : 0;
+    const int part_bytes = std::max(8 * nch, tb * L.ke * nch);
+    L.part = L.alias ? L.bas : take(part_bytes);
+    if (L.alias) off = std::max(off, align16(L.bas + part_bytes));
+    const int basis_end = off;
+    off = shared0;
+    L.up = take(2 * tb * 4 * (N + 1));
+    L.ue = take(tb * N);
+    L.fe = take(tb * N);
+    L.rho = take(8 * std::max(s.U[0], s.U[1]));
+    L.rinv = take(8 * (std::max(s.U[0], s.U[1]) + 1));
+    L.cvec = take(std::max(cv, 8));
+    return off = std::max(std::max(off, basis_end), scr_end);
+  };
+  // the pair tables, and both spins prepared at once (one electron per lane), where as many
+  // walkers share a block with them
+  auto fit = [&](int bytes) { return std::min(16, max_smem / std::max(bytes, 1)); };
+  const int most = fit(place(false, false, false));
+  const bool tri = fit(place(false, true, false)) == most;
+  const bool all = N <= 32 && fit(place(true, tri, false)) == most;
+  const bool rows = all && s.same_occ && fit(place(true, tri, true)) == most;
+  place(all, tri, rows);
   L.warp_bytes = off;
   int wpb = max_smem / off;
   if (wpb > 16) wpb = 16;

@@ -59,7 +59,13 @@ struct EvalLayout {
 // gw the weights g_u of the moving spin, wrow the row v^T B - e_i of an accepted move.
 struct SweepLayout {
   int wpb = 0, warp_bytes = 0;
-  int R, Rds, rtab, rtds, Binv0, Binv1, ldet, dsg, wk, PhiO, bas, vrow, part, rho, rinv, cvec, scratch, geo, geom;
+  int R, rtab, rtds, vrows, svn, den, Binv0, Binv1, ldet, dsg, wk, PhiO, bas, vrow, part, rho, rinv, cvec, scratch;
+  int up, ue, fe, Sv, ut = 0, ft = 0;
+  int ke;         // electrons whose proposal rows are formed together (float form: 4, 2 or 1)
+  int alias;      // the contraction's partial sums (one round) overlay the basis values
+  int all = 0;    // proposals and e-n changes of both spins prepared at once
+  int rows = 0;   // their orbital rows too (the spins use the same orbitals)
+  int tri = 0;    // Rbar and e-e value kept per electron pair (where that costs no walker per block)
   int T0 = 0, T1 = 0, qn = 0, cx = 0, Tn = 0, gw = 0, wrow = 0;
   int tab = 0;
   int nocc_max;

@@ -36,14 +36,174 @@ namespace vbq {
 // the walker state written by the evaluation at the same positions, or from a fresh LU of
 // double-precision orbital values (first sweep without state, and every 'refresh' sweeps).
 // The proposed orbital row uses the bulk type; ratios and Sherman-Morrison updates are double.
+//
+// What a move needs of its own electron alone is prepared for all electrons of a spin before their
+// moves (an electron's proposal depends on its own position only, and it moves once per sweep):
+// the proposals' orbital rows, for L.ke electrons at a time so that a coefficient and its index serve
+// them all and every round of 32 (shell, electron) items is full, and the nuclei's Rbar and e-n
+// changes over all (electron, nucleus) pairs.  A move is then left with the other electrons: the
+// distances from the proposal, against Rbar and the e-e value of the current pairs, which are kept
+// per pair (L.tri) and replaced when a move is accepted.  The float values and sums are those of a
+// move that forms everything by itself, bit for bit.  Bound by instruction issue (float) and the
+// FP64 pipe (double); a sweep of the ethylene-shaped system went from 1298 to 1080 us (16384 walkers,
+// mixed), 2303 to 2095 us (3001, double), one of the 48-electron system from 11.5 to 10.0 ms (8192).
 // One warp, walker w, shared-memory region 'base' of L.warp_bytes bytes.
-template <class Tb, bool TAB>
+
+// f of the Pade + polynomial form at R = r den, den = 1 / (1 + kappa r) (as pade_poly)
+template <class Tb> __device__ __forceinline__ Tb pade_value(const PadeT<Tb>& c, Tb r, Tb den) {
+  const Tb R = r * den;
+  const Tb pd = (Tb)1 / ((Tb)1 + c.a2 * R);
+  const Tb R2 = R * R, R3 = R2 * R, R4 = R3 * R, R5 = R4 * R;
+  return c.a1 * R * pd + c.q[0] * R2 + c.q[1] * R3 + c.q[2] * R4 + c.q[3] * R5;
+}
+
+// (x, y) pairs: the old and new side of a move's e-e-n sums.  In float each operation is one packed
+// instruction on both (independent, correctly rounded: the same values as two scalar ones).
+template <class Tb> struct Pair2 { Tb o, n; };
+__device__ __forceinline__ Pair2<double> pair_fma(Pair2<double> a, Pair2<double> b, Pair2<double> c) {
+  return {fma(a.o, b.o, c.o), fma(a.n, b.n, c.n)};
+}
+__device__ __forceinline__ Pair2<double> pair_mul(Pair2<double> a, Pair2<double> b) { return {a.o * b.o, a.n * b.n}; }
+__device__ __forceinline__ Pair2<double> pair_add(Pair2<double> a, Pair2<double> b) { return {a.o + b.o, a.n + b.n}; }
+__device__ __forceinline__ Pair2<float> pair_fma(Pair2<float> a, Pair2<float> b, Pair2<float> c) {
+  Pair2<float> d;
+  asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+      "fma.rn.f32x2 a, a, b, c;\n\tmov.b64 {%0, %1}, a;\n\t}"
+      : "=f"(d.o), "=f"(d.n)
+      : "f"(a.o), "f"(a.n), "f"(b.o), "f"(b.n), "f"(c.o), "f"(c.n));
+  return d;
+}
+__device__ __forceinline__ Pair2<float> pair_mul(Pair2<float> a, Pair2<float> b) {
+  Pair2<float> d;
+  asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "mul.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
+      : "=f"(d.o), "=f"(d.n)
+      : "f"(a.o), "f"(a.n), "f"(b.o), "f"(b.n));
+  return d;
+}
+__device__ __forceinline__ Pair2<float> pair_add(Pair2<float> a, Pair2<float> b) {
+  Pair2<float> d;
+  asm("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "add.rn.f32x2 a, a, b;\n\tmov.b64 {%0, %1}, a;\n\t}"
+      : "=f"(d.o), "=f"(d.n)
+      : "f"(a.o), "f"(a.n), "f"(b.o), "f"(b.n));
+  return d;
+}
+
+// r^2 of a proposal's basis functions: the products rounded one by one, or (FUSED) fused.  The
+// single-system and the batch kernels each keep to one form whatever the compiler would contract,
+// so that their trajectories stay the ones of earlier builds.
+template <bool FUSED> __device__ __forceinline__ float norm2(float x, float y, float z) {
+  if constexpr (FUSED) return fmaf(z, z, fmaf(x, x, __fmul_rn(y, y)));
+  return __fadd_rn(__fadd_rn(__fmul_rn(x, x), __fmul_rn(y, y)), __fmul_rn(z, z));
+}
+
+// Values of a shell (as gto_shell_emit with r^2 given): emit(c, chi_c)
+template <class Emit>
+__device__ __forceinline__ void shell_values(int l, float z, const float* nrm, float r2, float dx, float dy, float dz,
+                                             Emit&& emit) {
+  const float e = z < 0.0f ? vexp(z * vsqrt(r2)) : (z == 0.0f ? 1.0f : vexp(-z * r2));
+  if (l == 0) {
+    emit(0, __ldg(nrm) * e);
+  } else if (l == 1) {
+    const float d[3] = {dx, dy, dz};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) emit(c, __ldg(nrm + c) * e * d[c]);
+  } else {
+    constexpr int ia[6] = {0, 1, 2, 0, 0, 1}, ib[6] = {0, 1, 2, 1, 2, 2};  // xx yy zz xy xz yz
+    const float d[3] = {dx, dy, dz};
+#pragma unroll
+    for (int c = 0; c < 6; ++c) emit(c, __ldg(nrm + c) * e * (d[ia[c]] * d[ib[c]]));
+  }
+}
+
+// Rows of the proposals of cnt <= KE electrons (float form): rnd [cnt][3] their positions, out [cnt][ldo].
+template <int KE, bool FUSED>
+__device__ __forceinline__ void proposal_rows(const SysDev& s, int lane, int sp, int cnt, const dsf* rnd, float* bas,
+                                              float* part, bool alias, float* out, int ldo) {
+  constexpr int kLog = KE == 4 ? 2 : (KE == 2 ? 1 : 0);
+  const int Nn = s.Nn;
+  // the displacements, lane el Nn + a, shared by shuffles with the lanes of that nucleus's shells
+  // (too many nuclei: each item forms its own)
+  const bool shuf = KE * Nn <= 32;
+  float cx = 0.0f, cy = 0.0f, cz = 0.0f;
+  if (shuf && lane < cnt * Nn) {
+    const DivStep ea(lane, Nn);
+    cx = ds_diff_f(rnd[3 * ea.hi], nuc_coord_ds(s, ea.lo, 0));
+    cy = ds_diff_f(rnd[3 * ea.hi + 1], nuc_coord_ds(s, ea.lo, 1));
+    cz = ds_diff_f(rnd[3 * ea.hi + 2], nuc_coord_ds(s, ea.lo, 2));
+  }
+  for (int i0 = 0; i0 < KE * s.S; i0 += 32) {  // every lane takes part in each round (the shuffles)
+    const int i = i0 + lane, t = i >> kLog, el = i & (KE - 1);
+    const bool act = t < s.S && el < cnt;
+    // one 16-byte record per shell, in the order of l
+    const int4 p = act ? __ldg(reinterpret_cast<const int4*>(s.sh_pack_f) + t) : make_int4(0, 0, 0, 0);
+    const int c = p.x & 0xffff, l = p.x >> 16, f = p.y, sh = p.z;
+    float dx, dy, dz;
+    if (shuf) {
+      const int src = el * Nn + c;
+      dx = __shfl_sync(kFull, cx, src);
+      dy = __shfl_sync(kFull, cy, src);
+      dz = __shfl_sync(kFull, cz, src);
+    } else if (act) {
+      dx = ds_diff_f(rnd[3 * el], nuc_coord_ds(s, c, 0));
+      dy = ds_diff_f(rnd[3 * el + 1], nuc_coord_ds(s, c, 1));
+      dz = ds_diff_f(rnd[3 * el + 2], nuc_coord_ds(s, c, 2));
+    }
+    if (act)
+      shell_values(l, __int_as_float(p.w), s.sh_norm_f + 6 * sh, norm2<FUSED>(dx, dy, dz), dx, dy, dz,
+                   [&](int k, float v) { bas[KE * (f + k) + el] = v; });
+  }
+  __syncwarp();
+  // contraction in balanced chunks: one coefficient serves the KE electrons
+  for (int c0 = 0; c0 < s.n_occ_chunk[sp]; c0 += 32) {
+    const int c = c0 + lane;
+    float v[KE];
+#pragma unroll
+    for (int k = 0; k < KE; ++k) v[k] = 0.0f;
+    if (c < s.n_occ_chunk[sp]) {
+      const int4 ch = __ldg(reinterpret_cast<const int4*>(s.occ_chunk[sp]) + c);
+      const float* cb = s.orb_coef_f + ch.w;
+#pragma unroll 4
+      for (int mu = ch.y; mu < ch.z; ++mu) {
+        const float cm = __ldg(cb + mu);
+        float b[KE];
+        if constexpr (KE == 4) {
+          const float4 q = reinterpret_cast<const float4*>(bas)[mu];
+          b[0] = q.x; b[1] = q.y; b[2] = q.z; b[3] = q.w;
+        } else if constexpr (KE == 2) {
+          const float2 q = reinterpret_cast<const float2*>(bas)[mu];
+          b[0] = q.x; b[1] = q.y;
+        } else {
+          b[0] = bas[mu];
+        }
+#pragma unroll
+        for (int k = 0; k < KE; ++k) v[k] += cm * b[k];
+      }
+    }
+    if (alias) __syncwarp();  // one round: the partial sums take the place of the basis values
+    if (c < s.n_occ_chunk[sp])
+#pragma unroll
+      for (int k = 0; k < KE; ++k) part[KE * c + k] = v[k];
+  }
+  __syncwarp();
+  const int nocc = s.nocc[sp];
+  for (int i = lane; i < KE * nocc; i += 32) {
+    const int q = i >> kLog, el = i & (KE - 1);
+    const int c0 = __ldg(s.occ_chunk_off[sp] + q), c1 = __ldg(s.occ_chunk_off[sp] + q + 1);
+    float v = 0.0f;
+    for (int c = c0; c < c1; ++c) v += part[KE * c + el];
+    if (el < cnt) out[el * ldo + q] = v;
+  }
+  __syncwarp();
+}
+
+template <class Tb, bool TAB, bool BATCH>
 __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L, int w, unsigned char* base,
                                            double* __restrict__ Rg, int nsweeps, int refresh,
                                            double* __restrict__ state, int state_valid, double step, uint64_t seed,
                                            uint32_t step0, uint32_t tag, uint32_t woff, int* __restrict__ nacc) {
   const int lane = threadIdx.x & 31;
-  double* R = reinterpret_cast<double*>(base + L.R);
   double* Binv[2] = {reinterpret_cast<double*>(base + L.Binv0), reinterpret_cast<double*>(base + L.Binv1)};
   double* ldet = reinterpret_cast<double*>(base + L.ldet);
   double* dsg = reinterpret_cast<double*>(base + L.dsg);
@@ -58,41 +218,54 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
   double* rinv = reinterpret_cast<double*>(base + L.rinv);
   double* cvec = reinterpret_cast<double*>(base + L.cvec);
   double* scr = reinterpret_cast<double*>(base + L.scratch);
-  // the pair distances r_ij are formed where a move needs them (the distances of the moving
-  // electron, from the same coordinate differences the tables would hold)
-  Tb* rEN = reinterpret_cast<Tb*>(base + L.geo);       // [N][Nn] r_ia
-  // row strides padded by one so that lanes on different nuclei (powers) read different banks
+  // of the prepared electrons (L.all: every electron; else the moving spin's): proposed positions
+  // (and their float-float copies), Rbar and e-n change per nucleus; orbital rows of the moving spin's
+  double* rtab = reinterpret_cast<double*>(base + L.rtab);  // [][3]
+  dsf* rtds = reinterpret_cast<dsf*>(base + L.rtds);        // [][3]
+  Tb* svn = reinterpret_cast<Tb*>(base + L.svn);            // [][Nn]
+  Tb* den = reinterpret_cast<Tb*>(base + L.den);            // [][Nn]
+  Tb* vrows = reinterpret_cast<Tb*>(base + L.vrows);        // [n or (L.rows) N][nocc]
+  // current positions: [Nn][SA] Rbar(r_ja) (its powers formed where used; the row stride padded so that
+  // lanes on different nuclei read different banks), and per pair Rbar(r_ij) and the e-e value
   const int SA = s.N + 1, UP = s.N + 1;
-  Tb* Sv = rEN + s.N * s.Nn;                            // [Nn][SA]: Rbar(r_ja) at a*SA + j (its powers formed where used)
-  Tb* rnE = reinterpret_cast<Tb*>(base + L.geom);       // [N] r from the proposed position
-  Tb* roE = rnE + s.N;                                  // [N] r from the current position
-  Tb* rnN = roE + s.N;                                  // [Nn]
-  Tb* Snew = rnN + s.Nn;                                // [Nn][6]
-  Tb* Upo = Snew + 6 * s.Nn;                            // [5][UP] Rbar(r_ej)^k, current position of e
-  Tb* Upn = Upo + 5 * UP;                               // [5][UP] Rbar(r_ej)^k, proposed position
+  Tb* Sv = reinterpret_cast<Tb*>(base + L.Sv);
+  Tb* ut = reinterpret_cast<Tb*>(base + L.ut);
+  Tb* ft = reinterpret_cast<Tb*>(base + L.ft);
+  // the move: (current, proposed) powers 1..4 of Rbar(r_ej), and the proposed pairs' Rbar and e-e value
+  Pair2<Tb>* Up = reinterpret_cast<Pair2<Tb>*>(base + L.up);  // [4][UP]
+  Tb* ue = reinterpret_cast<Tb*>(base + L.ue);
+  Tb* fe = reinterpret_cast<Tb*>(base + L.fe);
 
   const int N = s.N, Nn = s.Nn, Nup = s.Nup, U0 = s.U[0], ldo = L.nocc_max;
   const Tb kap = (Tb)s.kappa;
-  const Tb* cf = orb_coefs<Tb>(s);
   const Tb* cE = een_coefs<Tb>(s);
-  for (int i = lane; i < 3 * N; i += 32) R[i] = Rg[(size_t)w * 3 * N + i];
+  double* Rw = Rg + (size_t)w * 3 * N;  // current positions in double; accepted moves are written through
   // positions as the bulk-type arithmetic reads them (float-float copies in the mixed form)
-  dsf* Rds = reinterpret_cast<dsf*>(base + L.Rds);
+  double* Rs = reinterpret_cast<double*>(base + L.R);
+  dsf* Rds = reinterpret_cast<dsf*>(base + L.R);
   Coords<Tb> C;
-  if constexpr (kSameType<Tb, double>) {
-    C.R = R;
-  } else {
-    for (int i = lane; i < 3 * N; i += 32) Rds[i] = ds_from_double(Rg[(size_t)w * 3 * N + i]);
-    C.R = Rds;
+  for (int i = lane; i < 3 * N; i += 32) {
+    if constexpr (kSameType<Tb, double>) Rs[i] = Rw[i];
+    else Rds[i] = ds_from_double(Rw[i]);
   }
+  if constexpr (kSameType<Tb, double>) C.R = Rs;
+  else C.R = Rds;
   __syncwarp();
-  // geometry tables
-  for (DivStep ia(lane, Nn); ia.hi < N; ia.next(Nn)) {
-    const int i = ia.hi, a = ia.lo, p = i * Nn + a;
-    const Tb dx = C.en(s, i, a, 0), dy = C.en(s, i, a, 1), dz = C.en(s, i, a, 2);
+  // Rbar and e-e value of a pair from its difference vector
+  auto pair_values = [&](Tb dx, Tb dy, Tb dz, bool same, Tb& u, Tb& f) {
     const Tb r = vsqrt(dx * dx + dy * dy + dz * dz);
-    rEN[p] = r;
-    Sv[a * SA + i] = (Tb)1 / ((Tb)1 + kap * r);
+    u = (Tb)1 / ((Tb)1 + kap * r);
+    f = pade_value<Tb>(ee_coef_t<Tb>(s, same), r, u);
+  };
+  auto tri = [](int i, int j) { return i > j ? i * (i - 1) / 2 + j : j * (j - 1) / 2 + i; };
+  // e-e-n lanes: (nucleus a, part of the partners); with more than 32 nuclei lanes loop over them
+  const int np = max(1, 32 / Nn);
+  int ea0 = lane, ej0 = 0, ej1 = N;
+  if (np > 1) {
+    const DivStep ap(lane, np);
+    ea0 = ap.hi;
+    ej0 = ap.lo * N / np;
+    ej1 = (ap.lo + 1) * N / np;
   }
   // walker state: [Binv spin 0][Binv spin 1][ln|det| (Ut)][sign (Ut)][r_k = D_k/Phi (nterm)]
   // [ln|Phi|][sign Phi]; the sweep starts from the inverses and the term ratios and carries
@@ -131,15 +304,19 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
     if (do_refresh) {
       // double-precision orbital values of every electron, then the inverse of every unique determinant
       auto orbital_values = [&](int e, int sp) {  // of electron e, in vrowd
-        basis_at<double, false>(s, lane, R[3 * e], R[3 * e + 1], R[3 * e + 2], basd, nullptr, nullptr, nullptr,
+        basis_at<double, false>(s, lane, Rw[3 * e], Rw[3 * e + 1], Rw[3 * e + 2], basd, nullptr, nullptr, nullptr,
                                 nullptr);
         __syncwarp();
-        for (int c = lane; c < s.n_occ_chunk[sp]; c += 32) {
-          const int4 ch = __ldg(reinterpret_cast<const int4*>(s.occ_chunk[sp]) + c);
-          const double* cb = s.orb_coef + ch.w;
+        for (int c0 = 0; c0 < s.n_occ_chunk[sp]; c0 += 32) {
+          const int c = c0 + lane;
           double v = 0.0;
-          for (int mu = ch.y; mu < ch.z; ++mu) v = fma(__ldg(cb + mu), basd[mu], v);
-          partd[c] = v;
+          if (c < s.n_occ_chunk[sp]) {
+            const int4 ch = __ldg(reinterpret_cast<const int4*>(s.occ_chunk[sp]) + c);
+            const double* cb = s.orb_coef + ch.w;
+            for (int mu = ch.y; mu < ch.z; ++mu) v = fma(__ldg(cb + mu), basd[mu], v);
+          }
+          if (L.alias) __syncwarp();
+          if (c < s.n_occ_chunk[sp]) partd[c] = v;
         }
         __syncwarp();
         for (int q = lane; q < s.nocc[sp]; q += 32) {
@@ -195,27 +372,128 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
       pe = 0;
       __syncwarp();
     }
-    const uint32_t st = step0 + (uint32_t)sw;
-    // the sweep's random numbers, one electron per lane: the proposed position R_e + step
-    // (2u - 1) per coordinate (electron e has not moved yet in this sweep when its turn comes)
-    // and the acceptance uniform; in the mixed form also the float-float copy of the proposal
-    double* rtab = reinterpret_cast<double*>(base + L.rtab);
-    dsf* rtds = reinterpret_cast<dsf*>(base + L.rtds);
-    for (int e = lane; e < N; e += 32) {
-      double u[4];
-      uniforms2(seed, wid, st, (uint32_t)e, tag, 0, u[0], u[1]);
-      uniforms2(seed, wid, st, (uint32_t)e, tag, 1, u[2], u[3]);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) {
-        const double x = __dadd_rn(R[3 * e + d], __dmul_rn(step, __dsub_rn(__dmul_rn(2.0, u[d]), 1.0)));
-        rtab[4 * e + d] = x;
-        if constexpr (!kSameType<Tb, double>) rtds[3 * e + d] = ds_from_double(x);
+    if (sw == 0 || do_refresh) {
+      // tables of the current positions (a refactorisation uses their place; moves keep them current)
+      for (DivStep ia(lane, Nn); ia.hi < N; ia.next(Nn)) {
+        const int i = ia.hi, a = ia.lo;
+        const Tb dx = C.en(s, i, a, 0), dy = C.en(s, i, a, 1), dz = C.en(s, i, a, 2);
+        const Tb r = vsqrt(dx * dx + dy * dy + dz * dz);
+        Sv[a * SA + i] = (Tb)1 / ((Tb)1 + kap * r);
       }
-      rtab[4 * e + 3] = u[3];
+      if (L.tri)
+        for (int p = lane; p < N * (N - 1) / 2; p += 32) {
+          int i = (int)((1.0f + sqrtf(1.0f + 8.0f * (float)p)) * 0.5f);  // row of the triangle, to one
+          if (i * (i - 1) / 2 > p) --i;
+          if (i * (i + 1) / 2 <= p) ++i;
+          const int j = p - i * (i - 1) / 2;
+          pair_values(C.ee(i, j, 0), C.ee(i, j, 1), C.ee(i, j, 2), (i < Nup) == (j < Nup), ut[p], ft[p]);
+        }
     }
-    __syncwarp();
+    const uint32_t st = step0 + (uint32_t)sw;
+    double uac = 0.0;  // acceptance uniform of the prepared electron 'lane' (at most 32 of them)
+    auto accept_position = [&](int e, int ip) {
+      if (lane < 3) {
+        const double x = rtab[3 * ip + lane];
+        Rw[3 * e + lane] = x;
+        if constexpr (kSameType<Tb, double>) Rs[3 * e + lane] = x;
+        else Rds[3 * e + lane] = rtds[3 * ip + lane];
+      }
+      for (int a = lane; a < Nn; a += 32) Sv[a * SA + e] = svn[ip * Nn + a];
+      if (L.tri)
+        for (int j = lane; j < N; j += 32)
+          if (j != e) {
+            ut[tri(e, j)] = ue[j];
+            ft[tri(e, j)] = fe[j];
+          }
+    };
     for (int e = 0; e < N; ++e) {
       const int sp = e >= Nup ? 1 : 0, ie = e - (sp ? Nup : 0), n = s.n[sp], G = sp ? L.G1 : L.G0;
+      if (e == 0 || e == Nup) {
+        // one electron per lane: the proposed position R_e + step (2u - 1) per coordinate (electron e
+        // has not moved yet in this sweep when its turn comes) and the acceptance uniform; in the
+        // mixed form also the float-float copy of the proposal
+        const int cnt = L.all ? N - e : n;
+        if (e == 0 || !L.all) {
+          if (lane < cnt) {
+            double u[4], Rc[3];  // the position's latency runs under the random numbers
+#pragma unroll
+            for (int d = 0; d < 3; ++d) Rc[d] = Rw[3 * (e + lane) + d];
+            uniforms2(seed, wid, st, (uint32_t)(e + lane), tag, 0, u[0], u[1]);
+            uniforms2(seed, wid, st, (uint32_t)(e + lane), tag, 1, u[2], u[3]);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+              const double x = __dadd_rn(Rc[d], __dmul_rn(step, __dsub_rn(__dmul_rn(2.0, u[d]), 1.0)));
+              rtab[3 * lane + d] = x;
+              if constexpr (!kSameType<Tb, double>) rtds[3 * lane + d] = ds_from_double(x);
+            }
+            uac = u[3];
+          }
+          __syncwarp();
+          // nuclei: Rbar at the proposals and the change of the e-n terms
+          for (DivStep ia(lane, Nn); ia.hi < cnt; ia.next(Nn)) {
+            const int i = ia.hi, a = ia.lo;
+            Tb dn[3], dc[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+              if constexpr (kSameType<Tb, double>) dn[d] = (Tb)(rtab[3 * i + d] - __ldg(s.nuc4 + 4 * a + d));
+              else dn[d] = ds_diff_f(rtds[3 * i + d], nuc_coord_ds(s, a, d));
+              dc[d] = C.en(s, e + i, a, d);
+            }
+            const PadeT<Tb> c = en_coef_t<Tb>(s, a);
+            const Tb rn_ = vsqrt(dn[0] * dn[0] + dn[1] * dn[1] + dn[2] * dn[2]);
+            const Tb rc_ = vsqrt(dc[0] * dc[0] + dc[1] * dc[1] + dc[2] * dc[2]);
+            const Tb sn = (Tb)1 / ((Tb)1 + kap * rn_), sc = (Tb)1 / ((Tb)1 + kap * rc_);
+            svn[i * Nn + a] = sn;
+            den[i * Nn + a] = pade_value<Tb>(c, rn_, sn) - pade_value<Tb>(c, rc_, sc);
+          }
+        }
+        const int p0 = L.all ? e : 0;  // the spin's first electron among the prepared ones
+        const int nr = L.rows ? (e == 0 ? N : 0) : n;
+        // orbital rows at the proposals (bulk type)
+        if constexpr (kSameType<Tb, double>) {
+          for (int i = 0; i < nr; ++i) {
+            const double* r = rtab + 3 * (p0 + i);
+            basis_at<double, false>(s, lane, r[0], r[1], r[2], bas, nullptr, nullptr, nullptr, nullptr);
+            __syncwarp();
+            for (int c0 = 0; c0 < s.n_occ_chunk[sp]; c0 += 32) {
+              const int c = c0 + lane;
+              double v = 0.0;
+              if (c < s.n_occ_chunk[sp]) {
+                const int4 ch = __ldg(reinterpret_cast<const int4*>(s.occ_chunk[sp]) + c);
+                const double* cb = s.orb_coef + ch.w;
+                for (int mu = ch.y; mu < ch.z; ++mu) v += __ldg(cb + mu) * bas[mu];
+              }
+              if (L.alias) __syncwarp();
+              if (c < s.n_occ_chunk[sp]) part[c] = v;
+            }
+            __syncwarp();
+            for (int q = lane; q < s.nocc[sp]; q += 32) {
+              const int c0 = __ldg(s.occ_chunk_off[sp] + q), c1 = __ldg(s.occ_chunk_off[sp] + q + 1);
+              double v = 0.0;
+              for (int c = c0; c < c1; ++c) v += part[c];
+              vrows[i * ldo + q] = v;
+            }
+            __syncwarp();
+          }
+        } else {
+          for (int i = 0; i < nr;) {
+            const int left = nr - i;
+            const dsf* r = rtds + 3 * (p0 + i);
+            float* out = vrows + i * ldo;
+            if (L.ke == 4 && left > 2) {
+              proposal_rows<4, BATCH>(s, lane, sp, min(left, 4), r, bas, part, L.alias, out, ldo);
+              i += 4;
+            } else if (L.ke >= 2 && left > 1) {
+              proposal_rows<2, BATCH>(s, lane, sp, 2, r, bas, part, L.alias, out, ldo);
+              i += 2;
+            } else {
+              proposal_rows<1, BATCH>(s, lane, sp, 1, r, bas, part, L.alias, out, ldo);
+              ++i;
+            }
+          }
+        }
+        __syncwarp();
+      }
       if (TAB && (e == 0 || e == Nup)) {
         // the moving spin's weights g_u and Sigma: the other spin's minors stay until the next spin
         const double* wo = wk + (sp ? 0 : s.tab[0].nv);
@@ -235,44 +513,13 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
         iSig = nonzero(Sig) ? recip(Sig) : 0.0;
         __syncwarp();
       }
-      const double uacc = rtab[4 * e + 3];
-      const double rn[3] = {rtab[4 * e], rtab[4 * e + 1], rtab[4 * e + 2]};
-      // the proposed position as the bulk-type arithmetic reads it
-      dsf rnd[3];
-      if constexpr (!kSameType<Tb, double>) {
-        rnd[0] = rtds[3 * e];
-        rnd[1] = rtds[3 * e + 1];
-        rnd[2] = rtds[3 * e + 2];
-      }
+      const int ip = L.all ? e : ie;  // its place among the prepared electrons
+      const double uacc = __shfl_sync(kFull, uac, ip);
       auto dnew_e = [&](int j, int d) -> Tb {  // proposed position minus electron j
-        if constexpr (kSameType<Tb, double>) return (Tb)(rn[d] - R[3 * j + d]);
-        else return ds_diff_f(rnd[d], Rds[3 * j + d]);
+        if constexpr (kSameType<Tb, double>) return (Tb)(rtab[3 * ip + d] - Rs[3 * j + d]);
+        else return ds_diff_f(rtds[3 * ip + d], Rds[3 * j + d]);
       };
-      auto dnew_n = [&](int a, int d) -> Tb {  // proposed position minus nucleus a
-        if constexpr (kSameType<Tb, double>) return (Tb)(rn[d] - __ldg(s.nuc4 + 4 * a + d));
-        else return ds_diff_f(rnd[d], nuc_coord_ds(s, a, d));
-      };
-      // orbital row at the proposed position (bulk type), contraction in balanced chunks
-      if constexpr (kSameType<Tb, double>)
-        basis_at<double, false>(s, lane, rn[0], rn[1], rn[2], bas, nullptr, nullptr, nullptr, nullptr);
-      else
-        basis_at_f<false>(s, lane, rnd, bas, nullptr, nullptr, nullptr, nullptr);
-      __syncwarp();
-      for (int c = lane; c < s.n_occ_chunk[sp]; c += 32) {
-        const int4 ch = __ldg(reinterpret_cast<const int4*>(s.occ_chunk[sp]) + c);
-        const Tb* cb = cf + ch.w;
-        Tb v = 0;
-        for (int mu = ch.y; mu < ch.z; ++mu) v += __ldg(cb + mu) * bas[mu];
-        part[c] = v;
-      }
-      __syncwarp();
-      for (int q = lane; q < s.nocc[sp]; q += 32) {
-        const int c0 = __ldg(s.occ_chunk_off[sp] + q), c1 = __ldg(s.occ_chunk_off[sp] + q + 1);
-        Tb v = 0;
-        for (int c = c0; c < c1; ++c) v += part[c];
-        if constexpr (kSameType<Tb, double>) vrowd[q] = v;
-        else vrowd[q] = f2d_bits(v);
-      }
+      for (int q = lane; q < s.nocc[sp]; q += 32) vrowd[q] = widen(vrows[(L.rows ? e : ie) * ldo + q]);
       __syncwarp();
       const LaneGroup lgp(lane, G);
       const int U = s.U[sp], ng = lgp.ng, g = lgp.g, gl = lgp.gl;
@@ -342,34 +589,37 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
           }
         }
       }
-      // Jastrow change of the terms that involve electron e (Sec. 2.1): distances from the
-      // proposed position, then items e-n (a), e-e (j) and e-e-n (a, k), the last through the
-      // pair sums Y^{k,q} = sum_{j != e} u_ej^k s_j^q (the terms of e are s_e^A Y^{k,B} + s_e^B Y^{k,A}).
-      for (int j = lane; j < N; j += 32) {
-        const Tb dx = dnew_e(j, 0), dy = dnew_e(j, 1), dz = dnew_e(j, 2);
-        const Tb rnew = j == e ? (Tb)0 : vsqrt(dx * dx + dy * dy + dz * dz);
-        const Tb ox = C.ee(e, j, 0), oy = C.ee(e, j, 1), oz = C.ee(e, j, 2);
-        const Tb rold = j == e ? (Tb)0 : vsqrt(ox * ox + oy * oy + oz * oz);
-        rnE[j] = rnew;
-        roE[j] = rold;
-        const Tb uo = (Tb)1 / ((Tb)1 + kap * rold), un = (Tb)1 / ((Tb)1 + kap * rnew);
-        Tb po = (Tb)1, pn = (Tb)1;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) {
-          Upo[k * UP + j] = po;
-          Upn[k * UP + j] = pn;
-          po *= uo;
-          pn *= un;
+      // Jastrow change of the terms that involve electron e (Sec. 2.1): items e-n (a) and e-e (j),
+      // then e-e-n (a, part of the partners) through the pair sums Y^{k,q} = sum_{j != e} u_ej^k s_j^q
+      // (the terms of e are s_e^A Y^{k,B} + s_e^B Y^{k,A}).
+      Tb dj = 0;
+      for (int t = lane; t < Nn + N; t += 32) {
+        if (t < Nn) {
+          dj += den[ip * Nn + t];
+          continue;
         }
-      }
-      for (int a = lane; a < Nn; a += 32) {
-        const Tb dx = dnew_n(a, 0), dy = dnew_n(a, 1), dz = dnew_n(a, 2);
-        const Tb r = vsqrt(dx * dx + dy * dy + dz * dz);
-        rnN[a] = r;
-        const Tb sv = (Tb)1 / ((Tb)1 + kap * r);
-        Tb pw = (Tb)1;
+        const int j = t - Nn;
+        if (j == e) continue;
+        const bool same = (e < Nup) == (j < Nup);
+        Tb un, f1, uo, f0;
+        pair_values(dnew_e(j, 0), dnew_e(j, 1), dnew_e(j, 2), same, un, f1);
+        if (L.tri) {
+          const int p = tri(e, j);
+          uo = ut[p];
+          f0 = ft[p];
+          ue[j] = un;
+          fe[j] = f1;
+        } else {
+          pair_values(C.ee(e, j, 0), C.ee(e, j, 1), C.ee(e, j, 2), same, uo, f0);
+        }
+        dj += f1 - f0;
+        const Pair2<Tb> u1{uo, un};
+        Pair2<Tb> pw = u1;
 #pragma unroll
-        for (int q = 0; q < 6; ++q) { Snew[a * 6 + q] = pw; pw *= sv; }
+        for (int k = 0; k < 4; ++k) {
+          Up[k * UP + j] = pw;
+          pw = pair_mul(pw, u1);
+        }
       }
       if constexpr (!TAB) {
         if (one_pass) {
@@ -384,66 +634,56 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
         for (int k = lane; k < s.nterm; k += 32)
           rphi += __ldg(s.term_coef + k) * wk[k] * rho[__ldg(s.term_det + 2 * k + sp)];
       }
-      Tb dj = 0;
-      for (int t = lane; t < Nn + N; t += 32) {
-        if (t < Nn) {
-          const PadeT<Tb> c = en_coef_t<Tb>(s, t);
-          Tb f1, f0, t0, t1;
-          pade_eval<Tb, false>(c, rnN[t], kap, f1, t0, t1);
-          pade_eval<Tb, false>(c, rEN[e * Nn + t], kap, f0, t0, t1);
-          dj += f1 - f0;
-        } else {
-          const int j = t - Nn;
-          if (j == e) continue;
-          const PadeT<Tb> c = ee_coef_t<Tb>(s, (e < Nup) == (j < Nup));
-          Tb f1, f0, t0, t1;
-          pade_eval<Tb, false>(c, rnE[j], kap, f1, t0, t1);
-          pade_eval<Tb, false>(c, roE[j], kap, f0, t0, t1);
-          dj += f1 - f0;
-        }
-      }
       if (s.een_on) {
         // e-e-n items (nucleus a, part of the partners j), every k in each: the pair sums
         // are linear in the partners, so each part adds its own share of the change, and all
         // lanes run the same code (no divergence over k)
-        const int np = max(1, 32 / Nn);
-        for (int t = lane; t < np * Nn; t += 32) {
-          const int a = t / np, part = t - np * a;
-          Tb Yo[5][6], Yn[5][6];
+        for (int a = ea0; a < Nn; a += (np > 1 ? Nn : 32)) {
+          Tb Y0[6];
+          Pair2<Tb> Y[4][5];  // k - 1, q <= 5 - k
 #pragma unroll
-          for (int k = 0; k < 5; ++k)
+          for (int q = 0; q < 6; ++q) Y0[q] = (Tb)0;
 #pragma unroll
-            for (int q = 0; q < 6; ++q) Yo[k][q] = Yn[k][q] = (Tb)0;
-          for (int j = part * N / np; j < (part + 1) * N / np; ++j) {
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int q = 0; q < 5; ++q) Y[k][q] = {(Tb)0, (Tb)0};
+          for (int j = ej0; j < ej1; ++j) {
             if (j == e) continue;
             const Tb svj = Sv[a * SA + j];
-            Tb sj[6];
-            sj[0] = (Tb)1;
+            const Pair2<Tb> s1{svj, svj};
+            Pair2<Tb> sj[6];
+            sj[1] = s1;
 #pragma unroll
-            for (int q = 1; q < 6; ++q) sj[q] = sj[q - 1] * svj;
+            for (int q = 2; q < 6; ++q) sj[q] = pair_mul(sj[q - 1], s1);
 #pragma unroll
-            for (int k = 0; k < 5; ++k) {
-              const Tb po = Upo[k * UP + j], pn = Upn[k * UP + j];
+            for (int q = 1; q < 6; ++q) Y0[q] += sj[q].o;
 #pragma unroll
-              for (int q = 0; q <= 5 - k; ++q) {
-                Yo[k][q] += po * sj[q];
-                Yn[k][q] += pn * sj[q];
-              }
+            for (int k = 0; k < 4; ++k) {
+              const Pair2<Tb> u = Up[k * UP + j];
+              Y[k][0] = pair_add(Y[k][0], u);
+#pragma unroll
+              for (int q = 1; q <= 4 - k; ++q) Y[k][q] = pair_fma(u, sj[q], Y[k][q]);
             }
           }
-          Tb So[6];
-          So[0] = (Tb)1;
-          {
-            const Tb sve = Sv[a * SA + e];
+          Pair2<Tb> S[6];
+          S[0] = {(Tb)1, (Tb)1};
+          S[1] = {Sv[a * SA + e], svn[ip * Nn + a]};
 #pragma unroll
-            for (int q = 1; q < 6; ++q) So[q] = So[q - 1] * sve;
-          }
-          const Tb* Sn = Snew + a * 6;
+          for (int q = 2; q < 6; ++q) S[q] = pair_mul(S[q - 1], S[1]);
           const Tb* c = cE + kNeen * __ldg(s.nuc_elem + a);
           een_for_each([&](auto tc) {
             constexpr int q = decltype(tc)::value;
             constexpr int tk = een_klm(q).k, A = een_klm(q).l + een_klm(q).m, B = een_klm(q).m;
-            dj += c[q] * ((Sn[A] * Yn[tk][B] + Sn[B] * Yn[tk][A]) - (So[A] * Yo[tk][B] + So[B] * Yo[tk][A]));
+            Pair2<Tb> YA, YB;
+            if constexpr (tk == 0) {
+              YA = {Y0[A], Y0[A]};
+              YB = {Y0[B], Y0[B]};
+            } else {
+              YA = Y[tk - 1][A];
+              YB = Y[tk - 1][B];
+            }
+            const Pair2<Tb> x = pair_fma(S[A], YB, pair_mul(S[B], YA));
+            dj += c[q] * (x.n - x.o);
           });
         }
       }
@@ -491,14 +731,7 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
         for (int u = lane; u < s.tab[sp].nv; u += 32) wk[vo + u] = qn[u];
         Sig = Sig_new;
         iSig = recip(Sig);  // an accepted ratio is nonzero, so Sigma is
-        if (lane < 3) {
-          R[3 * e + lane] = lane == 0 ? rn[0] : (lane == 1 ? rn[1] : rn[2]);
-          if constexpr (!kSameType<Tb, double>) Rds[3 * e + lane] = lane == 0 ? rnd[0] : (lane == 1 ? rnd[1] : rnd[2]);
-        }
-        for (int a = lane; a < Nn; a += 32) {
-          rEN[e * Nn + a] = rnN[a];
-          Sv[a * SA + e] = Snew[a * 6 + 1];
-        }
+        accept_position(e, ip);
         ++accepted;
       } else if (!TAB && acc) {
         // the reciprocals 1/rho_u and 1/(Phi'/Phi), one per lane
@@ -549,20 +782,12 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
         if (__double_as_longlong(rphi) < 0)
           sgnPhi = __longlong_as_double(__double_as_longlong(sgnPhi) ^ (long long)0x8000000000000000ull);
         for (int k = lane; k < s.nterm; k += 32) wk[k] *= rho[__ldg(s.term_det + 2 * k + sp)] * irphi;
-        if (lane < 3) {
-          R[3 * e + lane] = lane == 0 ? rn[0] : (lane == 1 ? rn[1] : rn[2]);
-          if constexpr (!kSameType<Tb, double>) Rds[3 * e + lane] = lane == 0 ? rnd[0] : (lane == 1 ? rnd[1] : rnd[2]);
-        }
-        for (int a = lane; a < Nn; a += 32) {
-          rEN[e * Nn + a] = rnN[a];
-          Sv[a * SA + e] = Snew[a * 6 + 1];
-        }
+        accept_position(e, ip);
         ++accepted;
       }
       __syncwarp();
     }
   }
-  for (int i = lane; i < 3 * N; i += 32) Rg[(size_t)w * 3 * N + i] = R[i];
   if (nacc && lane == 0) nacc[w] += accepted;
   lnPhi += log(pm) + (double)pe * 0.69314718055994530942;  // ln 2
   if (!TAB && state) {  // the carried inverses, term ratios and ln|Phi| at the final positions

@@ -129,6 +129,7 @@ struct SysDev {
   int N, Nup, Ndn, Nn, n_elem, S, M, Norb, Nvb;
   int n_ev, n_ev_det;
   int nocc[2], U[2], n[2];
+  int same_occ;  // both spins' determinants use the same orbitals (occ_list[0] = occ_list[1])
   int nterm, nsterm;
   int P, n_cparam, jas_param, een_on, n_kappa;
   int p_off_a, p_off_b, p_off_theta, p_off_kappa;
