@@ -135,7 +135,8 @@ cudaError_t launch_eval_t(const SysDev& s, const EvalLayout& L, int W, const dou
     e = launch_dettab<Tb>(s, L.tab, W, static_cast<const Tb*>(b.JG), static_cast<const Tb*>(b.JL), b.JS,
                           static_cast<const Tb*>(b.OB), b.OD, logpsi, sign, eloc, b.VG, grad, O, dEL, st);
   } else {
-    const DetLayout& D = carry ? L.detc : L.det;
+    DetLayout D = carry ? L.detc : L.det;
+    D.wpb = walkers_per_block(W, D.wpb, EvalBounds<Tb>::threads / 32, D.warp_bytes);
     const int smem = D.wpb * D.warp_bytes;
     e = cudaFuncSetAttribute(det_kernel<Tb>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;

@@ -78,10 +78,12 @@ template <class Tb>
 cudaError_t launch_dettab(const SysDev& s, const DetTabLayout& L, int W, const Tb* JG, const Tb* JL, const double* JS,
                           const Tb* OB, const double* OD, double* logpsi, double* sign, double* eloc, double* vg_ws,
                           double* grad, Tb* O, Tb* dEL, cudaStream_t st) {
-  const int smem = L.wpb * L.warp_bytes;
+  DetTabLayout D = L;
+  D.wpb = walkers_per_block(W, L.wpb, kDetTabWarps, L.warp_bytes);
+  const int smem = D.wpb * D.warp_bytes;
   cudaError_t e = cudaFuncSetAttribute(dettab_kernel<Tb>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  dettab_kernel<Tb><<<(W + L.wpb - 1) / L.wpb, 32 * L.wpb, smem, st>>>(s, L, W, JG, JL, JS, OB, OD, logpsi, sign, eloc,
+  dettab_kernel<Tb><<<(W + D.wpb - 1) / D.wpb, 32 * D.wpb, smem, st>>>(s, D, W, JG, JL, JS, OB, OD, logpsi, sign, eloc,
                                                                       vg_ws, grad, O, dEL);
   return cudaGetLastError();
 }

@@ -124,20 +124,24 @@ cudaError_t launch_jastrow(const SysDev& s, const JasLayout& L, int W, const dou
     jastrow_wide_kernel<Tb><<<W, 32 * L.nw, L.wide_bytes, st>>>(s, L, R, JG, JL, JS);
     return cudaGetLastError();
   }
-  const int smem = L.wpb * L.warp_bytes;
+  JasLayout D = L;
+  D.wpb = walkers_per_block(W, L.wpb, 8 * JasBounds<Tb>::min_blocks, L.warp_bytes);
+  const int smem = D.wpb * D.warp_bytes;
   cudaError_t e = set_smem(jastrow_kernel<Tb>, smem);
   if (e != cudaSuccess) return e;
-  jastrow_kernel<Tb><<<(W + L.wpb - 1) / L.wpb, 32 * L.wpb, smem, st>>>(s, L, W, R, JG, JL, JS);
+  jastrow_kernel<Tb><<<(W + D.wpb - 1) / D.wpb, 32 * D.wpb, smem, st>>>(s, D, W, R, JG, JL, JS);
   return cudaGetLastError();
 }
 
 template <class Tb>
 cudaError_t launch_jastrow_deriv(const SysDev& s, const JasLayout& L, int W, const double* R, const double* vg, Tb* O,
                                  Tb* dEL, cudaStream_t st) {
-  const int smem = L.wpb * L.warp_bytes;
+  JasLayout D = L;
+  D.wpb = walkers_per_block(W, L.wpb, 8 * JasBounds<Tb>::min_blocks, L.warp_bytes);
+  const int smem = D.wpb * D.warp_bytes;
   cudaError_t e = set_smem(jastrow_deriv_kernel<Tb>, smem);
   if (e != cudaSuccess) return e;
-  jastrow_deriv_kernel<Tb><<<(W + L.wpb - 1) / L.wpb, 32 * L.wpb, smem, st>>>(s, L, W, R, vg, O, dEL);
+  jastrow_deriv_kernel<Tb><<<(W + D.wpb - 1) / D.wpb, 32 * D.wpb, smem, st>>>(s, D, W, R, vg, O, dEL);
   return cudaGetLastError();
 }
 

@@ -161,24 +161,39 @@ int make_sweep_layout(const SysDev& s, int tb, int max_smem, SweepLayout& L) {
   return VBQMC_OK;
 }
 
+int walkers_per_block(int W, int most, int sm_warps, int bytes) {
+  int dev = 0, sms = 0, sm_smem = 0;
+  if (W < 1 || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess || sms < 1)
+    return most;
+  auto resident = [&](int p) { return std::max(1, std::min(sm_warps / p, sm_smem / (p * bytes + 1024))); };
+  int warps = 0;  // the most walkers on an SM
+  for (int p = 1; p <= most; ++p) warps = std::max(warps, p * resident(p));
+  if ((long)W > 2L * warps * sms)
+    for (int p = std::min(2, most); p <= most; ++p)
+      if (p * resident(p) == warps) return p;
+  long best_cost = 0;
+  int best = most;
+  for (int p = most; p >= 1; --p) {
+    const long res = resident(p);
+    const long blocks = ((long)W + p - 1) / p, full = blocks / (res * sms), rest = blocks - full * res * sms;
+    const long cost = full * (100 + 3 * p * res) + (rest ? 100 + 3 * p * ((rest + sms - 1) / sms) : 0);
+    if (full && res > 4) break;
+    if (p == most || 100 * cost < 98 * best_cost) {
+      best_cost = cost;
+      best = p;
+    }
+  }
+  return best;
+}
+
 template <class Tb>
 static cudaError_t launch_sweep_t(const SysDev& s, const SweepLayout& L, int W, double* R, int nsweeps, int refresh,
                                   double* state, int state_valid, double step, uint64_t seed, uint32_t step0, uint32_t tag,
                                   uint32_t woff, int* nacc, cudaStream_t st) {
-  // walkers per block: the most that fit, unless one or two fewer need no more waves of
-  // blocks over the SMs (a wave costs about 3 % more per extra warp on the SM, measured on the
-  // ethylene-shaped system; an idle part of the last wave costs its full share)
   SweepLayout Lw = L;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) ==
-                                               cudaSuccess && sms > 0 && W > 0) {
-    auto cost = [&](int p) {
-      const long waves = ((long)W + (long)p * sms - 1) / ((long)p * sms);
-      return waves * (100 + 3 * p);
-    };
-    for (int p = L.wpb - 1; p >= std::max(1, L.wpb - 2); --p)
-      if (cost(p) < cost(Lw.wpb)) Lw.wpb = p;
-  }
+  Lw.wpb = walkers_per_block(W, L.wpb, 16, L.warp_bytes);
   const int smem = Lw.wpb * Lw.warp_bytes;
   const void* fn = Lw.tab ? (const void*)sweep_kernel<Tb, true> : (const void*)sweep_kernel<Tb, false>;
   cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

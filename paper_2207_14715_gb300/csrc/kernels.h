@@ -150,6 +150,18 @@ struct OverlapMap {
 size_t overlap_part_doubles(int M, int nvb);
 cudaError_t launch_structure_overlap(int M, int ldo, int otype, const void* O, const double* wts, const OverlapMap& map,
                                      double* part, double* out, cudaStream_t st);
+// Walkers (warps) per block of a kernel of one warp per walker: W walkers, at most 'most' per block,
+// sm_warps warps on an SM by registers, 'bytes' of shared memory per walker.
+//  - More than two rounds of walkers over the SMs: the smallest blocks that keep as many walkers
+//    resident as any size does; a finished block is replaced at once, so rounds do not wait for
+//    their slowest walker (ethylene-shaped system, 16384 walkers: sweep 1082 us with blocks of 16,
+//    1032 of 4; 3001 walkers in double: Jastrow 1739 -> 1450 us, its derivatives 2057 -> 1714 us).
+//  - Fewer: a round of p warps on an SM takes about 100 + 3 p (the warps share the issue slots and
+//    the FP64 pipe); the fewest such units, counting the warps that the last, partly filled round
+//    puts on its busiest SM, larger blocks within 2 %.  A sample that would leave SMs idle with full
+//    blocks is spread over them (300 walkers in double, 5 sweeps: 6.7 -> 2.4 ms); blocks much smaller
+//    than an SM's share are placed unevenly there (4096 walkers, 10 sweeps: 3.75 ms with 14, 4.06 with 4).
+int walkers_per_block(int W, int most, int sm_warps, int bytes);
 // VMC sweeps; state (may be null): read when state_valid, written after the last sweep with the
 // carried inverses, term ratios and ln|Phi| (its ln|det| entries are left as they were).
 cudaError_t launch_sweep(int precision, const SysDev& s, const SweepLayout& L, int W, double* R, int nsweeps,
