@@ -338,8 +338,9 @@ int vbqmc_set_system(vbqmc_ctx* ctx, int sys_id, const vbqmc_system_desc* desc) 
     if (h.tab_ok && vbq::make_det_layout(d, 8, ctx->max_smem, probe) != VBQMC_OK) d.msd = 1;
   }
   make_layouts(ctx, ls);
-  if (!d.msd && h.tab_ok && d.n_kappa == 0 && ls.lay_rc_sweep[VBQMC_MIXED] == VBQMC_OK) {
-    const int bytes = ls.lay_sweep[VBQMC_MIXED].warp_bytes, U = std::max(d.U[0], d.U[1]);
+  const int bytes = vbq::per_determinant_region_bytes(d);
+  if (!d.msd && h.tab_ok && d.n_kappa == 0 && bytes <= ctx->max_smem) {
+    const int U = std::max(d.U[0], d.U[1]);
     if (bytes > 48 * 1024 || (bytes > 32 * 1024 && U >= 16)) {
       d.msd = 1;
       make_layouts(ctx, ls);

@@ -75,7 +75,7 @@ int make_det_layout(const SysDev& s, int tb, int max_smem, DetLayout& L, bool ca
   int scr = 16;
   for (int sp = 0; sp < 2; ++sp) {
     const int n = s.n[sp], G = sp ? L.G1 : L.G0;
-    if (!carried) scr = std::max(scr, inverse_scratch_bytes(n, s.U[sp], G));
+    if (!carried) scr = std::max(scr, inverse_scratch_bytes(n, s.U[sp], G, tb == 8));
     scr = std::max(scr, 8 * s.U[sp] * n);                  // carried state: trace partials
   }
   // Gam and Aux rows of both spins, one product B_u L_u

@@ -90,22 +90,23 @@ int make_sweep_layout(const SysDev& s, int tb, int max_smem, SweepLayout& L) {
     L.wk = take(8 * s.nterm);
   }
   L.vrow = take(8 * L.nocc_max);
-  L.ke = tb == 8 ? 1 : (4 * s.Nn <= 32 ? 4 : (2 * s.Nn <= 32 ? 2 : 1));
   const int nmax = std::max(s.n[0], s.n[1]), nch = std::max(std::max(s.n_occ_chunk[0], s.n_occ_chunk[1]), 1);
   int cv = 0, scr = 0;
   for (int sp = 0; sp < 2; ++sp) {
     const int n = s.n[sp], G = sp ? L.G1 : L.G0, ng = L.tab ? 1 : 32 / G;
     cv = std::max(cv, 8 * (L.tab ? 1 : 2) * ng * n);  // Sherman-Morrison stages two passes' columns
-    scr = std::max(scr, L.tab ? 4 * n + 16 : inverse_scratch_bytes(n, s.U[sp], G));
+    scr = std::max(scr, L.tab ? 4 * n + 16 : inverse_scratch_bytes(n, s.U[sp], G, true));
   }
   // What the moves keep (tables of the current positions, proposals) shares its place with a
   // refactorisation's ln|det|, signs and orbital matrix, consumed by the term ratios before the tables
   // are formed.  Then come the basis values and partial sums of either, over them the buffers of a
   // move, and over all of these the scratch of the inverses (past the orbital matrix).
   const int over0 = off;
-  auto place = [&](bool all, bool tri, bool rows) {  // end of the walker's region
+  auto place = [&](int grp, int ke, bool all, bool tri, bool rows) {  // end of the walker's region
     off = over0;
-    const int np = all ? N : nmax;
+    L.ke = ke;
+    L.grp = grp;
+    const int np = all ? N : grp;
     L.all = all ? 1 : 0;
     L.rows = rows ? 1 : 0;
     L.tri = tri ? 1 : 0;
@@ -113,7 +114,7 @@ int make_sweep_layout(const SysDev& s, int tb, int max_smem, SweepLayout& L) {
     L.rtds = take(tb == 4 ? 8 * 3 * np : 16);
     L.svn = take(tb * np * s.Nn);
     L.den = take(tb * np * s.Nn);
-    L.vrows = take(tb * (rows ? N : nmax) * L.nocc_max);
+    L.vrows = take(tb * (rows ? N : (all ? nmax : grp)) * L.nocc_max);
     L.Sv = take(tb * (N + 1) * s.Nn);
     L.ut = take(tri ? tb * (N * (N - 1) / 2 + 1) : 0);
     L.ft = take(tri ? tb * (N * (N - 1) / 2 + 1) : 0);
@@ -148,11 +149,18 @@ int make_sweep_layout(const SysDev& s, int tb, int max_smem, SweepLayout& L) {
   // the pair tables, and both spins prepared at once (one electron per lane), where as many
   // walkers share a block with them
   auto fit = [&](int bytes) { return std::min(16, max_smem / std::max(bytes, 1)); };
-  const int most = fit(place(false, false, false));
-  const bool tri = fit(place(false, true, false)) == most;
-  const bool all = N <= 32 && fit(place(true, tri, false)) == most;
-  const bool rows = all && s.same_occ && fit(place(true, tri, true)) == most;
-  place(all, tri, rows);
+  // electrons prepared at once: 16 of a spin (a second group of a large spin costs little and its
+  // place is saved), fewer where nothing fits otherwise
+  int grp = std::min(16, nmax);
+  while (grp > 1 && place(grp, 1, false, false, false) > max_smem) grp = grp > 4 ? 4 : 1;
+  const int most = fit(place(grp, 1, false, false, false));
+  int ke = 1;  // electrons a round of proposal rows takes: their displacements lie in one warp's lanes
+  for (int k = 4; k > 1 && ke == 1; k >>= 1)
+    if (tb == 4 && k * s.Nn <= 32 && fit(place(grp, k, false, false, false)) == most) ke = k;
+  const bool tri = fit(place(grp, ke, false, true, false)) == most;
+  const bool all = N <= 32 && fit(place(grp, ke, true, tri, false)) == most;
+  const bool rows = all && s.same_occ && fit(place(grp, ke, true, tri, true)) == most;
+  place(grp, ke, all, tri, rows);
   L.warp_bytes = off;
   int wpb = max_smem / off;
   if (wpb > 16) wpb = 16;
@@ -186,6 +194,32 @@ int walkers_per_block(int W, int most, int sm_warps, int bytes) {
     }
   }
   return best;
+}
+
+int per_determinant_region_bytes(const SysDev& s) {
+  int off = 0;
+  auto take = [&](int bytes) { off = align16(off + bytes); };
+  const int N = s.N, Ut = s.U[0] + s.U[1], nocc = std::max(std::max(s.nocc[0], s.nocc[1]), 1);
+  for (int b : {8 * 3 * N, 8 * 3 * N, 8 * s.U[0] * s.n[0] * s.n[0], 8 * s.U[1] * s.n[1] * s.n[1], 8 * s.nterm}) take(b);
+  const int over0 = off;
+  for (int b : {8 * 4 * N, 8 * 3 * N, 4 * (2 * N + 7 * s.Nn + 10 * (N + 1))}) take(b);
+  const int moves_end = off;
+  off = over0;
+  for (int b : {8 * Ut, 8 * Ut, 8 * N * nocc}) take(b);
+  off = std::max(off, moves_end);
+  int cv = 0, scr = 0;
+  for (int sp = 0; sp < 2; ++sp) {
+    const int n = s.n[sp], ng = 32 / group_size(n);
+    cv = std::max(cv, 16 * ng * n);
+    scr = std::max(scr, ng * (8 * n * n + 4 * n) + 16);
+  }
+  const int shared0 = off;
+  for (int b : {8 * s.M, 8 * nocc, 8 * std::max(std::max(s.n_occ_chunk[0], s.n_occ_chunk[1]), 1),
+                8 * std::max(s.U[0], s.U[1]), 8 * (std::max(s.U[0], s.U[1]) + 1), std::max(cv, 8)})
+    take(b);
+  off = std::max(off, align16(shared0 + std::max(scr, 16)));
+  take(4 * (N * s.Nn + (N + 1) * s.Nn));
+  return off;
 }
 
 template <class Tb>

@@ -63,6 +63,7 @@ struct SweepLayout {
   int up, ue, fe, Sv, ut = 0, ft = 0;
   int ke;         // electrons whose proposal rows are formed together (float form: 4, 2 or 1)
   int alias;      // the contraction's partial sums (one round) overlay the basis values
+  int grp = 1;    // electrons of a spin prepared at once (without all)
   int all = 0;    // proposals and e-n changes of both spins prepared at once
   int rows = 0;   // their orbital rows too (the spins use the same orbitals)
   int tri = 0;    // Rbar and e-e value kept per electron pair (where that costs no walker per block)
@@ -150,6 +151,10 @@ struct OverlapMap {
 size_t overlap_part_doubles(int M, int nvb);
 cudaError_t launch_structure_overlap(int M, int ldo, int otype, const void* O, const double* wts, const OverlapMap& map,
                                      double* part, double* out, cudaStream_t st);
+// Size of a walker by which the form of the determinants is chosen (inverses per determinant or
+// reference tables): inverses, positions, tables and buffers of a sweep whose moves form everything by
+// themselves.  The line was measured with that region; the sweep's own layout may be larger or smaller.
+int per_determinant_region_bytes(const SysDev& s);
 // Walkers (warps) per block of a kernel of one warp per walker: W walkers, at most 'most' per block,
 // sm_warps warps on an SM by registers, 'bytes' of shared memory per walker.
 //  - More than two rounds of walkers over the SMs: the smallest blocks that keep as many walkers

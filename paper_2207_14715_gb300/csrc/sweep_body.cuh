@@ -46,7 +46,8 @@ namespace vbq {
 // per pair (L.tri) and replaced when a move is accepted.  The float values and sums are those of a
 // move that forms everything by itself, bit for bit.  Bound by instruction issue (float) and the
 // FP64 pipe (double); a sweep of the ethylene-shaped system went from 1298 to 1080 us (16384 walkers,
-// mixed), 2303 to 2095 us (3001, double), one of the 48-electron system from 11.5 to 10.0 ms (8192).
+// mixed), 2303 to 2095 us (3001, double), one of the 48-electron system from 11.5 to 10.0 ms (8192), and to
+// 9.4 ms with at most 16 electrons prepared at once and small blocks.
 // One warp, walker w, shared-memory region 'base' of L.warp_bytes bytes.
 
 // f of the Pade + polynomial form at R = r den, den = 1 / (1 + kappa r) (as pade_poly)
@@ -218,13 +219,13 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
   double* rinv = reinterpret_cast<double*>(base + L.rinv);
   double* cvec = reinterpret_cast<double*>(base + L.cvec);
   double* scr = reinterpret_cast<double*>(base + L.scratch);
-  // of the prepared electrons (L.all: every electron; else the moving spin's): proposed positions
-  // (and their float-float copies), Rbar and e-n change per nucleus; orbital rows of the moving spin's
+  // of the prepared electrons (L.all: every electron; else up to L.grp of the moving spin): proposed positions
+  // (and their float-float copies), Rbar and e-n change per nucleus; orbital rows of the moving spin's (L.rows: all)
   double* rtab = reinterpret_cast<double*>(base + L.rtab);  // [][3]
   dsf* rtds = reinterpret_cast<dsf*>(base + L.rtds);        // [][3]
   Tb* svn = reinterpret_cast<Tb*>(base + L.svn);            // [][Nn]
   Tb* den = reinterpret_cast<Tb*>(base + L.den);            // [][Nn]
-  Tb* vrows = reinterpret_cast<Tb*>(base + L.vrows);        // [n or (L.rows) N][nocc]
+  Tb* vrows = reinterpret_cast<Tb*>(base + L.vrows);        // [][nocc]
   // current positions: [Nn][SA] Rbar(r_ja) (its powers formed where used; the row stride padded so that
   // lanes on different nuclei read different banks), and per pair Rbar(r_ij) and the e-e value
   const int SA = s.N + 1, UP = s.N + 1;
@@ -406,13 +407,15 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
             ft[tri(e, j)] = fe[j];
           }
     };
+    int e0 = 0;  // first of the electrons prepared together
     for (int e = 0; e < N; ++e) {
       const int sp = e >= Nup ? 1 : 0, ie = e - (sp ? Nup : 0), n = s.n[sp], G = sp ? L.G1 : L.G0;
-      if (e == 0 || e == Nup) {
+      if (e == 0 || e == Nup || (!L.all && e - e0 == L.grp)) {
+        e0 = e;
         // one electron per lane: the proposed position R_e + step (2u - 1) per coordinate (electron e
         // has not moved yet in this sweep when its turn comes) and the acceptance uniform; in the
         // mixed form also the float-float copy of the proposal
-        const int cnt = L.all ? N - e : n;
+        const int cnt = L.all ? N - e : min(L.grp, n - ie);
         if (e == 0 || !L.all) {
           if (lane < cnt) {
             double u[4], Rc[3];  // the position's latency runs under the random numbers
@@ -448,7 +451,7 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
           }
         }
         const int p0 = L.all ? e : 0;  // the spin's first electron among the prepared ones
-        const int nr = L.rows ? (e == 0 ? N : 0) : n;
+        const int nr = L.rows ? (e == 0 ? N : 0) : (L.all ? n : cnt);
         // orbital rows at the proposals (bulk type)
         if constexpr (kSameType<Tb, double>) {
           for (int i = 0; i < nr; ++i) {
@@ -513,13 +516,13 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
         iSig = nonzero(Sig) ? recip(Sig) : 0.0;
         __syncwarp();
       }
-      const int ip = L.all ? e : ie;  // its place among the prepared electrons
+      const int ip = L.all ? e : e - e0;  // its place among the prepared electrons
       const double uacc = __shfl_sync(kFull, uac, ip);
       auto dnew_e = [&](int j, int d) -> Tb {  // proposed position minus electron j
         if constexpr (kSameType<Tb, double>) return (Tb)(rtab[3 * ip + d] - Rs[3 * j + d]);
         else return ds_diff_f(rtds[3 * ip + d], Rds[3 * j + d]);
       };
-      for (int q = lane; q < s.nocc[sp]; q += 32) vrowd[q] = widen(vrows[(L.rows ? e : ie) * ldo + q]);
+      for (int q = lane; q < s.nocc[sp]; q += 32) vrowd[q] = widen(vrows[(L.rows ? e : e - e0) * ldo + q]);
       __syncwarp();
       const LaneGroup lgp(lane, G);
       const int U = s.U[sp], ng = lgp.ng, g = lgp.g, gl = lgp.gl;

@@ -182,9 +182,9 @@ __device__ __forceinline__ void pade_eval(const PadeCoef& c, Tb r, Tb kap, Tb& f
 // Inverse of every unique determinant of spin sp by lane groups, from the double orbital values
 // Phi[(e0 + e) * ld + idx[u][o]]: ldet[u], dsg[u], and each where given Bd[u], Bg[u] (double) and
 // Bf[u] (float), and t[u] = tr(A_u^-1 L) with L read at Lphi[(e0 + e) * ldL + idx[u][o]].
-// scr: inverse_scratch_bytes.
-__host__ __device__ inline int inverse_scratch_bytes(int n, int U, int G) {
-  return (32 / G) * (8 * n * (n | 1) * (n > 16 ? 2 : 1) + 4 * n) + 4 * U + 16;
+// scr: inverse_scratch_bytes (n > 16: solved in the place of the double inverses, or in scr without them).
+__host__ __device__ inline int inverse_scratch_bytes(int n, int U, int G, bool in_place) {
+  return (32 / G) * (8 * n * (n | 1) * (n > 16 && !in_place ? 2 : 1) + 4 * n) + 4 * U + 16;
 }
 template <class Tb>
 __device__ __forceinline__ void invert_all(const SysDev& s, int sp, int lane, const double* Phi, int ld, const int* idx,
@@ -204,8 +204,8 @@ __device__ __forceinline__ void invert_all(const SysDev& s, int sp, int lane, co
   const int ng = lgp.ng, g = lgp.g, gl = lgp.gl;
   double* A = scr + g * n * lda;
   double* end = scr + ng * n * lda;
-  double* B = end;  // n > 16 only
-  if (n > 16) end += n * lda;
+  double* B = end;  // n > 16 without Bd only
+  if (n > 16 && !Bd) end += n * lda;
   int* perm = reinterpret_cast<int*>(end) + g * n;
   int* ex = reinterpret_cast<int*>(end) + ng * n;
   for (int u0 = 0; u0 < U; u0 += ng) {
@@ -215,7 +215,7 @@ __device__ __forceinline__ void invert_all(const SysDev& s, int sp, int lane, co
     const double* P = Phi + e0 * ld;
     const GroupDet d = n <= 8    ? group_lu8(P, ld, iu, n, G, act, A, perm)
                        : n <= 16 ? group_lu16(P, ld, iu, n, G, act, A, perm)
-                                 : group_lu_smem(P, ld, iu, n, G, act, A, B, perm);
+                                 : group_lu_smem(P, ld, iu, n, G, act, A, Bd ? Bd + u * n * n : B, perm, Bd ? n : 0);
     double t = 0.0;
     if (tdet && act && gl < n) {
       const int col = __ldg(iu + gl);

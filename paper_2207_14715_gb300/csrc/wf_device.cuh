@@ -292,10 +292,11 @@ __device__ __forceinline__ GroupDet group_lu_n(const double* Phi, int ld, const 
   return group_det(diag, in, swaps, singular, G);
 }
 
-// the same with the matrix in shared memory (16 < n <= 32: one group); B: n (n | 1) doubles more
+// the same with the matrix in shared memory (16 < n <= 32: one group); B [n][ldb] (0: n | 1): place of the solution
 static __device__ __noinline__ GroupDet group_lu_smem(const double* Phi, int ld, const int* idx, int n, int G, bool active,
-                                                      double* A, double* B, int* perm) {
+                                                      double* A, double* B, int* perm, int ldb = 0) {
   const int lane = lane_id(), gl = lane & (G - 1), gbase = lane & ~(G - 1), lda = n | 1;
+  if (ldb == 0) ldb = lda;
   const bool in = active && gl < n;
   if (in) {
     perm[gl] = gl;
@@ -344,20 +345,20 @@ static __device__ __noinline__ GroupDet group_lu_smem(const double* Phi, int ld,
   for (int i = 0; i < n; ++i) {
     double y = in && perm[i] == gl ? 1.0 : 0.0;
     if (in)
-      for (int k = 0; k < i; ++k) y = fma(-A[i * lda + k], B[k * lda + gl], y);
-    if (in) B[i * lda + gl] = y;
+      for (int k = 0; k < i; ++k) y = fma(-A[i * lda + k], B[k * ldb + gl], y);
+    if (in) B[i * ldb + gl] = y;
   }
   for (int i = n - 1; i >= 0; --i) {
     const double di = __shfl_sync(kFull, dinv, (gbase + i) & 31);
     if (in) {
-      double x = B[i * lda + gl];
-      for (int k = i + 1; k < n; ++k) x = fma(-A[i * lda + k], B[k * lda + gl], x);
-      B[i * lda + gl] = x * di;
+      double x = B[i * ldb + gl];
+      for (int k = i + 1; k < n; ++k) x = fma(-A[i * lda + k], B[k * ldb + gl], x);
+      B[i * ldb + gl] = x * di;
     }
   }
   __syncwarp();
   if (in)
-    for (int i = 0; i < n; ++i) A[i * lda + gl] = singular ? 0.0 : B[i * lda + gl];
+    for (int i = 0; i < n; ++i) A[i * lda + gl] = singular ? 0.0 : B[i * ldb + gl];
   __syncwarp();
   return group_det(diag, in, swaps, singular, G);
 }
