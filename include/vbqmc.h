@@ -167,6 +167,11 @@ int vbqmc_eval_walkers(vbqmc_ctx* ctx, int sys_id, int precision, int W, const d
  * VBQMC_ERR_UNSUPPORTED for systems with Slater shells or on reference-determinant tables. */
 int vbqmc_eval_nuclear_derivs(vbqmc_ctx* ctx, int sys_id, int precision, int W, const double* R, double* logpsi,
                               double* sign, double* eloc, double* dlogpsi_dR, double* dEL_dR, void* stream);
+/* The same with the parameter derivatives O, dEL of vbqmc_eval_walkers (NULL: left out) from the one
+ * evaluation of the walkers. */
+int vbqmc_eval_all_derivs(vbqmc_ctx* ctx, int sys_id, int precision, int W, const double* R, double* logpsi,
+                          double* sign, double* eloc, void* O, void* dEL, double* dlogpsi_dR, double* dEL_dR,
+                          void* stream);
 
 /* Weighted sums over walkers of derivative rows, in double with a fixed summation order:
  *   out[k] = sum_w (ga[w] Ja[w][k] + gb[w] Jb[w][k]),  k < K.

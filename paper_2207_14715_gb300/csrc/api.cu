@@ -456,19 +456,22 @@ int vbqmc_eval_walkers(vbqmc_ctx* ctx, int sys_id, int precision, int W, const d
   return VBQMC_OK;
 }
 
-int vbqmc_eval_nuclear_derivs(vbqmc_ctx* ctx, int sys_id, int precision, int W, const double* R, double* logpsi,
-                              double* sign, double* eloc, double* dlogpsi_dR, double* dEL_dR, void* stream) {
+int vbqmc_eval_all_derivs(vbqmc_ctx* ctx, int sys_id, int precision, int W, const double* R, double* logpsi,
+                          double* sign, double* eloc, void* O, void* dEL, double* dlogpsi_dR, double* dEL_dR,
+                          void* stream) {
   int rc = check_call(ctx, sys_id, precision, W);
   if (rc) return rc;
   ctx->last_launches = 0;
   if (W == 0) return VBQMC_OK;
   if (!R || !logpsi || !sign || !eloc || !dlogpsi_dR) return fail(VBQMC_ERR_ARG, "null required pointer");
+  if (dEL && !O) return fail(VBQMC_ERR_ARG, "dEL requires O");
   LoadedSystem& s = ctx->sys[sys_id];
   if (s.lay_rc_eval[precision]) return fail(s.lay_rc_eval[precision], "per-walker state exceeds shared memory");
   if (s.dev.msd) return fail(VBQMC_ERR_UNSUPPORTED, "nucleus derivatives with reference-determinant tables");
   if (s.host.has_slater) return fail(VBQMC_ERR_UNSUPPORTED, "nucleus derivatives of Slater shells");
   if (s.lay_rc_force[precision])
     return fail(s.lay_rc_force[precision], "nucleus-derivative tables exceed shared memory");
+  if ((O || dEL) && s.dev.P == 0) O = dEL = nullptr;
   DeviceGuard g(ctx->device);
   const cudaStream_t st = (cudaStream_t)stream;
   rc = ensure_eval_ws(ctx, s, precision, W, st);
@@ -486,11 +489,17 @@ int vbqmc_eval_nuclear_derivs(vbqmc_ctx* ctx, int sys_id, int precision, int W, 
   }
   int nl = 0;
   cudaError_t e = vbq::launch_nuclear_derivs(precision, s.dev, s.lay_eval[precision], s.lay_force[precision], W, R,
-                                             logpsi, sign, eloc, dlogpsi_dR, dEL_dR, ctx->eval_work,
+                                             logpsi, sign, eloc, O, dEL, dlogpsi_dR, dEL_dR, ctx->eval_work,
                                              ctx->force_work, st, &nl);
   ctx->last_launches = nl;
   if (e != cudaSuccess) return cuda_fail(e, "nucleus-derivative kernel launch");
   return VBQMC_OK;
+}
+
+int vbqmc_eval_nuclear_derivs(vbqmc_ctx* ctx, int sys_id, int precision, int W, const double* R, double* logpsi,
+                              double* sign, double* eloc, double* dlogpsi_dR, double* dEL_dR, void* stream) {
+  return vbqmc_eval_all_derivs(ctx, sys_id, precision, W, R, logpsi, sign, eloc, nullptr, nullptr, dlogpsi_dR, dEL_dR,
+                               stream);
 }
 
 int vbqmc_weighted_colsum(vbqmc_ctx* ctx, int W, int K, int jtype, const double* ga, const void* Ja,

@@ -551,13 +551,13 @@ size_t force_workspace_bytes(const SysDev& s, int W) {
 }
 
 cudaError_t launch_nuclear_derivs(int precision, const SysDev& s, const EvalLayout& LE, const ForceLayout& LF, int W,
-                                  const double* R, double* logpsi, double* sign, double* eloc, double* dlp,
-                                  double* dEL, void* ws, void* fws, cudaStream_t st, int* nlaunch) {
+                                  const double* R, double* logpsi, double* sign, double* eloc, void* O, void* dELp,
+                                  double* dlp, double* dEL, void* ws, void* fws, cudaStream_t st, int* nlaunch) {
   const int tb = precision == VBQMC_MIXED ? 4 : 8;
   double* state = static_cast<double*>(fws);
   double* aux = reinterpret_cast<double*>(static_cast<unsigned char*>(fws) +
                                           (((size_t)std::max(W, 1) * s.state_doubles * 8 + 255) & ~size_t(255)));
-  cudaError_t e = launch_eval(precision, s, LE, W, R, logpsi, sign, eloc, nullptr, nullptr, nullptr, state, ws, st,
+  cudaError_t e = launch_eval(precision, s, LE, W, R, logpsi, sign, eloc, nullptr, O, dELp, state, ws, st,
                               nlaunch, nullptr, aux);
   if (e != cudaSuccess) return e;
   const EvalWs b = carve_eval_ws(s, tb, W, ws);

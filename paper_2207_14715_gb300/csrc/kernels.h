@@ -131,8 +131,8 @@ cudaError_t launch_eval(int precision, const SysDev& s, const EvalLayout& L, int
 // workspace; fws: force_workspace_bytes(s, W) bytes (walker state and determinant weights).
 size_t force_workspace_bytes(const SysDev& s, int W);
 cudaError_t launch_nuclear_derivs(int precision, const SysDev& s, const EvalLayout& LE, const ForceLayout& LF, int W,
-                                  const double* R, double* logpsi, double* sign, double* eloc, double* dlp,
-                                  double* dEL, void* ws, void* fws, cudaStream_t st, int* nlaunch);
+                                  const double* R, double* logpsi, double* sign, double* eloc, void* O, void* dELp,
+                                  double* dlp, double* dEL, void* ws, void* fws, cudaStream_t st, int* nlaunch);
 // out[k] = sum_w (ga[w] Ja[w][k] + gb[w] Jb[w][k]) (gradient.cu); J element type double
 // (jtype 0) or float (jtype 1), gb/Jb may be null; part: colsum_slices(W) * K doubles.
 int colsum_slices(int W);

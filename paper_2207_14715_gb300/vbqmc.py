@@ -56,7 +56,8 @@ EXPORTED = ["vbqmc_create", "vbqmc_destroy", "vbqmc_last_error", "vbqmc_set_syst
             "vbqmc_dmc_steps", "vbqmc_set_kernel_timing", "vbqmc_kernel_times", "vbqmc_batch_create",
             "vbqmc_batch_destroy", "vbqmc_batch_vmc_steps", "vbqmc_batch_tune", "vbqmc_batch_info",
             "vbqmc_eval_nuclear_derivs", "vbqmc_weighted_colsum", "vbqmc_lin_solve", "vbqmc_structure_overlap",
-            "vbqmc_structure_weights", "vbqmc_measure_alu_peaks", "vbqmc_lin_merge", "vbqmc_use_tables"]
+            "vbqmc_structure_weights", "vbqmc_measure_alu_peaks", "vbqmc_lin_merge", "vbqmc_use_tables",
+            "vbqmc_eval_all_derivs"]
 
 _LIB = None
 
@@ -79,6 +80,7 @@ def lib():
                                          vp]
         L.vbqmc_eval_nuclear_derivs.argtypes = [vp, ctypes.c_int, ctypes.c_int, ctypes.c_int, vp, vp, vp, vp, vp, vp,
                                                 vp]
+        L.vbqmc_eval_all_derivs.argtypes = [vp, ctypes.c_int, ctypes.c_int, ctypes.c_int] + [vp] * 9
         L.vbqmc_weighted_colsum.argtypes = [vp, ctypes.c_int, ctypes.c_int, ctypes.c_int, vp, vp, vp, vp, vp, vp]
         L.vbqmc_vmc_steps.argtypes = [vp, ctypes.c_int, ctypes.c_int, ctypes.c_int, vp, ctypes.c_int, ctypes.c_double,
                                       ctypes.c_uint64, ctypes.c_uint32, ctypes.c_uint32, ctypes.c_uint32, ctypes.c_int,
@@ -272,12 +274,15 @@ class Context:
         _check(lib().vbqmc_weighted_colsum(self.h, W, K, jtype, _ptr(ga), _ptr(Ja), _ptr(gb), _ptr(Jb), _ptr(out),
                                            _stream(stream)))
 
-    def eval_nuclear_derivs(self, sys_id, precision, R, logpsi, sign, eloc, dlogpsi_dR, dEL_dR=None, stream=None):
-        """Evaluation plus d ln|Psi|/dR_a and dE_L/dR_a ([W, Nn, 3] float64 CUDA tensors)."""
+    def eval_nuclear_derivs(self, sys_id, precision, R, logpsi, sign, eloc, dlogpsi_dR, dEL_dR=None, stream=None,
+                            O=None, dEL=None):
+        """Evaluation plus d ln|Psi|/dR_a and dE_L/dR_a ([W, Nn, 3] float64 CUDA tensors); O, dEL: the
+        parameter derivatives too (as eval_walkers), from the same evaluation."""
         W = R.shape[0]
-        _check(lib().vbqmc_eval_nuclear_derivs(self.h, int(sys_id), int(precision), int(W), _ptr(R), _ptr(logpsi),
-                                               _ptr(sign), _ptr(eloc), _ptr(dlogpsi_dR), _ptr(dEL_dR),
-                                               _stream(stream)))
+        _check_deriv(precision, O, dEL)
+        _check(lib().vbqmc_eval_all_derivs(self.h, int(sys_id), int(precision), int(W), _ptr(R), _ptr(logpsi),
+                                           _ptr(sign), _ptr(eloc), _ptr(O), _ptr(dEL), _ptr(dlogpsi_dR), _ptr(dEL_dR),
+                                           _stream(stream)))
 
     def vmc_steps(self, sys_id, precision, R, nsweeps, step, seed, step0=0, system_tag=0, walker_offset=0,
                   refresh=1, state=None, state_valid=False, nacc=None, logpsi=None, sign=None, eloc=None, O=None,
