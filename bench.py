@@ -38,9 +38,9 @@ WALKER_KERNEL_SOURCES = {"sweep": ["kernels.cu", "sweep_body.cuh"] + _COMMON_SOU
                          "orbitals": ["eval_orbitals.cu", "orbital_body.cuh"] + _COMMON_SOURCES,
                          "jastrow": ["eval_jastrow.cu", "jastrow_body.cuh"] + _COMMON_SOURCES}
 PROFILED_TRAFFIC = {
-    "sweep": ("282f97f15ec056b95ca54391cd230c827fe9b4dc3b04783db99c8ca6c38daa7d", 10862.5),
-    "det": ("2b71d97144b4651efed3caca6ec526642a0828cb1e515851c6e4a118689f42e1", 26410.8),
-    "orbitals": ("d68d06277ae1b8dbf8f9209074e417fc21ce06de2e3cdacab233c41ca3dd13dd", 9004.3),
+    "sweep": ("244f78b91ff5c8533fc44c0448802bb31cae4e8f8672ea368bd58aaf0bc5eb95", 10884.7),
+    "det": ("db53a660e3b55e8458d235d88a2d90e4903fb1f58eb9bb593146e1fed341424c", 26494.1),
+    "orbitals": ("21d607ab450fa5030d8fdbd7f2bad29956124f1bd9c616db9c6b2267c33129bb", 9048.9),
     "jastrow": ("9bb53d641580f851d7480ef8d5c101d8363dfc188579676e4813c39251a35a10", 392.2),
 }
 
