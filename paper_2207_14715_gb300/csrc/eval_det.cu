@@ -138,7 +138,7 @@ cudaError_t launch_eval_t(const SysDev& s, const EvalLayout& L, int W, const dou
     DetLayout D = carry ? L.detc : L.det;
     D.wpb = walkers_per_block(W, D.wpb, EvalBounds<Tb>::threads / 32, D.warp_bytes);
     const int smem = D.wpb * D.warp_bytes;
-    e = cudaFuncSetAttribute(det_kernel<Tb>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = open_shared_memory((const void*)det_kernel<Tb>);
     if (e != cudaSuccess) return e;
     det_kernel<Tb><<<(W + D.wpb - 1) / D.wpb, 32 * D.wpb, smem, st>>>(
         s, D, W, static_cast<const Tb*>(b.JG), static_cast<const Tb*>(b.JL), b.JS, static_cast<const Tb*>(b.OB), b.OD,

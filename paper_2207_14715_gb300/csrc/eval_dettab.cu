@@ -81,7 +81,7 @@ cudaError_t launch_dettab(const SysDev& s, const DetTabLayout& L, int W, const T
   DetTabLayout D = L;
   D.wpb = walkers_per_block(W, L.wpb, kDetTabWarps, L.warp_bytes);
   const int smem = D.wpb * D.warp_bytes;
-  cudaError_t e = cudaFuncSetAttribute(dettab_kernel<Tb>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = open_shared_memory((const void*)dettab_kernel<Tb>);
   if (e != cudaSuccess) return e;
   dettab_kernel<Tb><<<(W + D.wpb - 1) / D.wpb, 32 * D.wpb, smem, st>>>(s, D, W, JG, JL, JS, OB, OD, logpsi, sign, eloc,
                                                                       vg_ws, grad, O, dEL);

@@ -563,12 +563,12 @@ cudaError_t launch_nuclear_derivs(int precision, const SysDev& s, const EvalLayo
   const EvalWs b = carve_eval_ws(s, tb, W, ws);
   const int smem = LF.block_bytes, threads = 32 * LF.nwarps;
   if (precision == VBQMC_MIXED) {
-    e = cudaFuncSetAttribute(force_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = open_shared_memory((const void*)force_kernel<float>);
     if (e != cudaSuccess) return e;
     force_kernel<float><<<W, threads, smem, st>>>(s, LF, R, static_cast<const float*>(b.JG),
                                                   static_cast<const float*>(b.OB), state, aux, dlp, dEL);
   } else {
-    e = cudaFuncSetAttribute(force_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = open_shared_memory((const void*)force_kernel<double>);
     if (e != cudaSuccess) return e;
     force_kernel<double><<<W, threads, smem, st>>>(s, LF, R, static_cast<const double*>(b.JG),
                                                    static_cast<const double*>(b.OB), state, aux, dlp, dEL);

@@ -110,16 +110,11 @@ int make_jas_layout(const SysDev& s, int tb, int max_smem, JasLayout& L) {
   return VBQMC_OK;
 }
 
-template <class K>
-static cudaError_t set_smem(K kernel, int smem) {
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-}
-
 template <class Tb>
 cudaError_t launch_jastrow(const SysDev& s, const JasLayout& L, int W, const double* R, Tb* JG, Tb* JL, double* JS,
                            cudaStream_t st) {
   if (L.nw > 1) {
-    cudaError_t e = set_smem(jastrow_wide_kernel<Tb>, L.wide_bytes);
+    cudaError_t e = open_shared_memory((const void*)jastrow_wide_kernel<Tb>);
     if (e != cudaSuccess) return e;
     jastrow_wide_kernel<Tb><<<W, 32 * L.nw, L.wide_bytes, st>>>(s, L, R, JG, JL, JS);
     return cudaGetLastError();
@@ -127,7 +122,7 @@ cudaError_t launch_jastrow(const SysDev& s, const JasLayout& L, int W, const dou
   JasLayout D = L;
   D.wpb = walkers_per_block(W, L.wpb, 8 * JasBounds<Tb>::min_blocks, L.warp_bytes);
   const int smem = D.wpb * D.warp_bytes;
-  cudaError_t e = set_smem(jastrow_kernel<Tb>, smem);
+  cudaError_t e = open_shared_memory((const void*)jastrow_kernel<Tb>);
   if (e != cudaSuccess) return e;
   jastrow_kernel<Tb><<<(W + D.wpb - 1) / D.wpb, 32 * D.wpb, smem, st>>>(s, D, W, R, JG, JL, JS);
   return cudaGetLastError();
@@ -139,7 +134,7 @@ cudaError_t launch_jastrow_deriv(const SysDev& s, const JasLayout& L, int W, con
   JasLayout D = L;
   D.wpb = walkers_per_block(W, L.wpb, 8 * JasBounds<Tb>::min_blocks, L.warp_bytes);
   const int smem = D.wpb * D.warp_bytes;
-  cudaError_t e = set_smem(jastrow_deriv_kernel<Tb>, smem);
+  cudaError_t e = open_shared_memory((const void*)jastrow_deriv_kernel<Tb>);
   if (e != cudaSuccess) return e;
   jastrow_deriv_kernel<Tb><<<(W + D.wpb - 1) / D.wpb, 32 * D.wpb, smem, st>>>(s, D, W, R, vg, O, dEL);
   return cudaGetLastError();

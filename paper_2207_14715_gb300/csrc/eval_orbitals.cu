@@ -64,7 +64,7 @@ template <class Tb>
 cudaError_t launch_orbitals(const SysDev& s, const OrbLayout& L, int W, const double* R, Tb* OB, double* OD,
                             cudaStream_t st) {
   const int smem = L.wpb * L.warp_bytes;
-  cudaError_t e = cudaFuncSetAttribute(orbital_kernel<Tb>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = open_shared_memory((const void*)orbital_kernel<Tb>);
   if (e != cudaSuccess) return e;
   const long long points = (long long)W * s.N;
   orbital_kernel<Tb><<<(unsigned)((points + L.wpb - 1) / L.wpb), 32 * kOrbWarps, smem, st>>>(s, L, W, R, OB, OD);

@@ -196,6 +196,15 @@ int walkers_per_block(int W, int most, int sm_warps, int bytes) {
   return best;
 }
 
+cudaError_t open_shared_memory(const void* fn, int static_bytes) {
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  return e == cudaSuccess
+             ? cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most - static_bytes)
+             : e;
+}
+
 int per_determinant_region_bytes(const SysDev& s) {
   int off = 0;
   auto take = [&](int bytes) { off = align16(off + bytes); };
@@ -230,7 +239,7 @@ static cudaError_t launch_sweep_t(const SysDev& s, const SweepLayout& L, int W, 
   Lw.wpb = walkers_per_block(W, L.wpb, 16, L.warp_bytes);
   const int smem = Lw.wpb * Lw.warp_bytes;
   const void* fn = Lw.tab ? (const void*)sweep_kernel<Tb, true> : (const void*)sweep_kernel<Tb, false>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  cudaError_t e = open_shared_memory(fn);
   if (e != cudaSuccess) return e;
   const int blocks = (W + Lw.wpb - 1) / Lw.wpb;
   if (Lw.tab)
@@ -249,7 +258,9 @@ cudaError_t launch_sweep_batch(const BatchSys* sys, const BatchItem* items, int 
   return cudaGetLastError();
 }
 int batch_grid(const void* fn, int nitems, int warps, int smem, int persist) {
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return -1;
+  cudaFuncAttributes own;
+  if (cudaFuncGetAttributes(&own, fn) != cudaSuccess) return -1;
+  if (open_shared_memory(fn, (int)own.sharedSizeBytes) != cudaSuccess) return -1;
   if (persist <= 0) return nitems;
   int bps = 0, dev = 0, sms = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, 32 * warps, smem) != cudaSuccess) return -1;

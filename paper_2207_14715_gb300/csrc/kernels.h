@@ -167,6 +167,12 @@ int per_determinant_region_bytes(const SysDev& s);
 //    blocks is spread over them (300 walkers in double, 5 sweeps: 6.7 -> 2.4 ms); blocks much smaller
 //    than an SM's share are placed unevenly there (4096 walkers, 10 sweeps: 3.75 ms with 14, 4.06 with 4).
 int walkers_per_block(int W, int most, int sm_warps, int bytes);
+// Dynamic shared-memory limit of kernel fn on the current device: what the device allows a block, less
+// fn's own static shared memory.  The limit is a property of the function, shared by every host thread
+// and context, while the size of a launch depends on its system and population: a limit set to one
+// launch's size can be lowered between another thread's setting and its launch, which then fails.
+// Every caller sets the same value, before each launch.
+cudaError_t open_shared_memory(const void* fn, int static_bytes = 0);
 // VMC sweeps; state (may be null): read when state_valid, written after the last sweep with the
 // carried inverses, term ratios and ln|Phi| (its ln|det| entries are left as they were).
 cudaError_t launch_sweep(int precision, const SysDev& s, const SweepLayout& L, int W, double* R, int nsweeps,
