@@ -196,7 +196,7 @@ int vbqmc_set_system(vbqmc_ctx* ctx, int sys_id, const vbqmc_system_desc* desc) 
   for (int sp = 0; sp < 2; ++sp) {
     const vbq::TabMinorsHost& t = h.tab_min[sp];
     const std::vector<int>* const v[vbq::kTabLists] = {&t.sl, &t.l1, &t.l2, &t.l3, &t.l4, &t.rt_off, &t.rt, &t.du_off,
-                                                       &t.du, &t.ld};
+                                                       &t.du, &t.ld, &t.lr_off, &t.lh, &t.le};
     for (int k = 0; k < vbq::kTabLists; ++k) o_min[sp][k] = bb.add(*v[k]);
   }
   cudaError_t e = cudaMalloc(&ls.blob, bb.bytes.size());
@@ -260,9 +260,9 @@ int vbqmc_set_system(vbqmc_ctx* ctx, int sys_id, const vbqmc_system_desc* desc) 
     vbq::TabMinors& m = d.tab[sp];
     m.ns = t.ns; m.nx = t.nx; m.nv = t.nv;
     m.n1 = (int)t.l1.size() / 2; m.n2 = (int)t.l2.size() / 4; m.n3 = (int)t.l3.size() / 4; m.n4 = (int)t.l4.size() / 8;
-    m.nd = (int)t.ld.size() / 10;
+    m.nd = (int)t.ld.size() / 4;
     const int** const ptr[vbq::kTabLists] = {&m.sl, &m.l1, &m.l2, &m.l3, &m.l4, &m.rt_off, &m.rt, &m.du_off, &m.du,
-                                             &m.ld};
+                                             &m.ld, &m.lr_off, &m.lh, &m.le};
     for (int k = 0; k < vbq::kTabLists; ++k) *ptr[k] = (const int*)(B + o_min[sp][k]);
   }
   d.tab_xl[0] = (const int*)(B + o_txl0);

@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(MAXT, 1) batch_fused_kernel(const BatchSys* __
       for (int r = wl; r < item.count; r += cd) {
         const int w = item.first + r;
         if (b.dev.msd)
-          dettab_body<Tb>(b.dev, b.lay.tab, w, smem + wl * b.lay.tab.warp_bytes, static_cast<const Tb*>(b.JG),
+          dettab_body<Tb, true>(b.dev, b.lay.tab, w, smem + wl * b.lay.tab.warp_bytes, static_cast<const Tb*>(b.JG),
                           static_cast<const Tb*>(b.JL), b.JS, static_cast<const Tb*>(b.OB), b.OD, b.logpsi, b.sign,
                           b.eloc, b.VG, nullptr, d ? static_cast<Tb*>(b.O) : nullptr,
                           d ? static_cast<Tb*>(b.dEL) : nullptr);

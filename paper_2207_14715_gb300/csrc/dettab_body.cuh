@@ -9,7 +9,8 @@ namespace vbq {
 
 namespace {
 
-template <class Tb>
+// ALONE: whether the system may hold determinants formed by themselves.
+template <class Tb, bool ALONE>
 __device__ __forceinline__ void dettab_body(const SysDev& s, const DetTabLayout& L, int w, unsigned char* base,
                                             const Tb* JG, const Tb* JL, const double* JS, const Tb* OB,
                                             const double* OD, double* __restrict__ logpsi,
@@ -25,7 +26,7 @@ __device__ __forceinline__ void dettab_body(const SysDev& s, const DetTabLayout&
   double* V[2] = {reinterpret_cast<double*>(base + L.v0), reinterpret_cast<double*>(base + L.v1)};
   int* perm = reinterpret_cast<int*>(base + L.perm);
   double* Tn = reinterpret_cast<double*>(base + L.Tn);    // [ns][nx] the rows of T that the minors read
-  double* PX = reinterpret_cast<double*>(base + L.PX);    // [n][nx] Phi_X, then (with derivatives) L_X - L_0 T
+  double* PX = reinterpret_cast<double*>(base + L.PX);    // [n][nx] Phi_X, then staged cofactors, then (with derivatives) L_X - L_0 T
   double* Ls = reinterpret_cast<double*>(base + L.Ls);    // [n][nevd] dressed Laplacian of the spin's electrons
   double* adj = reinterpret_cast<double*>(base + L.adj);
   double* gT = reinterpret_cast<double*>(base + L.gT);    // [ns][nx] Gamma
@@ -64,7 +65,7 @@ __device__ __forceinline__ void dettab_body(const SysDev& s, const DetTabLayout&
         Tn[rx.hi * nx + rx.lo] = T[__ldg(tm.sl + rx.hi) * nx + rx.lo];
       __syncwarp();
     }
-    tab_values(tm, lane, Tn, V[sp]);
+    tab_values<ALONE, false>(tm, lane, Tn, V[sp]);
   }
 
   // ---- structure sum: Sigma = sum_k C_k q_up(k) q_dn(k), each spin's minors scaled by a power of
@@ -127,7 +128,7 @@ __device__ __forceinline__ void dettab_body(const SysDev& s, const DetTabLayout&
       Ls[eq.hi * nevd + eq.lo] = fma(2.0, d, widen(ob[4 * nev]));
     }
     __syncwarp();
-    tab_adjoint(tm, lane, Tn, V[sp], adj, gT);
+    tab_adjoint<ALONE>(tm, lane, Tn, V[sp], adj, gT, PX, L.sd);
     // h[x][i] = sum_o Gamma[o][x] B[o][i]
     for (DivStep xe(lane, n); xe.hi < nx; xe.next(n)) {
       double h = 0.0;
@@ -155,7 +156,7 @@ __device__ __forceinline__ void dettab_body(const SysDev& s, const DetTabLayout&
       }
       __syncwarp();
       double* td = tdet + (sp ? U0 : 0);
-      tab_derivatives(tm, U, lane, Tn, V[sp], gT, td);
+      tab_derivatives<ALONE>(tm, U, lane, Tn, V[sp], gT, td);
       for (int u = lane; u < U; u += 32) td[u] = nonzero(V[sp][u]) ? t0 + td[u] / V[sp][u] : 0.0;
       __syncwarp();
     }

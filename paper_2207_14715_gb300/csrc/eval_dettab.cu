@@ -22,8 +22,11 @@ namespace vbq {
 
 namespace {
 constexpr int kDetTabWarps = 12;
-template <class Tb>
-__global__ void __launch_bounds__(32 * kDetTabWarps, 1)
+// ALONE: for systems with determinants formed by themselves (tab_minors.cuh), whose functions would cost the
+// others registers (an evaluation of 4096 walkers with 10 active orbitals 0.49 in place of 0.41 ms).
+// 512: at most 128 registers, so that small blocks can put 16 warps on an SM (without spills; 137 otherwise).
+template <class Tb, bool ALONE>
+__global__ void __launch_bounds__(ALONE ? 512 : 32 * kDetTabWarps, 1)
     dettab_kernel(const SysDev s, const DetTabLayout L, int W, const Tb* __restrict__ JG, const Tb* __restrict__ JL,
                   const double* __restrict__ JS, const Tb* __restrict__ OB, const double* __restrict__ OD,
                   double* __restrict__ logpsi, double* __restrict__ sgn_out, double* __restrict__ eloc,
@@ -32,8 +35,8 @@ __global__ void __launch_bounds__(32 * kDetTabWarps, 1)
   const int wl = threadIdx.x >> 5;
   const int w = blockIdx.x * L.wpb + wl;
   if (w >= W) return;
-  dettab_body<Tb>(s, L, w, smem + wl * L.warp_bytes, JG, JL, JS, OB, OD, logpsi, sgn_out, eloc, vg_ws, grad, Og,
-                  dELg);
+  dettab_body<Tb, ALONE>(s, L, w, smem + wl * L.warp_bytes, JG, JL, JS, OB, OD, logpsi, sgn_out, eloc, vg_ws, grad, Og,
+                         dELg);
 }
 
 }  // namespace
@@ -61,11 +64,15 @@ int make_dettab_layout(const SysDev& s, int tb, int max_smem, DetTabLayout& L) {
   L.tdet = take(8 * (s.U[0] + s.U[1]));
   L.perm = take(4 * nmax);
   L.Tn = take(8 * nt);
-  L.PX = take(8 * nx);
   L.Ls = take(8 * nmax * nevd);
   L.adj = take(8 * std::max(s.U[0], s.U[1]));
   L.gT = take(8 * nt);
   L.Gam = take(8 * nx);
+  // Phi_X, and over it the cofactors of 32 determinants formed by themselves, of fewer where these
+  // would not fit (with the shared memory that a batched launch keeps for itself)
+  L.sd = m[0].nd + m[1].nd > 0 ? 32 : 1;
+  while (16 * L.sd > nx && L.sd > 1 && off + 128 * L.sd > max_smem - 1024) L.sd /= 2;
+  L.PX = take(8 * (m[0].nd + m[1].nd > 0 ? std::max(nx, 16 * L.sd) : nx));
   L.warp_bytes = off;
   int wpb = max_smem / off;
   if (wpb > kDetTabWarps) wpb = kDetTabWarps;
@@ -81,10 +88,11 @@ cudaError_t launch_dettab(const SysDev& s, const DetTabLayout& L, int W, const T
   DetTabLayout D = L;
   D.wpb = walkers_per_block(W, L.wpb, kDetTabWarps, L.warp_bytes);
   const int smem = D.wpb * D.warp_bytes;
-  cudaError_t e = open_shared_memory((const void*)dettab_kernel<Tb>);
+  const auto kernel = s.tab[0].nd + s.tab[1].nd > 0 ? dettab_kernel<Tb, true> : dettab_kernel<Tb, false>;
+  cudaError_t e = open_shared_memory((const void*)kernel);
   if (e != cudaSuccess) return e;
-  dettab_kernel<Tb><<<(W + D.wpb - 1) / D.wpb, 32 * D.wpb, smem, st>>>(s, D, W, JG, JL, JS, OB, OD, logpsi, sign, eloc,
-                                                                      vg_ws, grad, O, dEL);
+  kernel<<<(W + D.wpb - 1) / D.wpb, 32 * D.wpb, smem, st>>>(s, D, W, JG, JL, JS, OB, OD, logpsi, sign, eloc, vg_ws, grad,
+                                                            O, dEL);
   return cudaGetLastError();
 }
 template cudaError_t launch_dettab<float>(const SysDev&, const DetTabLayout&, int, const float*, const float*,

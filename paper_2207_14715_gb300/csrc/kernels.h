@@ -40,6 +40,7 @@ struct DetLayout {
 struct DetTabLayout {
   int wpb = 0, warp_bytes = 0;
   int vg, G, B0, B1, T0, T1, v0, v1, tdet, perm, Tn, PX, Ls, adj, gT, Gam;
+  int sd = 32;  // determinants formed by themselves whose cofactors are staged at once (over PX)
 };
 
 struct EvalLayout {

@@ -353,7 +353,7 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
           for (DivStep ox(lane, max(nx, 1)); ox.hi < s.tab[sp].ns && nx > 0; ox.next(nx))
             Tn[ox.hi * nx + ox.lo] = T[__ldg(s.tab[sp].sl + ox.hi) * nx + ox.lo];
           __syncwarp();
-          tab_values(s.tab[sp], lane, Tn, wk + (sp ? s.tab[0].nv : 0));
+          tab_values<true, true>(s.tab[sp], lane, Tn, wk + (sp ? s.tab[0].nv : 0));
         }
       } else {
         for (int e = 0; e < N; ++e) {
@@ -556,7 +556,7 @@ __device__ __forceinline__ void sweep_body(const SysDev& s, const SweepLayout& L
           Tn[ox.hi * nx + ox.lo] = fma(cvec[o], cxv[ox.lo], T[o * nx + ox.lo]);
         }
         __syncwarp();
-        tab_values(tm, lane, Tn, qn);
+        tab_values<true, true>(tm, lane, Tn, qn);
         double sg = 0.0;
         for (int u = lane; u < U; u += 32) sg = fma(qn[u], gw[u], sg);
         Sig_new = warp_sum(sg);

@@ -309,6 +309,7 @@ static void make_minors(const std::vector<int>& tab_det, int U, int nx, TabMinor
   const int nt = m.ns * nx;
   const int kNeg = (int)0x80000000u;
   std::vector<std::vector<int>> ut(nt);  // by Tn entry
+  std::vector<int> alone;  // determinants formed each by itself
   m.du_off.assign(1, 0);
   auto t_of = [&](int s, int x) { return row(s) * nx + x; };
   for (int q = 0; q < m.nv; ++q) {
@@ -320,12 +321,7 @@ static void make_minors(const std::vector<int>& tab_det, int U, int nx, TabMinor
     } else if (k == 2) {
       m.l2.insert(m.l2.end(), {q, t_of(S[0], Q[0]) | t_of(S[1], Q[1]) << 16, t_of(S[0], Q[1]) | t_of(S[1], Q[0]) << 16, 0});
     } else if (k >= 3 && direct) {
-      int e[10] = {q, k, 0, 0, 0, 0, 0, 0, 0, 0};
-      for (int j = 0; j < k; ++j) {
-        e[2 + j] = row(S[j]);
-        e[6 + j] = Q[j];
-      }
-      m.ld.insert(m.ld.end(), e, e + 10);
+      alone.push_back(q);
     } else if (k >= 3) {
       std::vector<int>& l = k == 3 ? m.l3 : m.l4;
       l.push_back(q);
@@ -349,6 +345,29 @@ static void make_minors(const std::vector<int>& tab_det, int U, int nx, TabMinor
     m.rt.insert(m.rt.end(), ut[t].begin(), ut[t].end());
     m.rt_off.push_back((int)(m.rt.size() / 2));
   }
+  std::stable_sort(alone.begin(), alone.end(),
+                   [&](int a, int b) { return node[a].first.size() > node[b].first.size(); });
+  m.lr_off.assign(1, 0);
+  for (size_t d0 = 0; d0 < alone.size(); d0 += 32) {
+    std::map<int, std::vector<int>> by_entry;
+    for (size_t d = d0; d < std::min(alone.size(), d0 + 32); ++d) {
+      const std::vector<int>&S = node[alone[d]].first, &Q = node[alone[d]].second;
+      const int k = (int)S.size();
+      int rows = 0, cols[2] = {0, 0};
+      for (int i = 0; i < k; ++i) {
+        rows |= row(S[i]) << (8 * i);
+        cols[i / 2] |= (int)((unsigned)Q[i] << (16 * (i & 1)));
+        for (int j = 0; j < k; ++j) by_entry[t_of(S[i], Q[j])].push_back((int)(d - d0) << 4 | (4 * i + j));
+      }
+      m.ld.insert(m.ld.end(), {(int)((unsigned)alone[d] | (unsigned)k << 28), rows, cols[0], cols[1]});
+    }
+    for (const auto& e : by_entry) {
+      m.lh.insert(m.lh.end(), {e.first, (int)m.le.size()});
+      m.le.insert(m.le.end(), e.second.begin(), e.second.end());
+    }
+    m.lr_off.push_back((int)(m.lh.size() / 2));
+  }
+  m.lh.insert(m.lh.end(), {nt, (int)m.le.size()});
 }
 
 #define VBQ_REQUIRE(cond, msg)                 \

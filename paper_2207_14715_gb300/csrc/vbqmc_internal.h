@@ -33,17 +33,20 @@ std::vector<EenTerm> een_term_list();
 //   l4 [n4][8] slot, the four terms (+ - + -), 0, 0, 0;
 // and the k^2 first derivatives of every determinant's minor, by Tn entry (rt: determinant with the
 // sign in bit 31, cofactor) and by determinant (du: Tn index with the sign, cofactor), the cofactor
-// as -1 for 1, a slot, or 0x10000 + t.  Where the added minors would outnumber the determinants
-// (many determinants over many orbitals), none is added and ld [nd][10] lists the determinants
-// with k >= 3 to be expanded each by itself: slot, k, the 4 rows, the 4 columns of Tn.
+// as -1 for 1, a slot, or 0x10000 + t.  Where determinants and added minors would be more than
+// 2 U + 256 (many determinants over many orbitals), none is added, and the determinants with k >= 3 are
+// formed each by itself (k = 4 before k = 3): ld [nd][4] slot | k << 28, the rows of Tn (8 bits each),
+// the columns (16 bits each), and for the derivatives by Tn entry, per round of 32 of them, heads
+// lh [..][2] (t, start in le; round r takes lr_off[r] .. lr_off[r + 1], a last one closes the list) with
+// the round's cofactors le: determinant in the round << 4 | 4 row + column.
 struct TabMinors {
   int ns, nx, nv, n1, n2, n3, n4, nd;
-  const int *sl, *l1, *l2, *l3, *l4, *rt_off, *rt, *du_off, *du, *ld;
+  const int *sl, *l1, *l2, *l3, *l4, *rt_off, *rt, *du_off, *du, *ld, *lr_off, *lh, *le;
 };
-constexpr int kTabLists = 10;
+constexpr int kTabLists = 13;
 struct TabMinorsHost {
   int ns = 0, nx = 0, nv = 0;
-  std::vector<int> sl, l1, l2, l3, l4, rt_off, rt, du_off, du, ld;
+  std::vector<int> sl, l1, l2, l3, l4, rt_off, rt, du_off, du, ld, lr_off, lh, le;
 };
 
 // Everything the kernels need, as host vectors (built by build_system).
