@@ -75,23 +75,6 @@ __device__ __forceinline__ void load4(const Tin* __restrict__ row, int c, int P,
   }
 }
 
-// Largest |x| seen, kept as the value's own bits: for finite doubles the order of the absolute
-// values is the order of their bit patterns, so the FP64 pipe (64 cycles per warp instruction, a
-// conversion to float like any other) takes no part; rounding to float commutes with the maximum.
-template <class Tin> struct AbsMax {
-  unsigned long long b = 0;
-  __device__ __forceinline__ void take(Tin x) {
-    const unsigned long long v = (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
-    b = v > b ? v : b;
-  }
-  __device__ __forceinline__ float value() const { return (float)__longlong_as_double((long long)b); }
-};
-template <> struct AbsMax<float> {
-  float m = 0.0f;
-  __device__ __forceinline__ void take(float x) { m = fmaxf(m, fabsf(x)); }
-  __device__ __forceinline__ float value() const { return m; }
-};
-
 // double -> float, round to nearest even, on the bit pattern (about ten integer instructions in
 // place of one on the FP64 pipe); values outside the normal float range take the conversion.
 __device__ __forceinline__ float to_float(double x) {
@@ -110,7 +93,9 @@ __device__ __forceinline__ float to_float(double x) {
 // Block (g, b) (column group fastest, so that the blocks sharing a sample range run together
 // and a 128-byte line that straddles two column groups comes from DRAM once) takes columns
 // [64 g, 64 g + 64): thread (r, q) = (tid / 16, tid % 16) columns 64 g + 4 q .. + 3 of samples
-// 256 b + r, + 16, ...; the 16 row partials are added in row order.
+// 256 b + r, + 16, ...; the 16 row partials are added in row order.  Double input: the maxima of the
+// converted values.  Kept as the doubles' bit patterns they take no conversion on the FP64 pipe but 12 to
+// 24 more registers, a block less per SM: 0.97 in place of 0.90 ms at 2^18 x 400, 9.07 of 8.42 at 2^24 x 1.
 template <class Tin, bool VEC>
 __global__ void __launch_bounds__(kColBlock) lin_colsum_kernel(int P, long long M, const Tin* __restrict__ O,
                                                                const Tin* __restrict__ dEL,
@@ -166,7 +151,7 @@ __global__ void __launch_bounds__(kColBlock) lin_colsum_kernel(int P, long long 
     }
     const int c = blockIdx.x * 64 + 4 * q;
     Tin so[4] = {0, 0, 0, 0}, sd[4] = {0, 0, 0, 0};
-    AbsMax<Tin> mo[4], md[4];
+    float mo[4] = {0.0f, 0.0f, 0.0f, 0.0f}, md[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     auto take = [&](int sl) {
       Tin o[4], d[4];
       load4<Tin, VEC>(O + (s0 + sl) * P, c, P, o);
@@ -176,8 +161,8 @@ __global__ void __launch_bounds__(kColBlock) lin_colsum_kernel(int P, long long 
       for (int u = 0; u < 4; ++u) {
         so[u] += ws * o[u];
         sd[u] += ws * d[u];
-        mo[u].take(o[u]);
-        md[u].take(d[u]);
+        mo[u] = fmaxf(mo[u], fabsf((float)o[u]));
+        md[u] = fmaxf(md[u], fabsf((float)d[u]));
       }
     };
     if (c < P) {
@@ -193,8 +178,8 @@ __global__ void __launch_bounds__(kColBlock) lin_colsum_kernel(int P, long long 
     for (int u = 0; u < 4; ++u) {
       red_o[r][4 * q + u] = so[u];
       red_d[r][4 * q + u] = sd[u];
-      red_mo[r][4 * q + u] = mo[u].value();
-      red_md[r][4 * q + u] = md[u].value();
+      red_mo[r][4 * q + u] = mo[u];
+      red_md[r][4 * q + u] = md[u];
     }
     __syncthreads();
     if (tid < 64) {
@@ -334,11 +319,14 @@ __device__ __forceinline__ void split_half2(float x, float y, __half& xh, __half
 // tile's loads before the stores was tried: at 85 registers and 3 blocks per SM it ran 1.55 in place
 // of 1.51 ms (2^20 x 400), so the blocks stay 4 to an SM and load at the top.  With double input the
 // FP64 pipe bounds the pass: three instructions per value (difference, y, w Ot E) and none for the
-// conversions to float (99 -> 59 us at 15001 x 216, with more and shorter blocks).
-template <class Tin> struct CenBlocks { static constexpr int n = 4; };
-template <> struct CenBlocks<double> { static constexpr int n = 2; };
+// conversions to float (99 -> 59 us at 15001 x 216, with more and shorter blocks).  Blocks of 8 tiles,
+// taken where the sample fills the chip, need four of them on an SM to cover their latency (64 registers;
+// two with 127: 1.44 in place of 1.39 ms at 2^18 x 400, 10.1 of 8.9 at 2^24 x 4); shorter ones run in about
+// one wave and gain more from the registers (30 in place of 38 us at 15000 x 20).
+template <class Tin, int ntile> struct CenBlocks { static constexpr int n = ntile == 8 ? 4 : 2; };
+template <int ntile> struct CenBlocks<float, ntile> { static constexpr int n = 4; };
 template <class Tin, bool VEC, int ntile>
-__global__ void __launch_bounds__(256, CenBlocks<Tin>::n)
+__global__ void __launch_bounds__(256, CenBlocks<Tin, ntile>::n)
     lin_center_kernel(int P, long long M, long long Mp, const Tin* __restrict__ O, const Tin* __restrict__ dEL,
                       const double* __restrict__ E, const double* __restrict__ w, const float* __restrict__ rwf,
                       const float* __restrict__ Ef, const double* __restrict__ acc, const float* __restrict__ scl,
