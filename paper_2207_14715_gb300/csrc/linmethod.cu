@@ -43,7 +43,8 @@ constexpr int kTa = 128;          // output tile rows i (MMA M, tensor-memory la
 constexpr int kTb = 112;          // widest output tile, columns j of S and of H: B = [X_j; Y_j], N = 224
 constexpr int kColBlock = 256;    // threads of a column-sum block (and samples per sub-tile)
 constexpr int kCenTiles = 8;      // most 64-sample tiles per centring block: 512 samples
-constexpr int kSeg = 64;          // rows the workspace's second partial array holds beyond one per 512 samples
+constexpr int kSeg = 64;          // most segments of many partial rows; also the rows that the workspace's second
+                                  // partial array holds beyond one per 512 samples
 constexpr float kScaleTop = 16384.0f;  // scaled values stay below 2^14 (half precision max 65504)
 
 __host__ __device__ inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
@@ -202,17 +203,42 @@ __global__ void __launch_bounds__(kColBlock) lin_colsum_kernel(int P, long long 
   }
 }
 
-// Sum over rows of part[row][q] for the 8 columns q0 + (tid & 7) < L, by a block of NT threads: thread
+// Partial rows are summed column by column in one go up to kRowsOnce of them.  More are first added in
+// segments of 'step' rows over the whole chip, a segment's sum in its own first row, since the few blocks
+// of the column sums would read them alone: at 2^24 samples x 113 parameters (float) these took 0.10 ms for
+// the first partials and 0.14 for the second, of 16.08 ms; 15.86 with the segments.
+constexpr int kRowsOnce = 4096;
+__global__ void __launch_bounds__(256) lin_seg_reduce(int L, int nb, int step, double* __restrict__ part) {
+  __shared__ double red[8][32];
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int q = blockIdx.x * 32 + lane;
+  const int b0 = blockIdx.y * step, b1 = min(nb, b0 + step);
+  double s = 0.0;
+  if (q < L)
+#pragma unroll 4
+    for (int b = b0 + wp; b < b1; b += 8) s += part[(size_t)b * L + q];
+  red[wp][lane] = s;
+  __syncthreads();
+  if (wp == 0 && q < L) {
+    double t = red[0][lane];
+#pragma unroll
+    for (int k = 1; k < 8; ++k) t += red[k][lane];
+    part[(size_t)b0 * L + q] = t;
+  }
+}
+
+// Sum over the rows b < n of part[b step][q] for the 8 columns q0 + (tid & 7) < L, by a block of NT threads: thread
 // (r, c) = (tid / 8, tid % 8) adds rows r, r + NT / 8, ... (64 contiguous bytes per row of threads),
 // then the row sums are added in a fixed order.  The sum is returned by the threads tid < 8.
 // 'red' holds NT doubles.
 template <int NT>
-__device__ __forceinline__ double column_sum(int L, int nrow, const double* __restrict__ part, int q0, double* red) {
+__device__ __forceinline__ double column_sum(int L, int n, int step, const double* __restrict__ part, int q0,
+                                             double* red) {
   const int c = threadIdx.x & 7, r = threadIdx.x >> 3;
   double s = 0.0;
   if (q0 + c < L)
 #pragma unroll 8
-    for (int b = r; b < nrow; b += NT / 8) s += part[(size_t)b * L + q0 + c];
+    for (int b = r; b < n; b += NT / 8) s += part[(size_t)b * step * L + q0 + c];
   __syncthreads();  // the previous use of red is over
   red[threadIdx.x] = s;
   __syncthreads();
@@ -239,7 +265,8 @@ __device__ __forceinline__ double column_sum(int L, int nrow, const double* __re
 // a per-sample launch: on a small sample these took 23 of 238 us, each a few microseconds of
 // latency with most SMs idle (15001 x 216 doubles).
 constexpr int kStatThreads = 512;
-__global__ void __launch_bounds__(kStatThreads) lin_stats_kernel(int P, int Pr, int nb, const double* __restrict__ part,
+__global__ void __launch_bounds__(kStatThreads) lin_stats_kernel(int P, int Pr, int n, int step,
+                                                                 const double* __restrict__ part,
                                                                  const unsigned* __restrict__ mx,
                                                                  double* __restrict__ acc, float* __restrict__ scl,
                                                                  int nq, long long M, const double* __restrict__ E,
@@ -259,7 +286,7 @@ __global__ void __launch_bounds__(kStatThreads) lin_stats_kernel(int P, int Pr, 
   {
     double s = 0.0;
 #pragma unroll 4
-    for (int b = threadIdx.x; b < nb; b += kStatThreads) s += part[(size_t)b * L];
+    for (int b = threadIdx.x; b < n; b += kStatThreads) s += part[(size_t)b * step * L];
     __syncthreads();
     red[threadIdx.x] = s;
     for (int k = kStatThreads / 2; k > 0; k >>= 1) {
@@ -269,7 +296,7 @@ __global__ void __launch_bounds__(kStatThreads) lin_stats_kernel(int P, int Pr, 
     __syncthreads();
     if (threadIdx.x == 0) sw = red[0];
   }
-  const double t = column_sum<kStatThreads>(L, nb, part, q0, red);
+  const double t = column_sum<kStatThreads>(L, n, step, part, q0, red);
   const int q = q0 + threadIdx.x;
   if (threadIdx.x < 8 && q < L) {
     acc[q] = q == 0 ? sw : t;  // one value of sum w for everyone
@@ -639,24 +666,26 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   if (warp == kMmaWarp) tmem_dealloc(tmem, 2 * kSetCols);
 }
 
-// (4) Blocks b < P * nj (nj = blocks per row): thread (i, j) forms S[i][j] and H[i][j] from the chunk
-// partials [chunk][2][Pa][Pb], unscaled; the blocks after them sum w Ot E over the centring blocks'
-// partials, 8 parameters each, for gL and gR.
+// (4) Blocks b < nj: thread (i, j), entries in row order, forms S[i][j] and H[i][j] from the chunk partials
+// [chunk][2][Pa][Pb], unscaled (blocks of whole rows and four chunks unrolled took 74 in place of 41 us for
+// 152 chunks of 100 x 100); the blocks after them sum w Ot E over the centring blocks' partials, 8
+// parameters each, for gL and gR.
 constexpr int kRedThreads = 256;
 __global__ void __launch_bounds__(kRedThreads)
-    lin_reduce_kernel(int P, int Pa, int Pb, int Pr, int nchunk, int nj, int nb2, const double* __restrict__ part,
+    lin_reduce_kernel(int P, int Pa, int Pb, int Pr, int nchunk, int nj, int n, int step,
+                      const double* __restrict__ part,
                       const double* __restrict__ acc, const double* __restrict__ part2, const float* __restrict__ scl,
                       double* E0, double* gL, double* gR, double* S, double* H, const int* __restrict__ err) {
   __shared__ double red[kRedThreads];
   // a timed-out tensor-core stage leaves NaN outputs
   const double isw = *err ? __longlong_as_double(0x7ff8000000000000ll) : 1.0 / acc[0];
   const int b = blockIdx.x;
-  if (b < P * nj) {
-    const int i = b / nj, j = (b - i * nj) * kRedThreads + threadIdx.x;
-    if (j >= P) return;
+  if (b < nj) {
+    const long long e = (long long)b * kRedThreads + threadIdx.x;
+    if (e >= (long long)P * P) return;
+    const int i = (int)(e / P), j = (int)(e - (long long)i * P);
     const size_t o = (size_t)i * Pb + j, plane = (size_t)Pa * Pb;
     double s = 0.0, h = 0.0;
-#pragma unroll 4
     for (int c = 0; c < nchunk; ++c) {
       s += part[(size_t)c * 2 * plane + o];
       h += part[(size_t)c * 2 * plane + plane + o];
@@ -666,8 +695,8 @@ __global__ void __launch_bounds__(kRedThreads)
     H[(size_t)i * P + j] = h / (sxi * syj) * isw;
     return;
   }
-  const int q0 = (b - P * nj) * 8;
-  const double t = column_sum<kRedThreads>(Pr, nb2, part2, q0, red);
+  const int q0 = (b - nj) * 8;
+  const double t = column_sum<kRedThreads>(Pr, n, step, part2, q0, red);
   const int q = q0 + threadIdx.x;
   if (threadIdx.x < 8 && q < P) {
     const double oe = t * isw;  // <Ot E>
@@ -827,8 +856,18 @@ static cudaError_t launch_lin_t(int P, long long M, const Tin* O, const Tin* dEL
     lin_colsum_kernel<Tin, true><<<gcol, kColBlock, 0, st>>>(P, M, O, dEL, E, w, L.part1, L.mx, nb1);
   else
     lin_colsum_kernel<Tin, false><<<gcol, kColBlock, 0, st>>>(P, M, O, dEL, E, w, L.part1, L.mx, nb1);
+  *nlaunch = 5;
+  auto segments = [&](int cols, int nb, double* part) {  // rows between those that are left to sum
+    if (nb <= kRowsOnce) return 1;
+    const int step = (nb + kSeg - 1) / kSeg;
+    lin_seg_reduce<<<dim3((cols + 31) / 32, (nb + step - 1) / step), 256, 0, st>>>(cols, nb, step, part);
+    ++*nlaunch;
+    return step;
+  };
+  const int step1 = segments(L1, nb1, L.part1);
   const int nq = (L1 + 7) / 8, ns = (int)std::min<long long>((M + 4 * kStatThreads - 1) / (4 * kStatThreads), 256);
-  lin_stats_kernel<<<nq + ns, kStatThreads, 0, st>>>(P, Pr, nb1, L.part1, L.mx, L.acc, L.scl, nq, M, E, w, L.rw, L.Ef);
+  lin_stats_kernel<<<nq + ns, kStatThreads, 0, st>>>(P, Pr, (nb1 + step1 - 1) / step1, step1, L.part1, L.mx, L.acc, L.scl,
+                                                  nq, M, E, w, L.rw, L.Ef);
   mark(1);
   const dim3 gcen(Pr / 64, (unsigned)std::min(nb2, 65535));
   auto center = [&](auto kernel) {
@@ -845,6 +884,7 @@ static cudaError_t launch_lin_t(int P, long long M, const Tin* O, const Tin* dEL
     if (nt == 2) center_nt(std::integral_constant<int, 2>{});
     else center_nt(std::integral_constant<int, 1>{});
   }
+  const int step2 = segments(Pr, nb2, L.part2);
   mark(2);
   // the narrowest tiles whose CTAs still run in one wave
   auto ctas = [&](int tb) { return (long long)(Pa / kTa) * ((P + tb - 1) / tb) * G.nchunk; };
@@ -852,11 +892,11 @@ static cudaError_t launch_lin_t(int P, long long M, const Tin* O, const Tin* dEL
                       : (ctas(64) <= nsm ? launch_tc<64>(L, P, M, Mp, G, st) : launch_tc<kTb>(L, P, M, Mp, G, st));
   if (e != cudaSuccess) return e;
   mark(3);
-  const int nj = (P + kRedThreads - 1) / kRedThreads;
-  lin_reduce_kernel<<<P * nj + (P + 7) / 8, kRedThreads, 0, st>>>(P, Pa, Pb, Pr, G.nchunk, nj, nb2, L.part, L.acc,
-                                                                  L.part2, L.scl, E0, gL, gR, S, H, L.err);
+  const int nj = (int)(((long long)P * P + kRedThreads - 1) / kRedThreads);
+  lin_reduce_kernel<<<nj + (P + 7) / 8, kRedThreads, 0, st>>>(
+      P, Pa, Pb, Pr, G.nchunk, nj, (nb2 + step2 - 1) / step2, step2, L.part, L.acc, L.part2, L.scl, E0, gL, gR, S, H,
+      L.err);
   mark(4);
-  *nlaunch = 5;
   return cudaGetLastError();
 }
 
