@@ -4,6 +4,7 @@
 // orbital-excitation tables (Sec. 2.2).
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <map>
 #include <sstream>
 
@@ -264,43 +265,100 @@ static void make_quads(SysHost& s) {
 }
 
 // The minors of one spin's reference tables (TabMinors) from its determinant rows tab_det.
+namespace {
+static_assert(kMaxExc <= 4, "a minor's rows and columns are 16 bits each of a word");
+struct Minor {  // reference slots and x indices, both ascending, 0xffff after the k of each
+  uint64_t rows = ~0ull, cols = ~0ull;
+  int k = 0;
+  static int at(uint64_t v, int i) { return (int)(v >> (16 * i) & 0xffff); }
+  int row(int i) const { return at(rows, i); }
+  int col(int j) const { return at(cols, j); }
+  static uint64_t without(uint64_t v, int i) {
+    const uint64_t low = (1ull << (16 * i)) - 1;
+    return (v & low) | (v >> 16 & ~low) | 0xffffull << 48;
+  }
+  Minor without(int i, int j) const {
+    Minor c;
+    c.rows = without(rows, i);
+    c.cols = without(cols, j);
+    c.k = k - 1;
+    return c;
+  }
+};
+
+// Minor -> its number, by open addressing (most: the largest count).  An ordered map of vectors
+// took 0.3 of the 1.26 ms that the set-up of the 48-electron system takes.
+class MinorTable {
+ public:
+  explicit MinorTable(size_t most) {
+    size_t n = 64;
+    while (n < 2 * most) n *= 2;
+    entry_.resize(n);
+  }
+  int& find(const Minor& m) {  // -1: not yet there
+    size_t h = (m.rows * 0x9e3779b97f4a7c15ull) ^ (m.cols * 0xc2b2ae3d27d4eb4full);
+    for (h ^= h >> 29;; ++h) {
+      Entry& e = entry_[h & (entry_.size() - 1)];
+      if (e.number < 0) {
+        e.rows = m.rows;
+        e.cols = m.cols;
+        return e.number;
+      }
+      if (e.rows == m.rows && e.cols == m.cols) return e.number;
+    }
+  }
+
+ private:
+  struct Entry {
+    uint64_t rows = 0, cols = 0;
+    int number = -1;
+  };
+  std::vector<Entry> entry_;
+};
+}  // namespace
+
 static void make_minors(const std::vector<int>& tab_det, int U, int nx, TabMinorsHost& m) {
-  typedef std::pair<std::vector<int>, std::vector<int>> Key;  // reference slots, x indices, both ascending
   m = TabMinorsHost();
   m.nx = nx;
-  std::vector<Key> node(U);
-  std::map<Key, int> slot;
+  m.nv = U;
   std::vector<int> sl;
   for (int u = 0; u < U; ++u) {
     const int* t = tab_det.data() + (size_t)u * kTabStride;
-    for (int j = 0; j < t[0]; ++j) {
-      node[u].first.push_back(t[2 + j]);
-      node[u].second.push_back(t[2 + kMaxExc + j]);
-      sl.push_back(t[2 + j]);
-    }
-    slot.insert({node[u], u});
+    sl.insert(sl.end(), t + 2, t + 2 + t[0]);
   }
   std::sort(sl.begin(), sl.end());
   sl.erase(std::unique(sl.begin(), sl.end()), sl.end());
   m.sl = sl;
   m.ns = (int)sl.size();
-  auto row = [&](int s) { return (int)(std::lower_bound(sl.begin(), sl.end(), s) - sl.begin()); };
-  auto minor = [&](const Key& k, int i, int j) {  // without row i and column j
-    Key c = k;
-    c.first.erase(c.first.begin() + i);
-    c.second.erase(c.second.begin() + j);
-    return c;
-  };
+  // no table of that size fits in shared memory, and its indices not in the lists' 15 bits
+  if ((size_t)m.ns * nx > 0x7fff) return;
   // a determinant of size >= 3 needs its cofactors; an added minor the ones of its first row
   const size_t most = std::min<size_t>(2 * (size_t)U + 256, 0x7fff);  // a slot fits the lists' 15 bits
+  std::vector<Minor> node(U);
+  node.reserve(std::max<size_t>(most, U) + 16);
+  MinorTable slot(std::max<size_t>(most, U) + 16);
+  for (int u = 0; u < U; ++u) {
+    const int* t = tab_det.data() + (size_t)u * kTabStride;
+    Minor& d = node[u];
+    d.k = t[0];
+    for (int j = 0; j < d.k; ++j) {
+      const int r = (int)(std::lower_bound(sl.begin(), sl.end(), t[2 + j]) - sl.begin());
+      d.rows ^= (uint64_t)(0xffff ^ r) << (16 * j);
+      d.cols ^= (uint64_t)(0xffff ^ t[2 + kMaxExc + j]) << (16 * j);
+    }
+    int& n = slot.find(d);
+    if (n < 0) n = u;
+  }
   for (size_t q = 0; q < node.size() && node.size() <= most; ++q) {
-    const Key k = node[q];
-    const int n = (int)k.first.size();
-    if (n < 3) continue;
-    for (int i = 0; i < ((int)q < U ? n : 1); ++i)
-      for (int j = 0; j < n; ++j) {
-        const Key c = minor(k, i, j);
-        if (slot.insert({c, (int)node.size()}).second) node.push_back(c);
+    const Minor d = node[q];
+    if (d.k < 3) continue;
+    for (int i = 0; i < ((int)q < U ? d.k : 1); ++i)
+      for (int j = 0; j < d.k; ++j) {
+        const Minor c = d.without(i, j);
+        int& n = slot.find(c);
+        if (n >= 0) continue;
+        n = (int)node.size();
+        node.push_back(c);
       }
   }
   const bool direct = node.size() > most;
@@ -308,63 +366,76 @@ static void make_minors(const std::vector<int>& tab_det, int U, int nx, TabMinor
   m.nv = (int)node.size();
   const int nt = m.ns * nx;
   const int kNeg = (int)0x80000000u;
-  std::vector<std::vector<int>> ut(nt);  // by Tn entry
   std::vector<int> alone;  // determinants formed each by itself
   m.du_off.assign(1, 0);
-  auto t_of = [&](int s, int x) { return row(s) * nx + x; };
+  auto t_of = [&](const Minor& d, int i, int j) { return d.row(i) * nx + d.col(j); };
   for (int q = 0; q < m.nv; ++q) {
-    const Key& key = node[q];
-    const std::vector<int>&S = key.first, &Q = key.second;
-    const int k = (int)S.size();
+    const Minor& d = node[q];
+    const int k = d.k;
     if (k == 1) {
-      m.l1.insert(m.l1.end(), {q, t_of(S[0], Q[0])});
+      m.l1.insert(m.l1.end(), {q, t_of(d, 0, 0)});
     } else if (k == 2) {
-      m.l2.insert(m.l2.end(), {q, t_of(S[0], Q[0]) | t_of(S[1], Q[1]) << 16, t_of(S[0], Q[1]) | t_of(S[1], Q[0]) << 16, 0});
+      m.l2.insert(m.l2.end(), {q, t_of(d, 0, 0) | t_of(d, 1, 1) << 16, t_of(d, 0, 1) | t_of(d, 1, 0) << 16, 0});
     } else if (k >= 3 && direct) {
       alone.push_back(q);
     } else if (k >= 3) {
       std::vector<int>& l = k == 3 ? m.l3 : m.l4;
       l.push_back(q);
-      for (int j = 0; j < k; ++j) l.push_back(t_of(S[0], Q[j]) | slot.at(minor(key, 0, j)) << 16);
+      for (int j = 0; j < k; ++j) l.push_back(t_of(d, 0, j) | slot.find(d.without(0, j)) << 16);
       if (k == 4) l.insert(l.end(), {0, 0, 0});
     }
     if (q < U) {
       if (k <= 2 || !direct)
         for (int i = 0; i < k; ++i)
           for (int j = 0; j < k; ++j) {
-            const int t = t_of(S[i], Q[j]), sg = ((i + j) & 1) ? kNeg : 0;
-            const int cof = k == 1 ? -1 : (k == 2 ? 0x10000 + t_of(S[1 - i], Q[1 - j]) : slot.at(minor(key, i, j)));
-            ut[t].insert(ut[t].end(), {q | sg, cof});
-            m.du.insert(m.du.end(), {t | sg, cof});
+            const int sg = ((i + j) & 1) ? kNeg : 0;
+            const int cof = k == 1 ? -1 : (k == 2 ? 0x10000 + t_of(d, 1 - i, 1 - j) : slot.find(d.without(i, j)));
+            m.du.insert(m.du.end(), {t_of(d, i, j) | sg, cof});
           }
       m.du_off.push_back((int)(m.du.size() / 2));
     }
   }
-  m.rt_off.assign(1, 0);
-  for (int t = 0; t < nt; ++t) {
-    m.rt.insert(m.rt.end(), ut[t].begin(), ut[t].end());
-    m.rt_off.push_back((int)(m.rt.size() / 2));
-  }
-  std::stable_sort(alone.begin(), alone.end(),
-                   [&](int a, int b) { return node[a].first.size() > node[b].first.size(); });
+  // the derivatives by Tn entry, each entry's in the order of the determinants
+  m.rt_off.assign(nt + 1, 0);
+  for (size_t e = 0; e < m.du.size(); e += 2) ++m.rt_off[(m.du[e] & 0x7fffffff) + 1];
+  for (int t = 0; t < nt; ++t) m.rt_off[t + 1] += m.rt_off[t];
+  m.rt.resize(m.du.size());
+  std::vector<int> fill(m.rt_off.begin(), m.rt_off.end() - 1);
+  for (int u = 0; u < U; ++u)
+    for (int e = m.du_off[u]; e < m.du_off[u + 1]; ++e) {
+      const int p = fill[m.du[2 * e] & 0x7fffffff]++;
+      m.rt[2 * p] = u | (m.du[2 * e] & kNeg);
+      m.rt[2 * p + 1] = m.du[2 * e + 1];
+    }
+  std::stable_sort(alone.begin(), alone.end(), [&](int a, int b) { return node[a].k > node[b].k; });
   m.lr_off.assign(1, 0);
+  std::vector<std::pair<int, int>> entry;  // of a round: Tn entry, cofactor
+  std::vector<int> count(nt);
   for (size_t d0 = 0; d0 < alone.size(); d0 += 32) {
-    std::map<int, std::vector<int>> by_entry;
-    for (size_t d = d0; d < std::min(alone.size(), d0 + 32); ++d) {
-      const std::vector<int>&S = node[alone[d]].first, &Q = node[alone[d]].second;
-      const int k = (int)S.size();
+    entry.clear();
+    std::fill(count.begin(), count.end(), 0);
+    for (size_t q = d0; q < std::min(alone.size(), d0 + 32); ++q) {
+      const Minor& d = node[alone[q]];
       int rows = 0, cols[2] = {0, 0};
-      for (int i = 0; i < k; ++i) {
-        rows |= row(S[i]) << (8 * i);
-        cols[i / 2] |= (int)((unsigned)Q[i] << (16 * (i & 1)));
-        for (int j = 0; j < k; ++j) by_entry[t_of(S[i], Q[j])].push_back((int)(d - d0) << 4 | (4 * i + j));
+      for (int i = 0; i < d.k; ++i) {
+        rows |= d.row(i) << (8 * i);
+        cols[i / 2] |= (int)((unsigned)d.col(i) << (16 * (i & 1)));
+        for (int j = 0; j < d.k; ++j) {
+          entry.push_back({t_of(d, i, j), (int)(q - d0) << 4 | (4 * i + j)});
+          ++count[entry.back().first];
+        }
       }
-      m.ld.insert(m.ld.end(), {(int)((unsigned)alone[d] | (unsigned)k << 28), rows, cols[0], cols[1]});
+      m.ld.insert(m.ld.end(), {(int)((unsigned)alone[q] | (unsigned)d.k << 28), rows, cols[0], cols[1]});
     }
-    for (const auto& e : by_entry) {
-      m.lh.insert(m.lh.end(), {e.first, (int)m.le.size()});
-      m.le.insert(m.le.end(), e.second.begin(), e.second.end());
+    int at = (int)m.le.size();
+    m.le.resize(m.le.size() + entry.size());
+    for (int t = 0; t < nt; ++t) {
+      const int c = count[t];
+      count[t] = at;  // where the entry's cofactors go
+      if (c) m.lh.insert(m.lh.end(), {t, at});
+      at += c;
     }
+    for (const auto& e : entry) m.le[count[e.first]++] = e.second;
     m.lr_off.push_back((int)(m.lh.size() / 2));
   }
   m.lh.insert(m.lh.end(), {nt, (int)m.le.size()});
