@@ -38,10 +38,10 @@ WALKER_KERNEL_SOURCES = {"sweep": ["kernels.cu", "sweep_body.cuh"] + _COMMON_SOU
                          "orbitals": ["eval_orbitals.cu", "orbital_body.cuh"] + _COMMON_SOURCES,
                          "jastrow": ["eval_jastrow.cu", "jastrow_body.cuh"] + _COMMON_SOURCES}
 PROFILED_TRAFFIC = {
-    "sweep": ("244f78b91ff5c8533fc44c0448802bb31cae4e8f8672ea368bd58aaf0bc5eb95", 10884.7),
-    "det": ("db53a660e3b55e8458d235d88a2d90e4903fb1f58eb9bb593146e1fed341424c", 26494.1),
-    "orbitals": ("21d607ab450fa5030d8fdbd7f2bad29956124f1bd9c616db9c6b2267c33129bb", 9048.9),
-    "jastrow": ("9bb53d641580f851d7480ef8d5c101d8363dfc188579676e4813c39251a35a10", 392.2),
+    "sweep": ("cde2a05112554ca8423adad5b5e6e08e028804f2158cf61551994a6d199093f0", 10866.8),
+    "det": ("804ad433cd8d108cb5063456942ee6ee797baffab644ecdb66cfdd12dc625281", 26026.9),
+    "orbitals": ("425e0e9ea485ea31ddee3f2abeb3ad73278f2b303b1bc0de95f60f816f4b1dca", 8597.9),
+    "jastrow": ("122c68b9801820319967152c6f8ae32247506fc73e29147e3970391bebb87af3", 392.4),
 }
 
 

@@ -435,11 +435,11 @@ int vbqmc_launch_info(vbqmc_ctx* ctx, int sys_id, int precision, int* out);
  * VMC sweeps and evaluations keep no walker state, orbital-excitation and nucleus derivatives
  * are refused.  vbqmc_set_system takes the tables when the per-determinant inverses of one
  * walker do not fit in shared memory, and, for systems without orbital-excitation parameters,
- * when the per-determinant sweep region of a walker exceeds 48 KB, or 32 KB with 16 or more
- * unique determinants of a spin (few walkers per SM: the measured crossover on molecules of
- * 2-32 electrons).  Errors: VBQMC_ERR_NOSYS, VBQMC_ERR_UNSUPPORTED (a
- * determinant differs from the reference in more than 4 columns), VBQMC_ERR_CAPACITY (on = 0
- * but the inverses do not fit). */
+ * when a walker's inverses and buffers of a plain per-determinant sweep exceed 48 KB, or 32 KB with 16
+ * or more unique determinants of a spin (few walkers per SM: the line measured for walker-steps from a
+ * carried state on molecules of 2-32 electrons; long runs of sweeps alone gain from on = 1 earlier).
+ * Errors: VBQMC_ERR_NOSYS, VBQMC_ERR_UNSUPPORTED (a determinant differs from the reference in more than
+ * 4 columns), VBQMC_ERR_CAPACITY (on = 0 but the inverses do not fit). */
 int vbqmc_use_tables(vbqmc_ctx* ctx, int sys_id, int on);
 
 /* Number of kernel launches enqueued by the last successful call on this context. */

@@ -329,9 +329,9 @@ int vbqmc_set_system(vbqmc_ctx* ctx, int sys_id, const vbqmc_system_desc* desc) 
   }
   // determinants through the reference-determinant tables when the per-determinant inverses of
   // one walker do not fit in shared memory, or when they hold so much of it that few walkers
-  // share an SM: a sweep region above 48 KB, or above 32 KB with 16 or more unique
-  // determinants of a spin (the measured crossover on molecules of 2-32 electrons; systems with
-  // orbital-excitation parameters keep the per-determinant form, whose derivatives they need)
+  // share an SM: more than 48 KB a walker by per_determinant_region_bytes, or 32 KB with 16 or more
+  // unique determinants of a spin (measured on both sides, see there; systems with orbital-excitation
+  // parameters keep the per-determinant form, whose derivatives they need)
   d.msd = 0;
   {
     vbq::DetLayout probe;

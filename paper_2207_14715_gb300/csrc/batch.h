@@ -7,7 +7,7 @@
 namespace vbq {
 
 // Work item: walkers first .. first + count - 1 of system sys (for the orbital kernel:
-// (walker, electron) pairs in the same walker-major order).  One warp per walker (pair).
+// (walker, electron) points in the same walker-major order, the block's warps on all of them).
 struct BatchItem {
   int sys, first, count, pad;
 };
@@ -66,8 +66,8 @@ cudaError_t launch_det_batch(const BatchSys* sys, const BatchItem* items, int ni
 // the evaluation kernels' bodies (if eval) and the Jastrow-parameter derivatives (if derivs) on
 // each tile in turn.  Every item's count fits the block's warps; in the per-walker phases of
 // system s, warps 0 .. s.cw[phase] - 1 take the tile's walkers in turn (cw[phase] regions of
-// that phase fit the shared memory smem), and the orbital phase spreads the tile's (walker,
-// electron) pairs over all warps.
+// that phase fit the shared memory smem), and the orbital phase takes the tile's (walker,
+// electron) points in groups with the whole block on each.
 cudaError_t launch_batch_fused(int is_float, const BatchSys* sys, const BatchItem* items, int nitems,
                                const BatchCall* call, int* queue, bool sweep, bool eval, bool derivs, int grid,
                                int warps, int smem, cudaStream_t st);

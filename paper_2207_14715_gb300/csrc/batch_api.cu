@@ -149,7 +149,8 @@ int build_plan(vbqmc_batch* b, int kind) {
 // Work items and shape of the one-launch step: with p.warps warps per block, tiles of T = p.warps
 // walkers (p.cap > 0: at most p.cap); one block per SM holds the opt-in shared memory, and in each
 // per-walker phase of system s as many walkers run at once as that phase's per-walker regions
-// fit it (cw, at most T); the orbital phase gives every warp its own region.
+// fit it (cw, at most T); in the orbital phase the whole block works on as many of the tile's (walker,
+// electron) points at a time as their regions fit (at most one per warp).
 int build_fused_plan(vbqmc_batch* b) {
   KernelPlan& p = b->plan[kFused];
   const bool f = b->precision == VBQMC_MIXED;

@@ -2,7 +2,7 @@
 // (arXiv:2207.14715, Sec. 2.1: every determinant of a spin shares the inactive orbitals and
 // differs from the others by a few active columns), for systems whose per-determinant
 // inverses do not fit in shared memory.  One warp per walker.  Per spin:
-//   A_0 = reference determinant (u = 0), B = A_0^-1 by the lane-group inverse (double);
+//   A_0 = reference determinant (u = 0), B = A_0^-1 by the whole-warp Gauss-Jordan (double);
 //   T = B Phi_X over the orbitals X outside the reference;
 //   determinant u replaces the reference slots S_u by the orbitals Q_u (k_u <= 4):
 //     D_u = sgn_u D_0 q_u,  q_u = det T[S_u, Q_u]  (tab_minors.cuh).
@@ -14,8 +14,8 @@
 // K[Phi]/Phi.  The traces t_u = tr(A_u^-1 L_u) are formed for structure-coefficient derivatives only.
 //
 // Bound: the FP64 pipe (about 2400 instructions per walker on 48 electrons, a quarter of them the
-// two inverses) and latency at 10 walkers per SM (22.5 KB each): 2.22 -> 0.88 ms per 4096 walkers
-// against traces and inverses of every determinant's own minor (36 KB, 6 walkers per SM).
+// two inverses) and latency at 10 walkers per SM (22.5 KB each): 0.85 ms per 4096 walkers,
+// 2.36 with traces and inverses of every determinant's own minor (36 KB, 6 walkers per SM).
 #include "dettab_body.cuh"
 
 namespace vbq {

@@ -153,8 +153,14 @@ size_t overlap_part_doubles(int M, int nvb);
 cudaError_t launch_structure_overlap(int M, int ldo, int otype, const void* O, const double* wts, const OverlapMap& map,
                                      double* part, double* out, cudaStream_t st);
 // Size of a walker by which the form of the determinants is chosen (inverses per determinant or
-// reference tables): inverses, positions, tables and buffers of a sweep whose moves form everything by
-// themselves.  The line was measured with that region; the sweep's own layout may be larger or smaller.
+// reference tables): inverses, positions, tables and buffers of a per-determinant sweep whose moves form
+// everything by themselves.  A measure of the system, not the region of the present sweep (which may be
+// larger or smaller): systems keep their form, and with it their walker state, whatever a layout gains.
+// Its line, above 48 KB or above 32 KB with 16 or more determinants of a spin, is one for walker-steps from a
+// carried state; with the present kernels, on the 59 of 64 molecules (2-32 electrons, 4096 walkers, mixed)
+// that can take both forms: the tables take 0.07-0.52 of the time above the line, 1.10-2.2 of it
+// below but for three at 27-32 KB (0.81-0.88).  Sweeps alone (10 from a fresh start) would put it lower,
+// at about 14 KB: there the tables take 1.0, at 20 KB 0.5.
 int per_determinant_region_bytes(const SysDev& s);
 // Walkers (warps) per block of a kernel of one warp per walker: W walkers, at most 'most' per block,
 // sm_warps warps on an SM by registers, 'bytes' of shared memory per walker.
@@ -164,9 +170,12 @@ int per_determinant_region_bytes(const SysDev& s);
 //    1032 of 4; 3001 walkers in double: Jastrow 1739 -> 1450 us, its derivatives 2057 -> 1714 us).
 //  - Fewer: a round of p warps on an SM takes about 100 + 3 p (the warps share the issue slots and
 //    the FP64 pipe); the fewest such units, counting the warps that the last, partly filled round
-//    puts on its busiest SM, larger blocks within 2 %.  A sample that would leave SMs idle with full
-//    blocks is spread over them (300 walkers in double, 5 sweeps: 6.7 -> 2.4 ms); blocks much smaller
-//    than an SM's share are placed unevenly there (4096 walkers, 10 sweeps: 3.75 ms with 14, 4.06 with 4).
+//    puts on its busiest SM.  A sample that would leave SMs idle with full blocks is spread over them (300
+//    walkers in double, 5 sweeps: 6.7 -> 2.4 ms).  Blocks much smaller than an SM's share are placed
+//    unevenly there (4096 walkers, 10 sweeps: 3.75 ms with 14 walkers, 4.06 with 4, 3.91 with 1), so
+//    that larger blocks win within 2 %, and once a round is full no block goes below a quarter of an SM.
+//  The unit was fitted to the ethylene-shaped sweep; the Jastrow and determinant kernels take the same rule
+//  (3001 walkers in double, all together 7.84 -> 6.61 ms; the determinant kernel alone lost, 318 -> 341 us).
 int walkers_per_block(int W, int most, int sm_warps, int bytes);
 // Dynamic shared-memory limit of kernel fn on the current device: what the device allows a block, less
 // fn's own static shared memory.  The limit is a property of the function, shared by every host thread

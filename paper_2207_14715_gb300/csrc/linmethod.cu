@@ -19,9 +19,9 @@
 //      rows (each row 32 high halves then 32 low halves); the same pass forms sum w Ot E from
 //      the centred values (block partials, fixed-order sum);
 //  (3) the products on the tensor cores (tcgen05, kind::f16, FP32 accumulators in tensor
-//      memory): per output tile of 128 parameters i x 112 parameters j and chunk of samples,
-//      D_S[i][j] = sum_s X_si X_sj and D_H[i][j] = sum_s X_si Y_sj in one MMA of N = 224 whose B
-//      operand stacks the j rows of X and of Y, each product formed as hi*lo + lo*hi + hi*hi
+//      memory): per output tile of 128 parameters i x 112 (small samples: 64 or 32) parameters j and
+//      chunk of samples, D_S[i][j] = sum_s X_si X_sj and D_H[i][j] = sum_s X_si Y_sj in one MMA of N = 224
+//      (128, 64) whose B operand stacks the j rows of X and of Y, each product formed as hi*lo + lo*hi + hi*hi
 //      (the lo*lo term is below the float accuracy);
 //  (4) the chunk partials added in double in a fixed order, unscaled and divided by sum w.
 // The half-precision split runs the tensor cores at twice the rate of the TF32 split with the
@@ -457,14 +457,14 @@ __global__ void __launch_bounds__(256, CenBlocks<Tin, ntile>::n)
   }
 }
 
-// (3) Partial tiles, one CTA per (128 x 112 output tile, chunk of samples):
+// (3) Partial tiles, one CTA per (128 x TB output tile, chunk of samples), TB = 112, 64 or 32:
 //   part[chunk][0][i][j] = sum_{s in chunk} X_si X_sj,   part[chunk][1][i][j] = sum X_si Y_sj
 // (scaled values).  Per stage of 32 samples (one group), TMA brings the A tile X_i (128 rows) and
-// the B tile [X_j; Y_j] (2 x 112 rows), each row 128 bytes [32 high halves | 32 low halves],
+// the B tile [X_j; Y_j] (2 x TB rows), each row 128 bytes [32 high halves | 32 low halves],
 // K-major with the 128-byte swizzle (the layout the MMA reads: the high and low operands of a
 // 16-sample slice start 32 bytes apart within the swizzled rows, at +32 kk and +64 + 32 kk).  Warp roles: warp 8 issues the copies into a ring of stages;
 // warp 9 owns the tensor memory and issues per 16-sample slice the MMAs A_hi B_lo, A_lo B_hi,
-// A_hi B_hi (M = 128, N = 224: columns 0-111 accumulate S, 112-223 H; the correction
+// A_hi B_hi (M = 128, N = 2 TB: the first TB columns accumulate S, the others H; the correction
 // products first, while the accumulator is small); warps 0-7 drain the accumulators.  The
 // tensor core's accumulation rounds at the accumulator's magnitude, so an accumulator covers 64
 // samples (two stages) and is then moved to registers and summed there in FP32 (round to

@@ -14,7 +14,7 @@ constexpr int kOrbWarps = 8;
 
 // Chunks c = lane, lane + 32, ... of the contraction with groups of WD orbitals (coefficients
 // interleaved, stride WD): partial sums of phi, grad phi and lap phi over the chunk's basis
-// functions into part[(5 t + k) nch + c].  Basis layout as written by orbital_body.
+// functions into part[(5 t + k) nch + c].  Basis layout as written by orbital_block.
 template <class Tb, int WD>
 __device__ __forceinline__ void contract_groups(const SysDev& s, int lane, int nch, const Tb* __restrict__ cq,
                                                 const Tb* bv, Tb* part) {

@@ -27,11 +27,11 @@ namespace vbq {
 //    sum_u q_u g_u, where g_u = sum over the terms of u of C_k times the other spin's minor stays
 //    as it is while the electrons of one spin move; an accepted move updates B by Sherman-Morrison,
 //    T to T' and q to q'.
-//    Bound: latency at 7 walkers per SM (the walker's region), over the FP64 pipe, whose
+//    Bound: latency at 9 walkers per SM (the walker's region), over the FP64 pipe, whose
 //    instructions are therefore counted: on 48 electrons (70 determinants per spin) about 60 per
 //    move and 55 more when it is accepted, where eliminating every determinant's matrix, summing
-//    the 256 terms and serial column sums took about 250 and 70: 16.5 -> 11.5 ms per sweep of
-//    8192 walkers.
+//    the 256 terms and serial column sums took about 250 and 70.  With the proposals below 9.4 ms per
+//    sweep of 8192 walkers, 16.4 with those.
 // Each sweep moves every electron once (Sec. 2.3.1).  The determinant inverses come from
 // the walker state written by the evaluation at the same positions, or from a fresh LU of
 // double-precision orbital values (first sweep without state, and every 'refresh' sweeps).
@@ -46,8 +46,8 @@ namespace vbq {
 // per pair (L.tri) and replaced when a move is accepted.  The float values and sums are those of a
 // move that forms everything by itself, bit for bit.  Bound by instruction issue (float) and the
 // FP64 pipe (double); a sweep of the ethylene-shaped system went from 1298 to 1080 us (16384 walkers,
-// mixed), 2303 to 2095 us (3001, double), one of the 48-electron system from 11.5 to 10.0 ms (8192), and to
-// 9.4 ms with at most 16 electrons prepared at once and small blocks.
+// mixed; 1030 in small blocks), 2303 to 2095 us (3001, double; 1512), one of the 48-electron system from 11.5
+// to 10.0 ms (8192; 9.4 with at most 16 electrons prepared at once and small blocks).
 // One warp, walker w, shared-memory region 'base' of L.warp_bytes bytes.
 
 // f of the Pade + polynomial form at R = r den, den = 1 / (1 + kappa r) (as pade_poly)

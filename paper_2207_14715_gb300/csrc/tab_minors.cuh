@@ -9,9 +9,9 @@
 // Accuracy: where the reference is small next to the other determinants, T is a large matrix of
 // rank one plus a remainder (the reference's own column), and minors cancel: the 2 x 2 minors are
 // formed as Kahan's difference of products and the 3 x 3 minors with the error terms of their
-// products and sums, so that the expansion loses no more than an elimination with pivoting
-// (which removes the rank-one part in its first step); the cofactors of the derivatives are minors
-// of this kind as well.
+// products and sums, so that a 4 x 4 minor's last sum is the only one that cancels (three times the error of an
+// elimination with pivoting, which removes the rank-one part in its first step; ln|Phi|, its gradient and
+// E_L are as accurate); the cofactors of the derivatives are minors of this kind as well.
 //
 // Work: 4, 23 and 4 instructions on the FP64 pipe per 32 minors of size 2, 3 and 4 (64 cycles of a
 // sub-partition each), where eliminating every determinant's own matrix took about 60 per 32
