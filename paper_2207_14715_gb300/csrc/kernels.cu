@@ -180,7 +180,10 @@ int walkers_per_block(int W, int most, int sm_warps, int bytes) {
   for (int p = 1; p <= most; ++p) warps = std::max(warps, p * resident(p));
   if ((long)W > 2L * warps * sms)
     for (int p = std::min(2, most); p <= most; ++p)
-      if (p * resident(p) == warps) return p;
+      if (p * resident(p) == warps) {
+        if (resident(p) > 1 || p == 1) return p;
+        break;  // one block fills the SM: whole rounds
+      }
   long best_cost = 0;
   int best = most;
   for (int p = most; p >= 1; --p) {

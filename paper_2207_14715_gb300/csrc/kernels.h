@@ -168,9 +168,11 @@ int per_determinant_region_bytes(const SysDev& s);
 //    resident as any size does; a finished block is replaced at once, so rounds do not wait for
 //    their slowest walker (ethylene-shaped system, 16384 walkers: sweep 1082 us with blocks of 16,
 //    1032 of 4; 3001 walkers in double: Jastrow 1739 -> 1450 us, its derivatives 2057 -> 1714 us).
-//  - Fewer: a round of p warps on an SM takes about 100 + 3 p (the warps share the issue slots and
-//    the FP64 pipe); the fewest such units, counting the warps that the last, partly filled round
-//    puts on its busiest SM.  A sample that would leave SMs idle with full blocks is spread over them (300
+//  - Fewer, or where only a block of the whole SM keeps that many: a round of p warps on an SM takes
+//    about 100 + 3 p (the warps share the issue slots and the FP64 pipe); the fewest such units, counting
+//    the warps that the last, partly filled round puts on its busiest SM.  Blocks of the whole SM run in
+//    whole rounds (30 electrons, 7 walkers of 32 KB: 2500 walkers are 2.35 rounds of 7, a sweep 2.58 ms, or
+//    2.74 of 6, 2.18 ms).  A sample that would leave SMs idle with full blocks is spread over them (300
 //    walkers in double, 5 sweeps: 6.7 -> 2.4 ms).  Blocks much smaller than an SM's share are placed
 //    unevenly there (4096 walkers, 10 sweeps: 3.75 ms with 14 walkers, 4.06 with 4, 3.91 with 1), so
 //    that larger blocks win within 2 %, and once a round is full no block goes below a quarter of an SM.
