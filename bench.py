@@ -38,10 +38,10 @@ WALKER_KERNEL_SOURCES = {"sweep": ["kernels.cu", "sweep_body.cuh"] + _COMMON_SOU
                          "orbitals": ["eval_orbitals.cu", "orbital_body.cuh"] + _COMMON_SOURCES,
                          "jastrow": ["eval_jastrow.cu", "jastrow_body.cuh"] + _COMMON_SOURCES}
 PROFILED_TRAFFIC = {
-    "sweep": ("cde2a05112554ca8423adad5b5e6e08e028804f2158cf61551994a6d199093f0", 10866.8),
-    "det": ("804ad433cd8d108cb5063456942ee6ee797baffab644ecdb66cfdd12dc625281", 26026.9),
-    "orbitals": ("425e0e9ea485ea31ddee3f2abeb3ad73278f2b303b1bc0de95f60f816f4b1dca", 8597.9),
-    "jastrow": ("122c68b9801820319967152c6f8ae32247506fc73e29147e3970391bebb87af3", 392.4),
+    "sweep": ("67e11a7444836e68f5bfd8db85c8df2c5bc700a2ebf9327bed2d620be4430022", 10826.2),
+    "det": ("de65609a5347e2ad6bf12611924bfbf7ac347aeab31c4a49d5fc16a061c4d04f", 26020.9),
+    "orbitals": ("5fca46e420032412e68dda7124c8f08e8ddeed56452c45003e8c56f9dda79861", 8583.9),
+    "jastrow": ("1834199c647dd6410b4165c6880b241176625bd4c6f3df3c61f23099ea8da641", 392.4),
 }
 
 
